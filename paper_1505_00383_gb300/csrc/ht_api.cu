@@ -7,7 +7,7 @@
 #include <cmath>
 
 #include "ht_internal.h"
-#include "ht_mpi.cuh"
+#include "ht_mpi_eval.cuh"
 
 namespace ht {
 
@@ -89,6 +89,7 @@ int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8
       return set_error(HT_EINVAL, "ht_create_system: n_terms[%d]=%d < 1", j, n_terms[j]);
     }
     s->h_poly_off[j + 1] = s->h_poly_off[j] + n_terms[j];
+    if (n_terms[j] > s->max_terms) s->max_terms = n_terms[j];
   }
   s->M = s->h_poly_off[n_polys];
   s->n_terms.assign(n_terms, n_terms + n_polys);
@@ -175,13 +176,30 @@ int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8
       const double mod = std::hypot(re[0], im[0]);
       hl[m] = mod == 0.0 ? -1000.0f : (float)std::log2(mod);
     }
+    // the sweep steps of every monomial (the integer variant takes at most 64 variables)
+    std::vector<uint32_t> steps;
+    std::vector<int32_t> step_off;
+    if (n_vars <= 64) {
+      step_off.assign(1, 0);
+      for (int64_t m = 0; m < s->M; ++m) {
+        mpi::sweep_steps(s->h_pairs.data() + s->h_mon_off[m], s->h_mon_off[m + 1] - s->h_mon_off[m], steps);
+        step_off.push_back((int32_t)steps.size());
+      }
+    }
+    const size_t b_hz = up(hz.size()), b_hl = up(hl.size() * sizeof(float)), b_so = up(step_off.size() * 4);
     void* blk = nullptr;
-    e = cudaMalloc(&blk, hz.size() + hl.size() * sizeof(float) + 256);
+    e = cudaMalloc(&blk, b_hz + b_hl + b_so + steps.size() * 4);
     if (e == cudaSuccess) {
       s->d_coef_fz = blk;
-      s->d_coef_lg = (float*)((char*)blk + ((hz.size() + 255) & ~(size_t)255));
+      s->d_coef_lg = (float*)((char*)blk + b_hz);
       e = cudaMemcpy(s->d_coef_fz, hz.data(), hz.size(), cudaMemcpyHostToDevice);
       if (e == cudaSuccess) e = cudaMemcpy(s->d_coef_lg, hl.data(), hl.size() * sizeof(float), cudaMemcpyHostToDevice);
+    }
+    if (e == cudaSuccess && !steps.empty()) {
+      s->d_step_off = (int32_t*)((char*)blk + b_hz + b_hl);
+      s->d_steps = (uint32_t*)((char*)blk + b_hz + b_hl + b_so);
+      e = cudaMemcpy(s->d_step_off, step_off.data(), step_off.size() * 4, cudaMemcpyHostToDevice);
+      if (e == cudaSuccess) e = cudaMemcpy(s->d_steps, steps.data(), steps.size() * 4, cudaMemcpyHostToDevice);
     }
     if (e != cudaSuccess) {
       cudaGetLastError();

@@ -22,6 +22,8 @@
 // Outputs are written in the vertical layout of Table tabtranspose; the
 // Jacobian row of the unit's polynomial accumulates in place in the output
 // array (it stays in L2 while the unit runs), so no scratch memory is used.
+#include <algorithm>
+
 #include "ht_eval.cuh"
 #include "ht_internal.h"
 #include "ht_int_row.cuh"
@@ -35,6 +37,7 @@ struct EvalArgs {
   double* val;
   double* jac;
   int64_t n_units;
+  int max_terms;  // largest number of monomials of a polynomial
 };
 
 template <int L, bool LOOP>
@@ -81,8 +84,8 @@ static int launch_v(const EvalArgs& a, int threads, cudaStream_t st) {
 //      in place in the output (2L doubles hold exactly 2 x 2L int32 limbs);
 //   4. converts the accumulators to L doubles.
 template <int L>
-__global__ void __launch_bounds__(128, 4) evaldiff_int_kernel(EvalArgs a, const mpi::fz<IntW<L>::W>* __restrict__ cfz,
-                                                           const float* __restrict__ clg) {
+__global__ void __launch_bounds__(128, 4) evaldiff_int_kernel(EvalArgs a, IntPoly ip,
+                                                           const mpi::fz<IntW<L>::W>* __restrict__ cfz) {
   using Z = mpi::fz<IntW<L>::W>;
   Z X[kIntMaxVars];
   float lg[kIntMaxVars];
@@ -97,35 +100,63 @@ __global__ void __launch_bounds__(128, 4) evaldiff_int_kernel(EvalArgs a, const 
     const int64_t p = (u / a.np) * 32 + lane;
     if (p >= n) continue;
     int_point<L>(a.v.x, a.nv, n, p, X, lg);
-    double vre[L], vim[L];
-    int_row<L>(a.v.mon_off, a.v.pairs, cfz, clg, a.poly_off[j], a.poly_off[j + 1], X, lg, a.nv,
-               a.jac + (int64_t)j * plane, n, p, vre, vim, P);
-#pragma unroll
-    for (int l = 0; l < L; ++l) {
-      a.val[((int64_t)(j * 2) * L + l) * n + p] = vre[l];
-      a.val[((int64_t)(j * 2 + 1) * L + l) * n + p] = vim[l];
-    }
+    int_row<L>(ip, cfz, a.poly_off[j], a.poly_off[j + 1], X, lg, a.nv, a.val + (int64_t)j * 2 * L * n,
+               a.jac + (int64_t)j * plane, n, p, P);
   }
 }
 
+// The block's 32 points as limb strings and log2 moduli in shared memory; all
+// threads of the CTA take part (lanes past the last point store zeros).
+template <int L>
+__device__ __forceinline__ void stage_points(const double* __restrict__ x, int nv, int64_t n, int64_t p, int32_t* xs,
+                                             float* lgs) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, T = blockDim.x >> 5;
+  for (int v = warp; v < nv; v += T) {
+    double re[L], im[L];
+#pragma unroll
+    for (int l = 0; l < L; ++l) {
+      re[l] = p < n ? x[((int64_t)(v * 2) * L + l) * n + p] : 0.0;
+      im[l] = p < n ? x[((int64_t)(v * 2 + 1) * L + l) * n + p] : 0.0;
+    }
+    store_point<L>(xs, v, lane, mpi::from_doubles<IntW<L>::W, L>(re, im));
+    lgs[v * 32 + lane] = mpi::log2_mod(re[0], im[0]);
+  }
+}
+
+// Largest CTA of the block organisation, in warps: 32 for double double (64
+// registers a thread without spills to speak of), 16 for quad double.  The
+// integer multiply-add pipe bounds both, and at n = 32, 65,536 points twice
+// the warps take DD from 33.2 to 29.4 ms; QD at 64 registers spills, and
+// gained 2 % there while it lost 3 to 8 % on smaller systems.
+template <int L>
+constexpr int kBlkWarps = L == 4 ? 16 : 32;
+// Row slots that pass through shared memory at a time in the split kernel
+// (2 KB a warp).
+template <int L>
+constexpr int kSplitSlots = 8 / L;
+
 // Block organisation of the same unit: a CTA takes a block of 32 points and
-// a group of polynomials (as many as it has warps: one each; 16 warps when
-// the system has at least 16 polynomials, else 8).  The block's
-// converted points live once in shared memory (lane-interleaved, so every
-// access is a conflict-free 32-word row) instead of once per lane and unit
-// in local memory; the warp still walks one monomial with all lanes in step.
+// a group of polynomials (as many as it has warps: one each).  The block's
+// converted points live once in shared memory instead of once per lane and
+// unit in local memory; the warp still walks one monomial with all lanes in
+// step.
 // Work items (polynomial group, point block) are ordered group-major, so a
 // CTA keeps one group's monomials and coefficients (a QD coefficient is 68
 // bytes) in its L1 across point blocks; the points are converted once per
 // item.  The sums are the same exact integers, so the results are those of
 // the per-unit kernel bit for bit.
+//
+// What bounds it: the integer multiply-add pipe (QD: 63 % busy, four fifths
+// of that the limb products), then the arithmetic around the products.  At
+// n = 32, 65,536 points: QD 79.4 -> 58.6 ms and DD 43.9 -> 29.4 ms with the
+// steps of ht_mpi_eval.cuh (one operand of every product stays in registers:
+// 27 % fewer instructions), the points and the row accumulators in 128-bit
+// words, and the column-by-column product.
 template <int L>
-__global__ void __launch_bounds__(512, 1) evaldiff_intblk_kernel(EvalArgs a, const mpi::fz<IntW<L>::W>* __restrict__ cfz,
-                                                              const float* __restrict__ clg) {
-  constexpr int W = IntW<L>::W;
-  using Z = mpi::fz<W>;
-  extern __shared__ __align__(16) int32_t xs[];  // [nv][2W+1][32] limb strings, then [nv][32] log2 moduli
-  float* lgs = reinterpret_cast<float*>(xs + (int64_t)a.nv * (2 * W + 1) * 32);
+__global__ void __launch_bounds__(32 * kBlkWarps<L>, 1) evaldiff_intblk_kernel(
+    EvalArgs a, IntPoly ip, const mpi::fz<IntW<L>::W>* __restrict__ cfz) {
+  extern __shared__ __align__(16) int32_t xs[];  // [nv][32][NW] limb strings, then [nv][32] log2 moduli
+  float* lgs = reinterpret_cast<float*>(xs + a.nv * 32 * SmemPoints<L>::NW);
   mpi::fzs<IntW<L>::W> P[64];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, T = blockDim.x >> 5;
   const int64_t n = a.v.npts, plane = (int64_t)a.nv * 2 * L * n, n_blocks = (n + 31) / 32;
@@ -134,62 +165,185 @@ __global__ void __launch_bounds__(512, 1) evaldiff_intblk_kernel(EvalArgs a, con
   const SmemLog lg{lgs, lane};
   for (int64_t item = blockIdx.x; item < n_blocks * n_groups; item += gridDim.x) {
     const int64_t b = item % n_blocks;
-    const int g = (int)(item / n_blocks);
+    const int j = (int)(item / n_blocks) * T + warp;
     const int64_t p = b * 32 + lane;
-    const bool live = p < n;
     __syncthreads();  // the previous block's points are no longer read
-    for (int v = warp; v < a.nv; v += T) {
-      double re[L], im[L];
-#pragma unroll
-      for (int l = 0; l < L; ++l) {
-        re[l] = live ? a.v.x[((int64_t)(v * 2) * L + l) * n + p] : 0.0;
-        im[l] = live ? a.v.x[((int64_t)(v * 2 + 1) * L + l) * n + p] : 0.0;
-      }
-      store_point<L>(xs, v, lane, mpi::from_doubles<W, L>(re, im));
-      lgs[v * 32 + lane] = mpi::log2_mod(re[0], im[0]);
+    stage_points<L>(a.v.x, a.nv, n, p, xs, lgs);
+    __syncthreads();
+    if (p >= n || j >= a.np) continue;  // lanes past the ragged tail and warps past the last polynomial
+    int_row<L>(ip, cfz, a.poly_off[j], a.poly_off[j + 1], X, lg, a.nv, a.val + (int64_t)j * 2 * L * n,
+               a.jac + (int64_t)j * plane, n, p, P);
+  }
+}
+
+// The same for few points: the monomials of a polynomial are dealt to S warps
+// of the CTA (contiguous ranges of about equal numbers of steps), G = T / S
+// polynomials at a time.  Each warp bounds its own monomials' terms; the
+// largest bounds over the S warps fix the frames.  Each accumulates its part
+// of the row, and the parts are added as integers, so the results are the
+// bits of the unsplit sums.  The time is one warp's share of a polynomial:
+// the 16 polynomials of 246 monomials at 999 points (512 polynomials x
+// blocks for 2,432 resident warps) took 4.4 ms unsplit, 1.14 ms with S = 4.
+template <int L>
+__global__ void __launch_bounds__(512, 1) evaldiff_intsplit_kernel(EvalArgs a, IntPoly ip,
+                                                                 const mpi::fz<IntW<L>::W>* __restrict__ cfz, int S) {
+  constexpr int W = IntW<L>::W, WA = IntW<L>::WA, Q = RowAcc<L>::Q, R = kSplitSlots<L>;
+  extern __shared__ __align__(16) int32_t xs[];
+  float* lgs = reinterpret_cast<float*>(xs + a.nv * 32 * SmemPoints<L>::NW);
+  float* red = lgs + a.nv * 32;                 // bounds [T][nv + 1][32], then
+  int4* part = reinterpret_cast<int4*>(red);    // row slots [T][R][Q][32]
+  mpi::fzs<W> P[64];
+  float Ev[kIntMaxVars + 1];
+  int Fv[kIntMaxVars + 1];
+  int4 acc[(kIntMaxVars + 1) * Q];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, T = blockDim.x >> 5, G = T / S;
+  const int s = warp % S, w0 = warp - s;  // this warp's part, its polynomial's first warp
+  const int nv = a.nv, n_slots = nv + 1;
+  const int64_t n = a.v.npts, plane = (int64_t)nv * 2 * L * n, n_blocks = (n + 31) / 32;
+  const int n_groups = (a.np + G - 1) / G;
+  const SmemPoints<L> X{xs, lane};
+  const SmemLog lg{lgs, lane};
+  RowAcc<L> row{acc, Fv, nv};
+  for (int64_t item = blockIdx.x; item < n_blocks * n_groups; item += gridDim.x) {
+    const int64_t p = (item % n_blocks) * 32 + lane;
+    const int j = (int)(item / n_blocks) * G + warp / S;
+    const bool work = j < a.np;  // uniform in a warp; every warp takes every barrier
+    __syncthreads();
+    stage_points<L>(a.v.x, nv, n, p, xs, lgs);
+    __syncthreads();
+    int m0 = 0, m1 = 0, mb = 0, me = 0;
+    if (work) {
+      m0 = a.poly_off[j];
+      m1 = a.poly_off[j + 1];
+      // monomials [mb, me): the first whose steps begin at or past s/S and (s+1)/S of the polynomial's
+      const int b0 = ip.step_off[m0];
+      const int64_t len = ip.step_off[m1] - b0;
+      auto cut = [&](int k) {
+        const int target = b0 + (int)(len * k / S);
+        int lo = m0, hi = m1;
+        while (lo < hi) {
+          const int mid = (lo + hi) / 2;
+          if (ip.step_off[mid] < target)
+            lo = mid + 1;
+          else
+            hi = mid;
+        }
+        return lo;
+      };
+      mb = cut(s);
+      me = cut(s + 1);
+      Ev[nv] = mpi::bounds_for_poly(ip.mon_off, ip.pairs, ip.clg, mb, me, lg, nv, Ev);
+      for (int i = 0; i < n_slots; ++i) red[(warp * n_slots + i) * 32 + lane] = Ev[i];
     }
     __syncthreads();
-    if (!live) continue;  // lanes past the ragged tail sit the block out
-    for (int j = g * T + warp; j < a.np && j < (g + 1) * T; j += T) {
-      double vre[L], vim[L];
-      int_row<L>(a.v.mon_off, a.v.pairs, cfz, clg, a.poly_off[j], a.poly_off[j + 1], X, lg, a.nv,
-                 a.jac + (int64_t)j * plane, n, p, vre, vim, P);
+    if (work) {
+      for (int i = 0; i < n_slots; ++i) {
+        float E = red[(w0 * n_slots + i) * 32 + lane];
+        for (int k = 1; k < S; ++k) E = fmaxf(E, red[((w0 + k) * n_slots + i) * 32 + lane]);
+        Fv[i] = mpi::frame_of<WA>(E, m1 - m0);
+        row.zero(i);
+      }
+      mpi::run_steps<L>(ip.steps + ip.step_off[mb], ip.steps + ip.step_off[me], cfz + mb, X, row, P);
+    }
+    // R slots of every polynomial at a time through shared memory
+    for (int i0 = 0; i0 < n_slots; i0 += R) {
+      __syncthreads();  // the bounds, or the previous slots, are no longer read
+      if (work)
+        for (int r = 0; r < R && i0 + r < n_slots; ++r)
 #pragma unroll
-      for (int l = 0; l < L; ++l) {
-        a.val[((int64_t)(j * 2) * L + l) * n + p] = vre[l];
-        a.val[((int64_t)(j * 2 + 1) * L + l) * n + p] = vim[l];
+          for (int k = 0; k < Q; ++k) part[((warp * R + r) * Q + k) * 32 + lane] = acc[(i0 + r) * Q + k];
+      __syncthreads();
+      for (int r = s; r < R; r += S) {
+        const int i = i0 + r;
+        if (!work || i >= n_slots || p >= n) continue;
+        int64_t c[2 * WA];
+#pragma unroll
+        for (int k = 0; k < 2 * WA; ++k) c[k] = 0;
+        for (int q = 0; q < S; ++q)
+#pragma unroll
+          for (int k = 0; k < Q; ++k) {
+            const int4 v = part[(((w0 + q) * R + r) * Q + k) * 32 + lane];
+            c[4 * k] += v.x;
+            c[4 * k + 1] += v.y;
+            c[4 * k + 2] += v.z;
+            c[4 * k + 3] += v.w;
+          }
+        mpi::carry<WA>(c);
+        mpi::carry<WA>(c + WA);
+        int32_t ar[WA], ai[WA];
+#pragma unroll
+        for (int k = 0; k < WA; ++k) {
+          ar[k] = (int32_t)c[k];
+          ai[k] = (int32_t)c[WA + k];
+        }
+        store_slot<L>(ar, ai, Fv[i], (i == nv ? a.val + (int64_t)j * 2 * L * n : a.jac + (int64_t)j * plane + (int64_t)i * 2 * L * n) + p, n);
       }
     }
+  }
+}
+
+// Raise a kernel's dynamic shared-memory limit (per device) only when a larger
+// system needs more, not on every launch.
+template <class K>
+static void raise_smem(K kern, size_t smem, size_t* set) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev < 0 || dev >= 64 || smem > set[dev]) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (dev >= 0 && dev < 64) set[dev] = smem;
   }
 }
 
 template <int L>
 static int launch_int(const EvalArgs& a, const ht_system* s, int threads, cudaStream_t st) {
   const auto* cf = reinterpret_cast<const mpi::fz<IntW<L>::W>*>(s->d_coef_fz);
+  const IntPoly ip{s->d_mon_off, s->d_pairs, s->d_step_off, s->d_steps, s->d_coef_lg};
   if (threads == 256) {  // block organisation (points in shared memory)
-    // 16 warps share one copy of the points where there are polynomials for
-    // them: half the shared memory of two 8-warp CTAs per SM, so more of the
-    // SM's L1 holds the lanes' forward products (8 % faster for QD at
-    // n = 32); the register cap (128) is the same for both sizes
-    const int cta = a.np >= 16 ? 512 : 256;
-    const size_t smem = (size_t)a.nv * 32 * ((2 * IntW<L>::W + 1) * sizeof(int32_t) + sizeof(float));
-    // raise the kernel's dynamic shared-memory limit (per device) only when a
-    // larger system needs more, not on every launch
-    static size_t smem_set[64] = {0};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64 || smem > smem_set[dev]) {
-      cudaFuncSetAttribute(evaldiff_intblk_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (dev >= 0 && dev < 64) smem_set[dev] = smem;
+    const int64_t n_blocks = (a.v.npts + 31) / 32, sms = sm_count();
+    const size_t xbytes = smem_points_bytes<L>(a.nv);
+    // Warps per polynomial: with up to 16 warps a CTA takes G polynomials on S
+    // warps each.  Of all S the one with the least time is taken, in units of
+    // one warp's pass over a polynomial: waves of CTAs over the SMs times 1/S,
+    // plus 1/20 a wave for the bounds' and slots' exchange.  A large batch
+    // has many waves whatever S, so it stays unsplit; at 999 points of the
+    // 16-polynomial system S = 4 fills the chip in one wave, and at 3,000
+    // points S = 8 cuts the last wave's idle part (4.4 -> 3.0 ms in QD).
+    int S = 1, G = 1;
+    double best = 1e300;
+    for (int c = 1; c <= 16 && c <= a.max_terms; ++c) {
+      const int most = std::min(a.np, 16 / c), groups = (a.np + most - 1) / most, g = (a.np + groups - 1) / groups;
+      const int64_t slots = sms * (16 / (c * g));
+      const double t = (double)((n_blocks * groups + slots - 1) / slots) * (1.0 / c + (c > 1 ? 0.05 : 0.0));
+      if (t < best * 0.98) {
+        best = t;
+        S = c;
+        G = g;
+      }
     }
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, evaldiff_intblk_kernel<L>, cta, smem);
-    if (per_sm < 1) per_sm = 1;
-    const int wpc = cta / 32;
-    int64_t want = (a.v.npts + 31) / 32 * ((a.np + wpc - 1) / wpc);  // (point block, polynomial group) items
-    int64_t grid = (int64_t)sm_count() * per_sm;
-    if (grid > want) grid = want;
-    evaldiff_intblk_kernel<L><<<(unsigned)grid, cta, smem, st>>>(a, cf, s->d_coef_lg);
+    const size_t smem_split = xbytes + (size_t)(S * G) * 32 *
+                                           std::max<size_t>((a.nv + 1) * sizeof(float), kSplitSlots<L> * 2 * IntW<L>::WA * 4);
+    if (S > 1 && smem_split <= 220 * 1024) {
+      static size_t set[64] = {0};
+      raise_smem(evaldiff_intsplit_kernel<L>, smem_split, set);
+      int per_sm = 0;
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, evaldiff_intsplit_kernel<L>, 32 * S * G, smem_split);
+      if (per_sm < 1) per_sm = 1;
+      const int64_t want = n_blocks * ((a.np + G - 1) / G);
+      const int64_t grid = want < sms * per_sm ? want : sms * per_sm;
+      evaldiff_intsplit_kernel<L><<<(unsigned)grid, 32 * S * G, smem_split, st>>>(a, ip, cf, S);
+    } else {
+      // as few groups of polynomials as the largest CTA allows, of equal size
+      const int groups = (a.np + kBlkWarps<L> - 1) / kBlkWarps<L>;
+      const int cta = 32 * ((a.np + groups - 1) / groups);
+      static size_t set[64] = {0};
+      raise_smem(evaldiff_intblk_kernel<L>, xbytes, set);
+      int per_sm = 0;
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, evaldiff_intblk_kernel<L>, cta, xbytes);
+      if (per_sm < 1) per_sm = 1;
+      const int64_t want = n_blocks * groups;  // (point block, polynomial group) items
+      const int64_t grid = want < sms * per_sm ? want : sms * per_sm;
+      evaldiff_intblk_kernel<L><<<(unsigned)grid, cta, xbytes, st>>>(a, ip, cf);
+    }
   } else {
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, evaldiff_int_kernel<L>, 128, 0);
@@ -197,7 +351,7 @@ static int launch_int(const EvalArgs& a, const ht_system* s, int threads, cudaSt
     int64_t want = (a.n_units + 3) / 4;
     int64_t grid = (int64_t)sm_count() * per_sm;
     if (grid > want) grid = want;
-    evaldiff_int_kernel<L><<<(unsigned)grid, 128, 0, st>>>(a, cf, s->d_coef_lg);
+    evaldiff_int_kernel<L><<<(unsigned)grid, 128, 0, st>>>(a, ip, cf);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "ht_eval_diff: launch");
@@ -219,8 +373,9 @@ int launch_evaldiff_l(const ht_system* s, int64_t n_pts, int j0, int j1, const d
   a.val = val;
   a.jac = jac;
   a.n_units = ((n_pts + 31) / 32) * a.np;
+  a.max_terms = s->max_terms;
   const int threads = s->eval_threads > 0 ? s->eval_threads : 128;
-  if (s->eval_variant == 2 && s->d_coef_fz && s->nv <= kIntMaxVars && s->max_k <= 64)
+  if (s->eval_variant == 2 && s->d_steps && s->nv <= kIntMaxVars && s->max_k <= 64)
     return launch_int<L>(a, s, threads, st);
   const bool loop = s->eval_variant != 0;  // default: compact bodies
   return loop ? launch_v<L, true>(a, threads, st) : launch_v<L, false>(a, threads, st);

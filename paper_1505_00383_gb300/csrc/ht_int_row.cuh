@@ -12,115 +12,49 @@ namespace ht {
 using mpi::IntW;
 constexpr int kIntMaxVars = 64;
 
-// The fixed-point accumulators of entry i of a row in the vertical layout
-// [i][2][L][n] (path/point index p fastest): 2L doubles hold 2 x 2L int32.
-template <int L>
-__device__ __forceinline__ void ld_fix(const double* jrow, int64_t i, int64_t n, int64_t p, int32_t* r, int32_t* im) {
-  const unsigned long long* q = reinterpret_cast<const unsigned long long*>(jrow) + (i * 2) * L * n + p;
-#pragma unroll
-  for (int t = 0; t < L; ++t) {
-    const unsigned long long a = q[t * n], b = q[(L + t) * n];
-    r[2 * t] = (int32_t)(uint32_t)a;
-    r[2 * t + 1] = (int32_t)(uint32_t)(a >> 32);
-    im[2 * t] = (int32_t)(uint32_t)b;
-    im[2 * t + 1] = (int32_t)(uint32_t)(b >> 32);
-  }
-}
-template <int L>
-__device__ __forceinline__ void st_fix(double* jrow, int64_t i, int64_t n, int64_t p, const int32_t* r,
-                                       const int32_t* im) {
-  unsigned long long* q = reinterpret_cast<unsigned long long*>(jrow) + (i * 2) * L * n + p;
-#pragma unroll
-  for (int t = 0; t < L; ++t) {
-    q[t * n] = (unsigned long long)(uint32_t)r[2 * t] | ((unsigned long long)(uint32_t)r[2 * t + 1] << 32);
-    q[(L + t) * n] = (unsigned long long)(uint32_t)im[2 * t] | ((unsigned long long)(uint32_t)im[2 * t + 1] << 32);
-  }
-}
-
-// The Jacobian row accumulates in place in the output slots: in the doubles
-// of the vertical layout (2L doubles hold the 2 x 2L int32 limbs) ...
+// The fixed-point accumulators of one polynomial's outputs at the lane's
+// point: slot i the derivative by x_i, slot nv the value, each 2 WA limbs
+// (re, im) in local memory, moved in 128-bit words.
 template <int L>
 struct RowAcc {
-  double* jrow;
-  int64_t n, p;
-  static constexpr int WA = IntW<L>::WA;
-  __device__ __forceinline__ void zero(int v) {
-    int32_t z[WA];
+  static constexpr int W = IntW<L>::W, WA = IntW<L>::WA, Q = WA / 2;  // int4 words per slot
+  int4* a;        // [(nv + 1) Q]
+  const int* Fv;  // frames of the slots
+  int nv;
+  __device__ __forceinline__ int at(int v) const { return v == mpi::step::VALUE ? nv : v; }
+  __device__ __forceinline__ void zero(int i) {
 #pragma unroll
-    for (int k = 0; k < WA; ++k) z[k] = 0;
-    st_fix<L>(jrow, v, n, p, z, z);
+    for (int k = 0; k < Q; ++k) a[i * Q + k] = make_int4(0, 0, 0, 0);
   }
-  __device__ __forceinline__ void add(int v, const mpi::fz<IntW<L>::W>& d, int e, int F) {
-    int32_t ar[WA], ai[WA];
-    ld_fix<L>(jrow, v, n, p, ar, ai);
-    mpi::acc_add_fast<IntW<L>::W, WA>(ar, ai, d, e, F);
-    st_fix<L>(jrow, v, n, p, ar, ai);
-  }
-  // entry v as L doubles per component, times scale (rounded once)
-  __device__ __forceinline__ void finish(int v, int F, double scale) {
-    int32_t ar[WA], ai[WA];
-    ld_fix<L>(jrow, v, n, p, ar, ai);
-    double o[L];
-    if (scale == 1.0)
-      mpi::fixed_to_doubles<WA, L>(ar, F, o);
-    else
-      mpi::fixed_scaled_to_doubles<WA, L>(ar, F, scale, o);
+  __device__ __forceinline__ void load(int i, int32_t* ar, int32_t* ai) const {
+    int32_t w[2 * WA];
 #pragma unroll
-    for (int l = 0; l < L; ++l) jrow[((int64_t)(v * 2) * L + l) * n + p] = o[l];
-    if (scale == 1.0)
-      mpi::fixed_to_doubles<WA, L>(ai, F, o);
-    else
-      mpi::fixed_scaled_to_doubles<WA, L>(ai, F, scale, o);
-#pragma unroll
-    for (int l = 0; l < L; ++l) jrow[((int64_t)(v * 2 + 1) * L + l) * n + p] = o[l];
-  }
-};
-
-// ... or in limb-string slots ([entry][2W+1][n] int32 words: exponent, re
-// limbs, im limbs; the accumulators use the limb words), finished as limb
-// strings for the integer least squares.
-template <int L>
-struct RowAccFz {
-  int32_t* zrow;
-  int64_t n, p;
-  static constexpr int W = IntW<L>::W, WA = IntW<L>::WA;
-  static_assert(WA <= W, "the accumulator limbs must fit the limb words");
-  __device__ __forceinline__ int32_t* at(int v) const { return zrow + (int64_t)v * (2 * W + 1) * n + p; }
-  __device__ __forceinline__ void zero(int v) {
-    int32_t* q = at(v);
-#pragma unroll
-    for (int k = 0; k < WA; ++k) q[(1 + k) * n] = q[(1 + W + k) * n] = 0;
-  }
-  __device__ __forceinline__ void add(int v, const mpi::fz<W>& d, int e, int F) {
-    int32_t* q = at(v);
-    int32_t ar[WA], ai[WA];
+    for (int k = 0; k < Q; ++k) {
+      const int4 q = a[i * Q + k];
+      w[4 * k] = q.x;
+      w[4 * k + 1] = q.y;
+      w[4 * k + 2] = q.z;
+      w[4 * k + 3] = q.w;
+    }
 #pragma unroll
     for (int k = 0; k < WA; ++k) {
-      ar[k] = q[(1 + k) * n];
-      ai[k] = q[(1 + W + k) * n];
-    }
-    mpi::acc_add_fast<W, WA>(ar, ai, d, e, F);
-#pragma unroll
-    for (int k = 0; k < WA; ++k) {
-      q[(1 + k) * n] = ar[k];
-      q[(1 + W + k) * n] = ai[k];
+      ar[k] = w[k];
+      ai[k] = w[WA + k];
     }
   }
-  __device__ __forceinline__ void finish(int v, int F, double scale) {
-    int32_t* q = at(v);
+  __device__ __forceinline__ void add(int v, const mpi::fz<W>& d, int e) {
+    const int i = at(v);
     int32_t ar[WA], ai[WA];
+    load(i, ar, ai);
+    mpi::acc_add_fast<W, WA>(ar, ai, d, e, Fv[i]);
+    int32_t w[2 * WA];
 #pragma unroll
     for (int k = 0; k < WA; ++k) {
-      ar[k] = q[(1 + k) * n];
-      ai[k] = q[(1 + W + k) * n];
+      w[k] = ar[k];
+      w[WA + k] = ai[k];
     }
-    const mpi::fz<W> z = mpi::fixed_scaled_to_fz<WA, W>(ar, ai, F, scale);
-    q[0] = z.f;
 #pragma unroll
-    for (int k = 0; k < W; ++k) {
-      q[(1 + k) * n] = z.r[k];
-      q[(1 + W + k) * n] = z.i[k];
-    }
+    for (int k = 0; k < Q; ++k) a[i * Q + k] = make_int4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
   }
 };
 
@@ -141,65 +75,89 @@ __device__ __forceinline__ void int_point(const double* __restrict__ x, int nv, 
   }
 }
 
-// Monomials m0..m1 of one polynomial at the lane's point: the value as L
-// doubles per component (vre, vim) and the gradient times scale in the row
-// storage (RowAcc: doubles in jrow's layout [nv][2][L][n]; RowAccFz: limb
-// strings), each entry rounded once from its exact fixed-point product.  X
-// and lg are indexable by variable (local arrays or shared-memory views); P
-// is scratch for the forward products (max monomial size entries).
-template <int L, class XA, class LG, class PS, class Row>
-__device__ void int_row_in(const int32_t* __restrict__ mon_off, const uint16_t* __restrict__ pairs,
-                           const mpi::fz<IntW<L>::W>* __restrict__ cfz, const float* __restrict__ clg, int m0,
-                           int m1, const XA& X, const LG& lg, int nv, Row& row, double* vre, double* vim, PS* P,
-                           double scale) {
+// Monomials m0..m1 of one polynomial at the lane's point.  X and lg are
+// indexable by variable (local arrays or shared-memory views); P is scratch
+// for the forward products (max monomial size entries).  Two forms: into the
+// doubles of the outputs (value vrow [2][L][n], gradient jrow [nv][2][L][n]),
+// or into limb strings: the gradient times scale (each entry rounded once
+// from its exact fixed-point product) in zrow, the value as L doubles.
+struct IntPoly {
+  const int32_t* mon_off;
+  const uint16_t* pairs;
+  const int32_t* step_off;  // range of each monomial in steps
+  const uint32_t* steps;
+  const float* clg;
+};
+template <int L, class XA, class LG, class PS>
+__device__ __forceinline__ void int_row_run(const IntPoly& s, const mpi::fz<IntW<L>::W>* __restrict__ cfz, int m0, int m1,
+                                            const XA& X, const LG& lg, int nv, RowAcc<L>& row, int* Fv, PS* P) {
+  Fv[nv] = mpi::frames_for_poly<IntW<L>::WA>(s.mon_off, s.pairs, s.clg, m0, m1, lg, nv, Fv);
+  for (int i = 0; i <= nv; ++i) row.zero(i);
+  mpi::run_steps<L>(s.steps + s.step_off[m0], s.steps + s.step_off[m1], cfz + m0, X, row, P);
+}
+// Slot i of a row (limbs ar, ai in frame F) to the output's doubles.
+template <int L>
+__device__ __forceinline__ void store_slot(const int32_t* ar, const int32_t* ai, int F, double* q, int64_t n) {
   constexpr int WA = IntW<L>::WA;
-  int Fv[kIntMaxVars];
-  const int F = mpi::frames_for_poly<WA>(mon_off, pairs, clg, m0, m1, lg, nv, Fv);
-  int32_t vr[WA], vi[WA];
+  double o[L];
+  mpi::fixed_to_doubles<WA, L>(ar, F, o);
 #pragma unroll
-  for (int k = 0; k < WA; ++k) vr[k] = vi[k] = 0;
-  for (int i = 0; i < nv; ++i) row.zero(i);
-  mpi::eval_poly_int<L>(mon_off, pairs, cfz, m0, m1, X, F, Fv, row, vr, vi, P);
-  mpi::fixed_to_doubles<WA, L>(vr, F, vre);
-  mpi::fixed_to_doubles<WA, L>(vi, F, vim);
-  for (int i = 0; i < nv; ++i) row.finish(i, Fv[i], scale);
+  for (int l = 0; l < L; ++l) q[l * n] = o[l];
+  mpi::fixed_to_doubles<WA, L>(ai, F, o);
+#pragma unroll
+  for (int l = 0; l < L; ++l) q[(L + l) * n] = o[l];
 }
 template <int L, class XA, class LG, class PS>
-__device__ void int_row(const int32_t* __restrict__ mon_off, const uint16_t* __restrict__ pairs,
-                        const mpi::fz<IntW<L>::W>* __restrict__ cfz, const float* __restrict__ clg, int m0, int m1,
-                        const XA& X, const LG& lg, int nv, double* jrow, int64_t n, int64_t p, double* vre,
-                        double* vim, PS* P, double scale = 1.0) {
-  RowAcc<L> row{jrow, n, p};
-  int_row_in<L>(mon_off, pairs, cfz, clg, m0, m1, X, lg, nv, row, vre, vim, P, scale);
+__device__ void int_row(const IntPoly& s, const mpi::fz<IntW<L>::W>* __restrict__ cfz, int m0, int m1, const XA& X,
+                        const LG& lg, int nv, double* vrow, double* jrow, int64_t n, int64_t p, PS* P) {
+  constexpr int WA = IntW<L>::WA;
+  int Fv[kIntMaxVars + 1];
+  int4 acc[(kIntMaxVars + 1) * RowAcc<L>::Q];
+  RowAcc<L> row{acc, Fv, nv};
+  int_row_run<L>(s, cfz, m0, m1, X, lg, nv, row, Fv, P);
+  for (int i = 0; i <= nv; ++i) {
+    int32_t ar[WA], ai[WA];
+    row.load(i, ar, ai);
+    store_slot<L>(ar, ai, Fv[i], (i == nv ? vrow : jrow + (int64_t)i * 2 * L * n) + p, n);
+  }
 }
 template <int L, class XA, class LG, class PS>
-__device__ void int_row_fz(const int32_t* __restrict__ mon_off, const uint16_t* __restrict__ pairs,
-                           const mpi::fz<IntW<L>::W>* __restrict__ cfz, const float* __restrict__ clg, int m0,
-                           int m1, const XA& X, const LG& lg, int nv, int32_t* zrow, int64_t n, int64_t p,
-                           double* vre, double* vim, PS* P, double scale) {
-  RowAccFz<L> row{zrow, n, p};
-  int_row_in<L>(mon_off, pairs, cfz, clg, m0, m1, X, lg, nv, row, vre, vim, P, scale);
+__device__ void int_row_fz(const IntPoly& s, const mpi::fz<IntW<L>::W>* __restrict__ cfz, int m0, int m1, const XA& X,
+                           const LG& lg, int nv, int32_t* zrow, int64_t n, int64_t p, double* vre, double* vim, PS* P,
+                           double scale) {
+  constexpr int W = IntW<L>::W, WA = IntW<L>::WA;
+  int Fv[kIntMaxVars + 1];
+  int4 acc[(kIntMaxVars + 1) * RowAcc<L>::Q];
+  RowAcc<L> row{acc, Fv, nv};
+  int_row_run<L>(s, cfz, m0, m1, X, lg, nv, row, Fv, P);
+  int32_t ar[WA], ai[WA];
+  row.load(nv, ar, ai);
+  mpi::fixed_to_doubles<WA, L>(ar, Fv[nv], vre);
+  mpi::fixed_to_doubles<WA, L>(ai, Fv[nv], vim);
+  for (int i = 0; i < nv; ++i) {
+    row.load(i, ar, ai);
+    const mpi::fz<W> z = mpi::fixed_scaled_to_fz<WA, W>(ar, ai, Fv[i], scale);
+    int32_t* q = zrow + (int64_t)i * (2 * W + 1) * n + p;
+    q[0] = z.f;
+#pragma unroll
+    for (int k = 0; k < W; ++k) {
+      q[(1 + k) * n] = z.r[k];
+      q[(1 + W + k) * n] = z.i[k];
+    }
+  }
 }
 
-// Views of a CTA's converted points in shared memory, lane-interleaved so a
-// warp's load of one word is 32 consecutive words: limb string words
-// [var][2W+1][32] (word 0 the exponent, then re limbs, then im limbs) and
-// log2 moduli [var][32].
+// Views of a CTA's converted points in shared memory: limb strings padded to
+// NW words, [var][lane][NW] (a multiple of 16 bytes, moved in 128-bit words;
+// the 12- and 20-word strides of DD and QD put the eight lanes of each
+// quarter-warp access in distinct banks), and log2 moduli [var][32].
 template <int L>
 struct SmemPoints {
-  static constexpr int W = IntW<L>::W, WORDS = 2 * W + 1;
+  static constexpr int W = IntW<L>::W, NW = mpi::fzs<W>::NW;
   const int32_t* x;
   int lane;
   __device__ __forceinline__ mpi::fz<W> operator[](int v) const {
-    const int32_t* q = x + (int64_t)v * WORDS * 32 + lane;
-    mpi::fz<W> z;
-    z.f = q[0];
-#pragma unroll
-    for (int k = 0; k < W; ++k) {
-      z.r[k] = q[(1 + k) * 32];
-      z.i[k] = q[(1 + W + k) * 32];
-    }
-    return z;
+    return static_cast<mpi::fz<W>>(reinterpret_cast<const mpi::fzs<W>*>(x)[v * 32 + lane]);
   }
 };
 struct SmemLog {
@@ -209,14 +167,12 @@ struct SmemLog {
 };
 template <int L>
 __device__ __forceinline__ void store_point(int32_t* x, int v, int lane, const mpi::fz<IntW<L>::W>& z) {
-  constexpr int W = IntW<L>::W, WORDS = 2 * W + 1;
-  int32_t* q = x + (int64_t)v * WORDS * 32 + lane;
-  q[0] = z.f;
-#pragma unroll
-  for (int k = 0; k < W; ++k) {
-    q[(1 + k) * 32] = z.r[k];
-    q[(1 + W + k) * 32] = z.i[k];
-  }
+  reinterpret_cast<mpi::fzs<IntW<L>::W>*>(x)[v * 32 + lane] = mpi::fzs<IntW<L>::W>(z);
+}
+// Bytes of shared memory for the points of nv variables.
+template <int L>
+constexpr size_t smem_points_bytes(int nv) {
+  return (size_t)nv * 32 * (sizeof(mpi::fzs<IntW<L>::W>) + sizeof(float));
 }
 
 }  // namespace ht

@@ -12,7 +12,7 @@
 struct ht_system {
   int nv = 0, np = 0, limbs = 0, device = 0;
   int64_t M = 0, n_pairs = 0;
-  int max_k = 0, max_exp = 0, max_deg = 0;
+  int max_k = 0, max_exp = 0, max_deg = 0, max_terms = 0;
   int eval_variant = -1;         // 0 unrolled, 1 compact FP64 bodies, 2 integer limbs, -1 default
   int eval_threads = 0;          // CTA size of the evaluation kernel, 0 = default (128)
   int track_team = 0;            // tuned tracker team size and rounds per launch (0: defaults)
@@ -29,6 +29,8 @@ struct ht_system {
   double* d_coef = nullptr;      // [M][2][L]
   void* d_coef_fz = nullptr;     // [M] coefficients in the integer format (L = 2, 4)
   float* d_coef_lg = nullptr;    // [M] log2 |c| (-1000 for zero)
+  int32_t* d_step_off = nullptr; // [M + 1] range of each monomial in d_steps
+  uint32_t* d_steps = nullptr;   // integer evaluation's sweep steps (systems of at most 64 variables, else NULL)
   void* d_ws = nullptr;          // workspace for the host-buffer entry points
   size_t ws_bytes = 0;
   cudaStream_t host_streams[2] = {nullptr, nullptr};  // pipelined host-buffer evaluation

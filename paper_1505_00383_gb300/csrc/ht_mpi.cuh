@@ -228,63 +228,68 @@ HT_HD void normalize_top(fz<W>& z) {
 
 // Complex product.  Columns W-2 .. 2W-1 of the exact limb product (the lower
 // ones only feed a carry below the result's last limb and are dropped).
+//
+// Three real limb products per column pair:
+//   k1 = br (ar + ai),  re = k1 - ai (br + bi),  im = k1 + ar (bi - br).
+// The columns are formed one after the other from the lowest, each on top of
+// the carry out of the one below, so only one column's sums and the carries
+// are live (forming every column before the carries held 60 accumulator
+// registers).  The operand sums have limbs below 2^30 and a column takes at
+// most W products, summed modulo 2^64; the exact column values fit in int64.
+// (The four-product form with two chains per column takes a third more
+// multiply-adds and measured 10 % slower in the QD evaluation.)
 template <int W>
 HT_HD fz<W> mul(const fz<W>& a, const fz<W>& b) {
   constexpr int C0 = W - 2 > 0 ? W - 2 : 0;  // lowest column kept
   constexpr int NC = 2 * W - C0;             // columns C0 .. 2W-1
-  // Three real limb products per column (Gauss): re = ar br - ai bi,
-  // im = (ar + ai)(br + bi) - ar br - ai bi.  The operand sums have limbs
-  // below 2^30, so a column of at most W products stays below 2^63; the
-  // columns are summed modulo 2^64 (unsigned) and the exact column values,
-  // which fit in int64, come out of the subtraction -- the same integers as
-  // the four-product form.
-  int32_t sa[W], sb[W];
+  int32_t dr[NC], di[NC];
+  int64_t cr = 0, ci = 0;  // carry into the column
+  int32_t sa[W], na[W], sb[W], db[W];
 #pragma unroll
   for (int x = 0; x < W; ++x) {
     sa[x] = a.r[x] + a.i[x];
+    na[x] = -a.i[x];
     sb[x] = b.r[x] + b.i[x];
+    db[x] = b.i[x] - b.r[x];
   }
-  uint64_t c1[NC], c2[NC], c3[NC];
 #pragma unroll
-  for (int c = 0; c < NC; ++c) c1[c] = c2[c] = c3[c] = 0;
+  for (int c = 0; c < NC - 1; ++c) {
+    int64_t k1 = 0;
 #pragma unroll
-  for (int x = 0; x < W; ++x)
-#pragma unroll
-    for (int y = 0; y < W; ++y) {
-      if (x + y < C0) continue;
-      const int c = x + y - C0;
-      c1[c] += (uint64_t)((int64_t)a.r[x] * b.r[y]);
-      c2[c] += (uint64_t)((int64_t)a.i[x] * b.i[y]);
-      c3[c] += (uint64_t)((int64_t)sa[x] * sb[y]);
+    for (int x = 0; x < W; ++x) {
+      const int y = c + C0 - x;
+      if (y < 0 || y >= W) continue;
+      k1 = (int64_t)((uint64_t)k1 + (uint64_t)((int64_t)sa[x] * b.r[y]));
     }
-  int64_t cr[NC], ci[NC];
+    uint64_t ur = (uint64_t)cr + (uint64_t)k1, ui = (uint64_t)ci + (uint64_t)k1;
 #pragma unroll
-  for (int c = 0; c < NC; ++c) {
-    cr[c] = (int64_t)(c1[c] - c2[c]);
-    ci[c] = (int64_t)(c3[c] - c1[c] - c2[c]);
+    for (int x = 0; x < W; ++x) {
+      const int y = c + C0 - x;
+      if (y < 0 || y >= W) continue;
+      ur += (uint64_t)((int64_t)na[x] * sb[y]);
+      ui += (uint64_t)((int64_t)a.r[x] * db[y]);
+    }
+    cr = (int64_t)ur;
+    ci = (int64_t)ui;
+    dr[c] = (int32_t)cr & MASK;
+    di[c] = (int32_t)ci & MASK;
+    cr >>= RB;
+    ci >>= RB;
   }
-  carry<NC>(cr);
-  carry<NC>(ci);
+  dr[NC - 1] = (int32_t)cr;
+  di[NC - 1] = (int32_t)ci;
   // window: columns [W-1, 2W-2] if the top column is only a sign, else [W, 2W-1]
-  const int64_t tr = cr[NC - 1], ti = ci[NC - 1];
+  const int32_t tr = dr[NC - 1], ti = di[NC - 1];
   const bool high = !((tr == 0 || tr == -1) && (ti == 0 || ti == -1));
   fz<W> z;
-  if (high) {
-    z.f = a.f + b.f + RB * W;
+  z.f = a.f + b.f + (high ? RB * W : RB * (W - 1));
 #pragma unroll
-    for (int k = 0; k < W; ++k) {
-      z.r[k] = (int32_t)cr[k + W - C0];
-      z.i[k] = (int32_t)ci[k + W - C0];
-    }
-  } else {
-    z.f = a.f + b.f + RB * (W - 1);
-#pragma unroll
-    for (int k = 0; k < W; ++k) {
-      z.r[k] = (int32_t)cr[k + W - 1 - C0];
-      z.i[k] = (int32_t)ci[k + W - 1 - C0];
-    }
-    z.r[W - 1] += (int32_t)(tr * (1LL << RB));  // fold a sign-only top column
-    z.i[W - 1] += (int32_t)(ti * (1LL << RB));
+  for (int k = 0; k < W; ++k) {
+    // the low window's top limb takes the sign-only top column as its bits 29 and up
+    const int32_t lr = k == W - 1 ? dr[k + W - 1 - C0] + (int32_t)((uint32_t)tr << RB) : dr[k + W - 1 - C0];
+    const int32_t li = k == W - 1 ? di[k + W - 1 - C0] + (int32_t)((uint32_t)ti << RB) : di[k + W - 1 - C0];
+    z.r[k] = high ? dr[k + W - C0] : lr;
+    z.i[k] = high ? di[k + W - C0] : li;
   }
   normalize_top<W>(z);
   return z;
@@ -327,7 +332,8 @@ HT_HD bool acc_add(int32_t* acc_r, int32_t* acc_i, const fz<W>& z, int e, int F)
 // digits 0..WA-2 come out in [0, 2^29), the top one signed.  With one zero
 // digit prepended below limb 0, digit j is bits [r, r + 29) of string digits
 // j + q and j + q + 1; the string is shifted down by q one bit of q at a time
-// (static indices only).
+// (static indices only; shifts by four and more limbs, for terms far below
+// the frame, are rare and skipped by a branch).
 template <int W, int WA>
 HT_HD void shifted_digits(const int32_t* z, int q, int r, int32_t* v) {
   constexpr int N = W + WA + 4;
@@ -340,8 +346,16 @@ HT_HD void shifted_digits(const int32_t* z, int q, int r, int32_t* v) {
   D[W] = z[W - 1] & MASK;
 #pragma unroll
   for (int k = W + 1; k < N; ++k) D[k] = ext;
+  if (TOP >= 4 && q >= 4) {
 #pragma unroll
-  for (int b = TOP; b >= 1; b >>= 1) {
+    for (int b = TOP; b >= 4; b >>= 1) {
+      const bool take = (q & b) != 0;
+#pragma unroll
+      for (int k = 0; k < N; ++k) D[k] = take ? (k + b < N ? D[k + b] : ext) : D[k];
+    }
+  }
+#pragma unroll
+  for (int b = 2; b >= 1; b >>= 1) {
     const bool take = (q & b) != 0;
 #pragma unroll
     for (int k = 0; k < N; ++k) D[k] = take ? (k + b < N ? D[k + b] : ext) : D[k];

@@ -3,6 +3,7 @@
 // tests run it as is).  The reverse-mode sweep is the one of ht_eval.cuh.
 #pragma once
 #include <cmath>
+#include <vector>
 
 #include "ht_mpi.cuh"
 
@@ -47,10 +48,11 @@ HT_HD int frame_of(float E, int cnt) {
   const int Eint = (int)std::ceil((E > -3.0e4f ? E : -3.0e4f) + 1.0f) + head + 1;
   return Eint - (RB * (WA - 1) + 28);
 }
-template <int WA, class LG>
-HT_HD int frames_for_poly(const int32_t* mon_off, const uint16_t* pairs, const float* clg, int m0, int m1,
-                          const LG& lg, int nv, int* Fv) {
-  float Ev[64];
+// The bounds themselves: the returned one for the value's terms, Ev[i] for the
+// derivative's by x_i, over the monomials m0..m1.
+template <class LG>
+HT_HD float bounds_for_poly(const int32_t* mon_off, const uint16_t* pairs, const float* clg, int m0, int m1,
+                            const LG& lg, int nv, float* Ev) {
   for (int i = 0; i < nv; ++i) Ev[i] = -3.0e4f;
   float E = -3.0e4f;
   for (int m = m0; m < m1; ++m) {
@@ -68,140 +70,122 @@ HT_HD int frames_for_poly(const int32_t* mon_off, const uint16_t* pairs, const f
       Ev[v] = Ev[v] > d ? Ev[v] : d;
     }
   }
+  return E;
+}
+template <int WA, class LG>
+HT_HD int frames_for_poly(const int32_t* mon_off, const uint16_t* pairs, const float* clg, int m0, int m1,
+                          const LG& lg, int nv, int* Fv) {
+  float Ev[64];
+  const float E = bounds_for_poly(mon_off, pairs, clg, m0, m1, lg, nv, Ev);
   const int cnt = m1 - m0;
   for (int i = 0; i < nv; ++i) Fv[i] = frame_of<WA>(Ev[i], cnt);
   return frame_of<WA>(E, cnt);
 }
 
-// Value (through val_add(term)) and gradient (through acc.add(var, d, e,
-// Fv[var])) of monomial m at the point X (converted variables); P is scratch
-// for k forward products.
-//
 // The reverse-mode sweep of one monomial c x_{v_0}^{a_0} ... x_{v_{k-1}}^{a_{k-1}}
-// is a sequence of steps, each at most one product followed by one action:
-//   common factor  cf <- cf x_{v_r}              (a_r - 1 times for each r)
-//   forward        P_r <- (r ? P_{r-1} : cf) x_{v_r};  value += P_{k-1}
-//   backward       d_{k-1} = P_{k-2}; S = x_{v_{k-1}};
-//                  for r = k-2 .. 1: d_r = P_{r-1} S, S <- S x_{v_r};
-//                  d_0 = cf S                     (k = 1: d_0 = cf)
-// with every d_r added into the row as a_r d_r (acc.add) and the value through
-// val_add.  The loop runs the steps of a monomial through a single product
-// and a single accumulation site, so the multi-limb product is emitted once
-// (the 8-limb product is several hundred instructions) and its operands stay
-// in registers.
-template <int L, class XA, class Acc, class ValAdd, class PS>
-HT_HD void sweep_monomial(const int32_t* mon_off, const uint16_t* pairs, const fz<IntW<L>::W>* cfz, int m,
-                          const XA& X, const int* Fv, Acc& acc, ValAdd& val_add, PS* P) {
+// as a list of steps, built once per system (sweep_steps).  The state is one
+// running limb string cur (the common factor, then the forward products, then
+// the product S of the variables behind the derivative at hand) and the
+// stored forward products P (P[0] = cf, P[r] = cf x_{v_0} .. x_{v_{r-1}}):
+//   START  cur = c
+//   MULX   cur <- cur x_v      common factor, forward products, S
+//   TOP    cur = x_{v_{k-1}};  the derivative by it is P[k-1]
+//   MULP   the derivative by x_{v_r} is P[r] cur
+// A step may store its result in P, and may add it to an output: to the value,
+// or a_r times to the derivative by x_{v_r}.  Every product has cur as one
+// operand and a string read from memory as the other, so the product and the
+// accumulation are each emitted once (the 8-limb product is several hundred
+// instructions) and only cur and the result stay in registers.
+namespace step {
+enum : uint32_t { START = 0, MULX = 1, TOP = 2, MULP = 3 };
+constexpr int VALUE = 127;  // output slot of the polynomial's value
+// bits 0-1 kind, 2 store, 3 add, 4-10 variable, 11-17 index of P (stored, or
+// TOP's and MULP's source), 18-24 output slot, 25-31 exponent (at most 127)
+inline uint32_t make(uint32_t kind, int var, int p, bool store, bool add, int slot, int e) {
+  return kind | (store ? 4u : 0u) | (add ? 8u : 0u) | (uint32_t)var << 4 | (uint32_t)p << 11 | (uint32_t)slot << 18 |
+         (uint32_t)e << 25;
+}
+}  // namespace step
+
+// Append the steps of a monomial with the k <= 64 variables pr (variable | exponent << 8).
+template <class Out>
+inline void sweep_steps(const uint16_t* pr, int k, Out& out) {
+  int chain = 0;  // products of the common factor
+  for (int r = 0; r < k; ++r) chain += (pr[r] >> 8) - 1;
+  out.push_back(step::make(step::START, 0, 0, k > 0 && chain == 0, k == 0, step::VALUE, 1));
+  for (int r = 0; r < k; ++r)
+    for (int e = 1; e < (pr[r] >> 8); ++e) {
+      --chain;
+      out.push_back(step::make(step::MULX, pr[r] & 0xff, 0, chain == 0, false, 0, 1));
+    }
+  for (int r = 0; r < k; ++r)  // the last forward product is the value
+    out.push_back(step::make(step::MULX, pr[r] & 0xff, (r + 1) & 63, r + 1 < k, r + 1 == k, step::VALUE, 1));
+  for (int r = k - 1; r >= 0; --r) {
+    const int v = pr[r] & 0xff, e = pr[r] >> 8;
+    out.push_back(step::make(r == k - 1 ? step::TOP : step::MULP, v, r, false, true, v, e));
+    if (r >= 1 && r < k - 1) out.push_back(step::make(step::MULX, v, 0, false, false, 0, 1));
+  }
+}
+
+// Run the steps st..end of consecutive monomials with the coefficients cf[0..]
+// at the point X (converted variables): acc.add(slot, t, e) receives every
+// result that is added; P is scratch for the forward products.
+template <int L, class XA, class Acc, class PS>
+HT_HD void run_steps(const uint32_t* st, const uint32_t* end, const fz<IntW<L>::W>* cf, const XA& X, Acc& acc, PS* P) {
   constexpr int W = IntW<L>::W;
   using Z = fz<W>;
-  enum : int { CHAIN, FWD, BWD0, BWD_D, BWD_S, LAST, DONE };
-  const int beg = mon_off[m], k = mon_off[m + 1] - beg;
-  const uint16_t* pr = pairs + beg;
-  Z cf = cfz[m], S = cf;
-  if (k == 0) {
-    val_add(cf);
-    return;
-  }
-  int phase = CHAIN, r = 0, e = 1;
-  while (phase != DONE) {
-    // the step: operands, whether to multiply, and the action
-    Z lhs, rhs;
-    bool prod = true;
-    int act = 0;  // 0 cf, 1 P[r] (+ value at r = k - 1), 2 S, 3 row entry of var
-    int var = 0, ex = 1;
-    if (phase == CHAIN) {
-      while (r < k && e >= (pr[r] >> 8)) {  // next variable with exponent left
-        ++r;
-        e = 1;
-      }
-      if (r == k) {
-        phase = FWD;
-        r = 0;
-        continue;
-      }
-      lhs = cf;
-      rhs = X[pr[r] & 0xff];
-      act = 0;
-      ++e;
-    } else if (phase == FWD) {
-      lhs = r == 0 ? cf : static_cast<Z>(P[r - 1]);
-      rhs = X[pr[r] & 0xff];
-      act = 1;
-    } else if (phase == BWD0) {  // d_{k-1} = P_{k-2} (k >= 2) or d_0 = cf (k = 1)
-      lhs = k == 1 ? cf : static_cast<Z>(P[k - 2]);
-      prod = false;
-      act = 3;
-      var = pr[k - 1] & 0xff;
-      ex = pr[k - 1] >> 8;
-    } else if (phase == BWD_D) {
-      lhs = static_cast<Z>(P[r - 1]);
-      rhs = S;
-      act = 3;
-      var = pr[r] & 0xff;
-      ex = pr[r] >> 8;
-    } else if (phase == BWD_S) {
-      lhs = S;
-      rhs = X[pr[r] & 0xff];
-      act = 2;
-    } else {  // LAST: d_0 = cf S
-      lhs = cf;
-      rhs = S;
-      act = 3;
-      var = pr[0] & 0xff;
-      ex = pr[0] >> 8;
-    }
-    const Z t = prod ? mul<W>(lhs, rhs) : lhs;
-    if (act == 0) {
-      cf = t;
-    } else if (act == 1) {
-      if (r == k - 1)
-        val_add(t);  // the last forward product is the value; the backward sweep never reads it
-      else
-        P[r] = t;
-    } else if (act == 2) {
-      S = t;
+  Z cur;
+  uint32_t next = st != end ? *st : 0;
+  while (st != end) {
+    const uint32_t o = next, kind = o & 3u;
+    if (++st != end) next = *st;
+    const int p = (int)(o >> 11) & 127;
+    Z t;
+    if (kind == step::START) {
+      t = cur = *cf++;
+    } else if (kind == step::TOP) {
+      t = static_cast<Z>(P[p]);
+      cur = X[(o >> 4) & 127];
     } else {
-      acc.add(var, t, ex, Fv[var]);
+      Z b;
+      if (kind == step::MULX)
+        b = X[(o >> 4) & 127];
+      else
+        b = static_cast<Z>(P[p]);
+      t = mul<W>(cur, b);
+      if (kind == step::MULX) cur = t;
     }
-    // next step
-    if (phase == FWD) {
-      if (++r == k) phase = BWD0;
-    } else if (phase == BWD0) {
-      if (k == 1) {
-        phase = DONE;
-      } else {
-        S = X[pr[k - 1] & 0xff];
-        r = k - 2;
-        phase = r >= 1 ? BWD_D : LAST;
-      }
-    } else if (phase == BWD_D) {
-      phase = BWD_S;
-    } else if (phase == BWD_S) {
-      --r;
-      phase = r >= 1 ? BWD_D : LAST;
-    } else if (phase == LAST) {
-      phase = DONE;
-    }
+    if (o & 4u) P[p] = t;
+    if (o & 8u) acc.add((int)(o >> 18) & 127, t, (int)(o >> 25));
   }
 }
 
-// Multiplications of one monomial's sweep (for balancing work over lanes).
-HT_HD int sweep_products(const uint16_t* pr, int k) {
-  int c = 0;
-  for (int r = 0; r < k; ++r) c += (pr[r] >> 8) - 1;
-  return k == 0 ? 0 : c + (k == 1 ? 1 : 3 * k - 3);
-}
-
-// Value (fixed-point vr, vi in frame F) and gradient of the monomials m0..m1.
-// X is anything indexable by variable that yields the converted limb string
-// (a local array, or a view of shared memory).
+#if !defined(__CUDACC__)
+// Value (fixed-point vr, vi in frame F) and gradient (through acc.add(var, d,
+// e, Fv[var])) of the monomials m0..m1 given by their pairs, on the host: the
+// steps the device runs, built here.  X is anything indexable by variable
+// that yields the converted limb string.
 template <int L, class XA, class Acc, class PS>
-HT_HD void eval_poly_int(const int32_t* mon_off, const uint16_t* pairs, const fz<IntW<L>::W>* cfz, int m0, int m1,
-                         const XA& X, int F, const int* Fv, Acc& acc, int32_t* vr, int32_t* vi, PS* P) {
+inline void eval_poly_int(const int32_t* mon_off, const uint16_t* pairs, const fz<IntW<L>::W>* cfz, int m0, int m1,
+                          const XA& X, int F, const int* Fv, Acc& acc, int32_t* vr, int32_t* vi, PS* P) {
   constexpr int W = IntW<L>::W, WA = IntW<L>::WA;
-  auto val_add = [&](const fz<W>& t) { acc_add_fast<W, WA>(vr, vi, t, 1, F); };
-  for (int m = m0; m < m1; ++m) sweep_monomial<L>(mon_off, pairs, cfz, m, X, Fv, acc, val_add, P);
+  std::vector<uint32_t> st;
+  for (int m = m0; m < m1; ++m) sweep_steps(pairs + mon_off[m], mon_off[m + 1] - mon_off[m], st);
+  struct {
+    Acc& acc;
+    const int* Fv;
+    int F;
+    int32_t *vr, *vi;
+    void add(int slot, const fz<W>& t, int e) {
+      if (slot == step::VALUE)
+        acc_add_fast<W, WA>(vr, vi, t, 1, F);
+      else
+        acc.add(slot, t, e, Fv[slot]);
+    }
+  } out{acc, Fv, F, vr, vi};
+  run_steps<L>(st.data(), st.data() + st.size(), cfz + m0, X, out, P);
 }
+#endif
 
 }  // namespace mpi
 }  // namespace ht

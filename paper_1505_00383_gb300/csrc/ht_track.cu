@@ -565,10 +565,10 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
   // L1 capacity from the Newton workspace.  Only warp 0's sample staging
   // lives in shared memory.
   __shared__ MlpWarpSmem mlp_stage;
-  // INT: the group's converted working points ([n][2W+1][32] words, then
+  // INT: the group's converted working points ([n][32][NW] words, then
   // [n][32] log2 moduli), dynamic shared memory sized by the launcher
   extern __shared__ __align__(16) int32_t xs_int[];
-  float* lgs_int = reinterpret_cast<float*>(xs_int + (int64_t)a.n * (2 * IntW<L>::W + 1) * 32);
+  float* lgs_int = reinterpret_cast<float*>(xs_int + a.n * 32 * SmemPoints<L>::NW);
   const int cap = a.prm.max_order + 1;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, T = blockDim.x >> 5;
   // the tangent predictors solve J v = -dh/dt as a second right-hand side
@@ -811,8 +811,8 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
           double vre[L], vim[L];
           // the row comes out as tt times the gradient, scaled in the exact
           // fixed-point sums, as the limb strings the least squares reads
-          int_row_fz<L>(a.mon_off, a.pairs, static_cast<const Z*>(a.cfz), a.clg, __ldg(a.poly_off + j),
-                        __ldg(a.poly_off + j + 1), X, lg, n, Zrow.base, m, p, vre, vim, P, tt);
+          int_row_fz<L>(IntPoly{a.mon_off, a.pairs, a.step_off, a.sweep, a.clg}, static_cast<const Z*>(a.cfz),
+                        __ldg(a.poly_off + j), __ldg(a.poly_off + j + 1), X, lg, n, Zrow.base, m, p, vre, vim, P, tt);
           const ZW fj = mpi::from_doubles<WZ, L>(vre, vim);
           const int d = __ldg(a.deg + j);
           const ZW xj = X[j];
@@ -839,23 +839,10 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
        }
       } else if (act) {
         cx<L> gs = cscale_r(gamma, r_diff<L>(1.0, tt));
-        mpi::fzs<IntW<L>::W> P[INT ? kIntMaxTrack : 1];
-        const SmemPoints<L> X{xs_int, lane};
-        const SmemLog lg{lgs_int, lane};
         for (int j = warp; j < n; j += T) {
           double* Arow = a.A + (int64_t)j * rowA;
-          cx<L> fj;
-          if constexpr (INT) {
-            double vre[L], vim[L];
-            // the row comes out as tt times the gradient, scaled in the
-            // exact fixed-point sums (one rounding, no FP64 multiplies)
-            int_row<L>(a.mon_off, a.pairs, static_cast<const Z*>(a.cfz), a.clg, __ldg(a.poly_off + j),
-                       __ldg(a.poly_off + j + 1), X, lg, n, Arow, m, p, vre, vim, P, tt);
-            fj = cx_from<L>(vre, vim);
-          } else {
-            fj = eval_poly<L>(v, __ldg(a.poly_off + j), __ldg(a.poly_off + j + 1), n, p, Arow);
-            for (int i = 0; i < n; ++i) st<L>(Arow, i, m, p, cscale(ld<L>(Arow, i, m, p), tt));
-          }
+          const cx<L> fj = eval_poly<L>(v, __ldg(a.poly_off + j), __ldg(a.poly_off + j + 1), n, p, Arow);
+          for (int i = 0; i < n; ++i) st<L>(Arow, i, m, p, cscale(ld<L>(Arow, i, m, p), tt));
           const int d = __ldg(a.deg + j);
           cx<L> xj = ld<L>(a.xp, j, m, p);
           cx<L> xd1 = creal<L>(1.0);
@@ -1147,7 +1134,7 @@ int launch_track_l(const TrackArgs& a, int team, int64_t max_groups, cudaStream_
   const bool learn = a.mlp_img != nullptr;
   const bool in = L > 1 && a.int_eval;  // the double tracker keeps FP64 evaluation
   // dynamic shared memory of the integer instantiations: the converted points
-  const size_t dsm = in ? (size_t)a.n * 32 * ((2 * IntW<L>::W + 1) * sizeof(int32_t) + sizeof(float)) : 0;
+  const size_t dsm = in ? smem_points_bytes<L>(a.n) : 0;
   auto go = [&](auto kern) {
     // the kernel's static shared memory counts against the same 48 KB default,
     // so the limit is raised for any dynamic size (n = 32 DD asks for 48 KB)

@@ -34,6 +34,8 @@ struct TrackArgs {
   const double* coef;
   const void* cfz;     // coefficients in the integer format (mpi::fz<W>), for int_eval
   const float* clg;    // log2 |c|
+  const int32_t* step_off;  // the integer evaluation's sweep steps
+  const uint32_t* sweep;
   int int_eval;        // DD/QD: evaluate f on the integer pipe
   const int32_t* deg;  // start system degrees [n]
   double gamma_re, gamma_im;

@@ -330,6 +330,8 @@ int ht_track_paths_ex(ht_system* s, const int32_t* start_deg, const double* gamm
   a.coef = s->d_coef;
   a.cfz = s->d_coef_fz;
   a.clg = s->d_coef_lg;
+  a.step_off = s->d_step_off;
+  a.sweep = s->d_steps;
   a.int_eval = int_eval;
   a.deg = (const int32_t*)(w + o_deg);
   a.gamma_re = gamma[0];
