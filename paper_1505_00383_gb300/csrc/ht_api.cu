@@ -1,4 +1,5 @@
 // C ABI entry points: argument checks, system upload, dispatch.
+#include <algorithm>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -186,9 +187,35 @@ int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8
         step_off.push_back((int32_t)steps.size());
       }
     }
-    const size_t b_hz = up(hz.size()), b_hl = up(hl.size() * sizeof(float)), b_so = up(step_off.size() * 4);
+    // double: the terms of every output
+    std::vector<uint32_t> terms;
+    std::vector<int32_t> term_off;
+    for (int j = 0; j < n_polys; ++j) {
+      const int64_t b = s->h_poly_off[j], e2 = s->h_poly_off[j + 1];
+      const int64_t slots = (e2 - b) + s->h_mon_off[e2] - s->h_mon_off[b];
+      s->max_slots = (int)std::max<int64_t>(s->max_slots, std::min<int64_t>(slots, 1 << 30));
+    }
+    if (limbs == 1 && s->max_slots < (1 << 24) && s->n_pairs + s->M < (1LL << 31)) {
+      std::vector<std::vector<uint32_t>> of(n_vars + 1);
+      term_off.assign(1, 0);
+      for (int j = 0; j < n_polys; ++j) {
+        for (auto& o : of) o.clear();
+        uint32_t slot = 0;
+        for (int64_t m = s->h_poly_off[j]; m < s->h_poly_off[j + 1]; ++m) {
+          of[0].push_back(slot++);
+          for (int32_t r = s->h_mon_off[m]; r < s->h_mon_off[m + 1]; ++r, ++slot)
+            of[1 + (s->h_pairs[r] & 0xff)].push_back(slot | (uint32_t)(s->h_pairs[r] >> 8) << 24);
+        }
+        for (auto& o : of) {
+          terms.insert(terms.end(), o.begin(), o.end());
+          term_off.push_back((int32_t)terms.size());
+        }
+      }
+    }
+    const size_t b_hz = up(hz.size()), b_hl = up(hl.size() * sizeof(float)), b_so = up(step_off.size() * 4),
+                 b_st = up(steps.size() * 4), b_to = up(term_off.size() * 4);
     void* blk = nullptr;
-    e = cudaMalloc(&blk, b_hz + b_hl + b_so + steps.size() * 4);
+    e = cudaMalloc(&blk, b_hz + b_hl + b_so + b_st + b_to + terms.size() * 4);
     if (e == cudaSuccess) {
       s->d_coef_fz = blk;
       s->d_coef_lg = (float*)((char*)blk + b_hz);
@@ -200,6 +227,12 @@ int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8
       s->d_steps = (uint32_t*)((char*)blk + b_hz + b_hl + b_so);
       e = cudaMemcpy(s->d_step_off, step_off.data(), step_off.size() * 4, cudaMemcpyHostToDevice);
       if (e == cudaSuccess) e = cudaMemcpy(s->d_steps, steps.data(), steps.size() * 4, cudaMemcpyHostToDevice);
+    }
+    if (e == cudaSuccess && !terms.empty()) {
+      s->d_term_off = (int32_t*)((char*)blk + b_hz + b_hl + b_so + b_st);
+      s->d_terms = (uint32_t*)((char*)blk + b_hz + b_hl + b_so + b_st + b_to);
+      e = cudaMemcpy(s->d_term_off, term_off.data(), term_off.size() * 4, cudaMemcpyHostToDevice);
+      if (e == cudaSuccess) e = cudaMemcpy(s->d_terms, terms.data(), terms.size() * 4, cudaMemcpyHostToDevice);
     }
     if (e != cudaSuccess) {
       cudaGetLastError();

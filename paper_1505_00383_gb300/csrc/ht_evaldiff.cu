@@ -22,6 +22,11 @@
 // Outputs are written in the vertical layout of Table tabtranspose; the
 // Jacobian row of the unit's polynomial accumulates in place in the output
 // array (it stays in L2 while the unit runs), so no scratch memory is used.
+#ifndef HT_LIMBS
+#error "compile once per precision with -DHT_LIMBS=1, 2 or 4"
+#endif
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "ht_eval.cuh"
@@ -34,6 +39,7 @@ struct EvalArgs {
   PolyView v;
   const int32_t* poly_off;  // advanced to the first polynomial of the range
   int nv, np;               // np: polynomials in the range; val and jac hold them from index 0
+  int j0;                   // first polynomial of the range
   double* val;
   double* jac;
   int64_t n_units;
@@ -55,6 +61,144 @@ __global__ void __launch_bounds__(256) evaldiff_kernel(EvalArgs a) {
     st<L>(a.val, j, n, p, v);
   }
 }
+
+#if HT_LIMBS == 1
+// The same for few points, in double: a cluster of CTAs takes one polynomial
+// for 32 points and deals its monomials to its warps.  A monomial's value and
+// derivatives go to slots in its CTA's shared memory (the forward products
+// wait in the derivatives' slots), and one warp per output then adds that
+// output's terms in monomial order, from the whole cluster's shared memory,
+// so every operation and its order are those of evaldiff_kernel, and so are
+// the bits.  Polynomials of more terms than there are slots go in chunks.
+//
+// Why: GB300 issues a double-precision warp instruction every 64 clocks on
+// each SM sub-partition, so a polynomial's time on one warp (evaldiff_kernel)
+// is its instruction count times 64 clocks, whatever the batch; here the
+// sub-partitions of one to eight SMs share it.
+__global__ void __launch_bounds__(512) evaldiff_split_kernel(EvalArgs a, const int32_t* __restrict__ term_off,
+                                                             const uint32_t* __restrict__ terms, int n_slots, int max_k) {
+  extern __shared__ __align__(16) double sm[];  // slots [n_slots][2][32], sums [nv + 1][2][32], points [nv][2][32]
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, T = blockDim.x >> 5;
+  __shared__ int cut_m[9], cut_s[9];  // the parts' first monomials and slots
+  const auto cluster = cooperative_groups::this_cluster();
+  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  double* sums = sm + (int64_t)n_slots * 64;
+  double* xs = sums + (int64_t)(a.nv + 1) * 64;
+  int* cursor = reinterpret_cast<int*>(xs + (int64_t)a.nv * 64);  // [nv + 1] next term of each output
+  const int64_t n = a.v.npts, plane = (int64_t)a.nv * 2 * n;
+  for (int64_t u = blockIdx.x / C; u < a.n_units; u += gridDim.x / C) {
+    const int j = (int)(u % a.np);
+    const int64_t pt = (u / a.np) * 32 + lane, p = pt < n ? pt : n - 1;  // lanes past the end repeat the last point
+    const int m0 = __ldg(a.poly_off + j), m1 = __ldg(a.poly_off + j + 1), o0 = (a.j0 + j) * (a.nv + 1);
+    // slot of monomial m (its value, then its derivatives), from the polynomial's first
+    auto slot_of = [&](int m) { return __ldg(a.v.mon_off + m) - __ldg(a.v.mon_off + m0) + (m - m0); };
+    for (int v = warp; v < a.nv; v += T) st<1>(xs, v, 32, lane, ld<1>(a.v.x, v, n, p));
+    __syncthreads();
+    for (int c0 = m0; c0 < m1;) {
+      // the chunk from monomial c0 in C parts, CTA k's beginning at the first
+      // monomial at or past slot s0 + k q; a part overshoots q by less than
+      // one monomial, so it fits in n_slots
+      const int s0 = slot_of(c0), q = min((slot_of(m1) - s0 + C - 1) / C, n_slots - max_k);
+      if (threadIdx.x <= C) {
+        int lo = c0, hi = m1;
+        while (lo < hi) {
+          const int mid = (lo + hi) / 2;
+          if (slot_of(mid) - s0 < (int)threadIdx.x * q)
+            lo = mid + 1;
+          else
+            hi = mid;
+        }
+        cut_m[threadIdx.x] = lo;
+        cut_s[threadIdx.x] = slot_of(lo);
+      }
+      __syncthreads();
+      const int cb = cut_m[rank], ce = cut_m[rank + 1], c1 = cut_m[C], sb = cut_s[rank];
+      for (int m = cb + warp; m < ce; m += T) {
+        const int beg = __ldg(a.v.mon_off + m), k = __ldg(a.v.mon_off + m + 1) - beg;
+        const uint16_t* pr = a.v.pairs + beg;
+        double* sl = sm + (int64_t)(slot_of(m) - sb) * 64;
+        cx<1> cf = ld_coef<1>(a.v.coef + (int64_t)m * 2);
+        for (int r = 0; r < k; ++r) {
+          const uint16_t w = __ldg(pr + r);
+          if ((w >> 8) == 1) continue;
+          const cx<1> xr = ld<1>(xs, w & 0xff, 32, lane);
+          for (int e = 1; e < (w >> 8); ++e) cf = cmul(cf, xr);
+        }
+        cx<1> P = cf;
+        for (int r = 0; r < k; ++r) {
+          st<1>(sl, 1 + r, 32, lane, P);
+          P = cmul(P, ld<1>(xs, __ldg(pr + r) & 0xff, 32, lane));
+        }
+        st<1>(sl, 0, 32, lane, P);
+        if (k < 2) continue;
+        cx<1> S = ld<1>(xs, __ldg(pr + k - 1) & 0xff, 32, lane);
+        for (int r = k - 2; r >= 1; --r) {
+          st<1>(sl, 1 + r, 32, lane, cmul(ld<1>(sl, 1 + r, 32, lane), S));
+          S = cmul(S, ld<1>(xs, __ldg(pr + r) & 0xff, 32, lane));
+        }
+        st<1>(sl, 1, 32, lane, cmul(cf, S));
+      }
+      cluster.sync();
+      for (int o = rank + C * warp; o <= a.nv; o += C * T) {
+        const int end = __ldg(term_off + o0 + o + 1);
+        int t = c0 == m0 ? __ldg(term_off + o0 + o) : cursor[o];
+        cx<1> acc = c0 == m0 ? czero<1>() : ld<1>(sums, o, 32, lane);
+        // the terms' loads go ahead of the additions, which wait for each other
+        for (int k = 0; k < C; ++k) {  // the parts hold ascending slots
+          const int b = cut_s[k];
+          const double* part = cluster.map_shared_rank(sm, k);
+          int te = t, hi = end;  // terms t..te lie in this part
+          while (te < hi) {
+            const int mid = (te + hi) / 2;
+            if ((int)(__ldg(terms + mid) & 0xffffffu) < cut_s[k + 1])
+              te = mid + 1;
+            else
+              hi = mid;
+          }
+          constexpr int U = 8;
+          while (t < te) {
+            uint32_t w[U];
+            cx<1> v[U];
+#pragma unroll
+            for (int i = 0; i < U; ++i) w[i] = __ldg(terms + min(t + i, te - 1));
+#pragma unroll
+            for (int i = 0; i < U; ++i) v[i] = ld<1>(part, (int)(w[i] & 0xffffffu) - b, 32, lane);
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+              if (t + i >= te) break;
+              // (an exponent's conversion costs as much as an addition on the
+              // FP64 pipe; an FMA by 1 rounds as the addition does)
+              const int ex = (int)(w[i] >> 24);
+              if (ex <= 1)
+                acc = cadd(acc, v[i]);
+              else
+                acc = jacc<1>(acc, (double)ex, v[i]);
+            }
+            t = min(t + U, te);
+          }
+        }
+        if (c1 < m1) {
+          st<1>(sums, o, 32, lane, acc);
+          if (lane == 0) cursor[o] = t;
+        } else if (pt < n) {
+          if (o == 0)
+            st<1>(a.val, j, n, p, acc);
+          else
+            st<1>(a.jac + (int64_t)j * plane, o - 1, n, p, acc);
+        }
+        __syncwarp();
+      }
+      cluster.sync();  // the slots are read: the next chunk, or the end of the CTA
+      c0 = c1;
+    }
+  }
+}
+
+// Shared memory of the split kernel with n_slots slots.
+static size_t split_smem(int nv, int n_slots) {
+  return (size_t)n_slots * 512 + (size_t)(2 * nv + 1) * 512 + (size_t)(nv + 1) * sizeof(int);
+}
+#endif
 
 template <int L, bool LOOP>
 static int launch_v(const EvalArgs& a, int threads, cudaStream_t st) {
@@ -358,6 +502,46 @@ static int launch_int(const EvalArgs& a, const ht_system* s, int threads, cudaSt
   return HT_OK;
 }
 
+#if HT_LIMBS == 1
+// A cluster of C CTAs per unit: the largest of 1, 2, 4, 8 that the SMs and
+// the monomials have room for (10 points, the call: 10 polynomials of 10
+// monomials 77 us on one warp each, 30 us with C = 1, 25 us with 4; 16 of 246
+// monomials 709, 205 and, with 8, 105 us).  Returns false if the system needs
+// more shared memory.
+static bool launch_split(const EvalArgs& a, const ht_system* s, cudaStream_t st, int* rc) {
+  const int64_t sms = sm_count();
+  int C = 8;
+  while (C > 1 && (a.n_units * C > sms || C * 2 > a.max_terms)) C /= 2;
+  // slots for a CTA's part of a polynomial, up to 96 KB of them (two CTAs a SM)
+  const int n_slots = std::min(192, (s->max_slots + C - 1) / C + s->max_k);
+  const size_t smem = split_smem(a.nv, n_slots);
+  if (smem > 220 * 1024) return false;
+  static size_t set[64] = {0};
+  raise_smem(evaldiff_split_kernel, smem, set);
+  // 16 warps, fewer when a part has fewer monomials and outputs
+  const int warps = std::max(1, std::min(16, std::max(a.max_terms, a.nv + 1)));
+  int per_sm = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, evaldiff_split_kernel, 32 * warps, smem);
+  if (per_sm < 1) per_sm = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(std::min<int64_t>(a.n_units, std::max<int64_t>(1, sms * per_sm / C)) * C));
+  cfg.blockDim = dim3(32 * warps);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = C;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, evaldiff_split_kernel, a, (const int32_t*)s->d_term_off,
+                                     (const uint32_t*)s->d_terms, n_slots, s->max_k);
+  if (e == cudaSuccess) e = cudaGetLastError();
+  *rc = e == cudaSuccess ? HT_OK : cuda_fail(e, "ht_eval_diff: launch");
+  return true;
+}
+#endif
+
 template <int L>
 int launch_evaldiff_l(const ht_system* s, int64_t n_pts, int j0, int j1, const double* x, double* val, double* jac,
                       cudaStream_t st) {
@@ -370,6 +554,7 @@ int launch_evaldiff_l(const ht_system* s, int64_t n_pts, int j0, int j1, const d
   a.poly_off = s->d_poly_off + j0;  // polynomials j0 .. j1 - 1, written from output row 0
   a.nv = s->nv;
   a.np = j1 - j0;
+  a.j0 = j0;
   a.val = val;
   a.jac = jac;
   a.n_units = ((n_pts + 31) / 32) * a.np;
@@ -378,12 +563,18 @@ int launch_evaldiff_l(const ht_system* s, int64_t n_pts, int j0, int j1, const d
   if (s->eval_variant == 2 && s->d_steps && s->nv <= kIntMaxVars && s->max_k <= 64)
     return launch_int<L>(a, s, threads, st);
   const bool loop = s->eval_variant != 0;  // default: compact bodies
+#if HT_LIMBS == 1
+  // few units: two per SM sub-partition is where one warp per polynomial
+  // catches up (nash8 shape: 0.39 -> 0.18 ms at 1,000 points, 0.50 and 0.49
+  // ms at 3,000)
+  if (loop && s->d_terms && a.n_units <= 8 * (int64_t)sm_count()) {
+    int rc;
+    if (launch_split(a, s, st, &rc)) return rc;
+  }
+#endif
   return loop ? launch_v<L, true>(a, threads, st) : launch_v<L, false>(a, threads, st);
 }
 
-#ifndef HT_LIMBS
-#error "compile once per precision with -DHT_LIMBS=1, 2 or 4"
-#endif
 template int launch_evaldiff_l<HT_LIMBS>(const ht_system*, int64_t, int, int, const double*, double*, double*,
                                          cudaStream_t);
 

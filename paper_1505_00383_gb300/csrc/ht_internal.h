@@ -31,6 +31,12 @@ struct ht_system {
   float* d_coef_lg = nullptr;    // [M] log2 |c| (-1000 for zero)
   int32_t* d_step_off = nullptr; // [M + 1] range of each monomial in d_steps
   uint32_t* d_steps = nullptr;   // integer evaluation's sweep steps (systems of at most 64 variables, else NULL)
+  // double: terms of every output (polynomial j's value is output j (nv + 1),
+  // its derivative by x_i the (1 + i)-th after it) in monomial order, as slot
+  // of the polynomial (a monomial's value, then its derivatives) | exponent << 24
+  int32_t* d_term_off = nullptr; // [np (nv + 1) + 1]
+  uint32_t* d_terms = nullptr;   // NULL for a polynomial of 2^24 slots and more
+  int max_slots = 0;             // largest number of slots of a polynomial
   void* d_ws = nullptr;          // workspace for the host-buffer entry points
   size_t ws_bytes = 0;
   cudaStream_t host_streams[2] = {nullptr, nullptr};  // pipelined host-buffer evaluation

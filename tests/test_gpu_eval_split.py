@@ -43,3 +43,19 @@ def test_integer_split_matches_the_unit_kernel(ht, name, n, L):
     x[s.n_vars // 2, :, :, 0] = 0.0
     for got, ref in zip(_eval(ht, s, L, x, 2, 256), _eval(ht, s, L, x, 2, 128)):
         assert np.array_equal(got, ref)
+
+
+@pytest.mark.parametrize("name,n", [("cyclic10_shape", 1), ("cyclic10_shape", 33), ("nash8_shape", 31),
+                                    ("pieri44_shape", 999), ("pieri44_shape", 3001), ("evaldiff_n32", 70),
+                                    ("plain_n6_d", 5), ("extreme", 40)])
+def test_double_split_matches_the_unrolled_bodies(ht, name, n):
+    """The default kernel at few points (monomials over the warps of a CTA, the
+    terms of 246 monomials in chunks) against variant 0, which never splits:
+    the same operations in the same order, so the same bits."""
+    s = synth.extreme_system(3, 64, 5) if name == "extreme" else synth.config_system(name)
+    x = synth.unit_points(43, s.n_vars, n, 1)
+    x[s.n_vars // 2, :, :, 0] = 0.0
+    ref = _eval(ht, s, 1, x, 0, 0)
+    for variant in (-1, 1):
+        for got, want in zip(_eval(ht, s, 1, x, variant, 0), ref):
+            assert np.array_equal(got, want)
