@@ -25,41 +25,59 @@ HT_HD int bound_exp(const fz<W>& z) {
   return -30000;
 }
 
+// The window of W limbs of carried fixed-point strings (limbs 0..WA-2 in
+// [0, 2^29), the top signed, frame F) from the highest significant limb of
+// |re| and |im| down, the sign folded into its top limb; N components
+// (2: re and im; 1: a real).  The strings move up limb by limb while their top
+// limb only repeats the sign (mostly not at all, or once), so every index is
+// static.  A value -2^(29 k) needs limb k, although that limb is all sign.
+template <int WA, int W, int N>
+HT_HD void top_window(int32_t (*d)[WA], int& F) {
+  int up = 0;
+  while (up < WA - 1) {
+    bool only_sign = true;
+#pragma unroll
+    for (int c = 0; c < N; ++c) {
+      const int32_t sg = d[c][WA - 1] >> 31;
+      int32_t low = 0;
+#pragma unroll
+      for (int k = 0; k < WA - 1; ++k) low |= d[c][k];
+      only_sign = only_sign && d[c][WA - 1] == sg && (sg == 0 || low != 0);
+    }
+    if (!only_sign) break;
+    ++up;
+#pragma unroll
+    for (int c = 0; c < N; ++c) {
+      const int32_t sg = d[c][WA - 1] >> 31;
+#pragma unroll
+      for (int k = WA - 1; k >= 1; --k) d[c][k] = d[c][k - 1];
+      d[c][0] = 0;
+      d[c][WA - 1] += (int32_t)((uint32_t)sg << RB);
+    }
+  }
+  F += RB * (WA - W - up);
+}
+
 // Fixed-point complex (WA limbs each, frame F) to a floating fz<W>: the W
 // limbs from the highest significant one down (the sign folded into the top).
 template <int WA, int W>
 HT_HD fz<W> fixed_to_fz(const int32_t* ar_in, const int32_t* ai_in, int F) {
-  int64_t r[WA], im[WA], mr[WA], mi[WA];
+  static_assert(WA >= W, "the window lies inside the string");
+  int32_t d[2][WA];
+#pragma unroll
   for (int k = 0; k < WA; ++k) {
-    r[k] = ar_in[k];
-    im[k] = ai_in[k];
+    d[0][k] = ar_in[k];
+    d[1][k] = ai_in[k];
   }
-  carry<WA>(r);
-  carry<WA>(im);
-  const bool nr = r[WA - 1] < 0, ni = im[WA - 1] < 0;
-  for (int k = 0; k < WA; ++k) {
-    mr[k] = nr ? -r[k] : r[k];
-    mi[k] = ni ? -im[k] : im[k];
-  }
-  carry<WA>(mr);
-  carry<WA>(mi);
-  int t = 0;
-  for (int k = 0; k < WA; ++k)
-    if (mr[k] != 0 || mi[k] != 0) t = k;
+  carry32<WA>(d[0]);
+  carry32<WA>(d[1]);
   fz<W> z;
-  const int lo = t - (W - 1);  // window [lo, t]
-  z.f = F + RB * lo;
+  z.f = F;
+  top_window<WA, W, 2>(d, z.f);
+#pragma unroll
   for (int k = 0; k < W; ++k) {
-    const int src = lo + k;
-    z.r[k] = src >= 0 ? (int32_t)r[src] : 0;
-    z.i[k] = src >= 0 ? (int32_t)im[src] : 0;
-  }
-  if (t < WA - 1) {  // fold the sign extension above t into the window's top
-    if (nr) z.r[W - 1] -= (1 << RB);
-    if (ni) z.i[W - 1] -= (1 << RB);
-  } else {
-    z.r[W - 1] = (int32_t)r[WA - 1];
-    z.i[W - 1] = (int32_t)im[WA - 1];
+    z.r[k] = d[0][WA - W + k];
+    z.i[k] = d[1][WA - W + k];
   }
   normalize_top<W>(z);
   return z;
@@ -139,17 +157,49 @@ HT_HD fz<W> sum(const fz<W>* z, const int* e, int n) {
     if (e[k] != 0 && !is_zero<W>(z[k])) acc_add_fast<W, WA>(ar, ai, z[k], e[k], F);
   return fixed_to_fz<WA, W>(ar, ai, F);
 }
+// a + b or a - b: sum's frame and rounding for two terms.
+template <int W, bool SUB>
+HT_HD fz<W> add_sub(const fz<W>& a, const fz<W>& b) {
+  constexpr int WA = W + 1;
+  const int ea = bound_exp<W>(a), eb = bound_exp<W>(b);  // -30000: zero
+  const int E = ea > eb ? ea : eb;
+  const int fa = ea > -30000 ? a.f : -30000, fb = eb > -30000 ? b.f : -30000;
+  const int fmax = fa > fb ? fa : fb;
+  fz<W> z;
+  if (fmax == -30000) {
+    z.f = 0;
+#pragma unroll
+    for (int k = 0; k < W; ++k) z.r[k] = z.i[k] = 0;
+    return z;
+  }
+  int F = E + 2 - (RB * (WA - 1) + 28);
+  F = F > fmax - (RB - 1) ? F : fmax - (RB - 1);
+  int32_t ar[WA], ai[WA], dr[WA], di[WA];
+#pragma unroll
+  for (int k = 0; k < WA; ++k) ar[k] = ai[k] = dr[k] = di[k] = 0;
+  const int pa = F - a.f + RB, pb = F - b.f + RB;
+  if (ea > -30000 && pa < RB * (W + 1)) {
+    shifted_digits<W, WA>(a.r, pa / RB, pa % RB, ar);
+    shifted_digits<W, WA>(a.i, pa / RB, pa % RB, ai);
+  }
+  if (eb > -30000 && pb < RB * (W + 1)) {
+    shifted_digits<W, WA>(b.r, pb / RB, pb % RB, dr);
+    shifted_digits<W, WA>(b.i, pb / RB, pb % RB, di);
+  }
+#pragma unroll
+  for (int k = 0; k < WA; ++k) {
+    ar[k] = SUB ? ar[k] - dr[k] : ar[k] + dr[k];
+    ai[k] = SUB ? ai[k] - di[k] : ai[k] + di[k];
+  }
+  return fixed_to_fz<WA, W>(ar, ai, F);
+}
 template <int W>
 HT_HD fz<W> add(const fz<W>& a, const fz<W>& b) {
-  fz<W> t[2] = {a, b};
-  const int e[2] = {1, 1};
-  return sum<W, 2>(t, e, 2);
+  return add_sub<W, false>(a, b);
 }
 template <int W>
 HT_HD fz<W> sub(const fz<W>& a, const fz<W>& b) {
-  fz<W> t[2] = {a, b};
-  const int e[2] = {1, -1};
-  return sum<W, 2>(t, e, 2);
+  return add_sub<W, true>(a, b);
 }
 template <int W>
 HT_HD fz<W> conj(fz<W> a) {
@@ -180,20 +230,116 @@ HT_HD double real_to_double(const fz<W>& z) {
   }
   return acc;
 }
+// Real limb strings (the re part of an fz<W> whose im is zero), for 1/sqrt:
+// the product and the difference take a third of the complex ones' work and
+// give the same limbs.
+template <int W>
+struct rz {
+  int32_t f;
+  int32_t r[W];
+};
+template <int W>
+HT_HD void normalize_top(rz<W>& z) {
+  const int32_t t = z.r[W - 1] < 0 ? -z.r[W - 1] : z.r[W - 1];
+  const int s = t >= (1 << 29) ? 2 : (t >= (1 << 28) ? 1 : 0);
+  if (s == 0) return;
+#pragma unroll
+  for (int k = 0; k < W - 1; ++k)
+    z.r[k] = (int32_t)((((uint32_t)z.r[k] >> s) | ((uint32_t)z.r[k + 1] << (RB - s))) & (uint32_t)MASK);
+  z.r[W - 1] >>= s;
+  z.f += s;
+}
+template <int W>
+HT_HD rz<W> mul(const rz<W>& a, const rz<W>& b) {
+  constexpr int C0 = W - 2 > 0 ? W - 2 : 0, NC = 2 * W - C0;
+  int32_t d[NC];
+  int64_t c = 0;
+#pragma unroll
+  for (int k = 0; k < NC - 1; ++k) {
+#pragma unroll
+    for (int x = 0; x < W; ++x) {
+      const int y = k + C0 - x;
+      if (y < 0 || y >= W) continue;
+      c += (int64_t)a.r[x] * b.r[y];
+    }
+    d[k] = (int32_t)c & MASK;
+    c >>= RB;
+  }
+  d[NC - 1] = (int32_t)c;
+  const int32_t t = d[NC - 1];
+  const bool high = !(t == 0 || t == -1);
+  rz<W> z;
+  z.f = a.f + b.f + (high ? RB * W : RB * (W - 1));
+#pragma unroll
+  for (int k = 0; k < W; ++k) {
+    const int32_t lo = k == W - 1 ? d[k + W - 1 - C0] + (int32_t)((uint32_t)t << RB) : d[k + W - 1 - C0];
+    z.r[k] = high ? d[k + W - C0] : lo;
+  }
+  normalize_top<W>(z);
+  return z;
+}
+// a - b for nonzero a (b may be zero)
+template <int W>
+HT_HD rz<W> sub(const rz<W>& a, const rz<W>& b) {
+  constexpr int WA = W + 1;
+  auto bound = [](const rz<W>& z) {
+    for (int k = W - 1; k >= 0; --k) {
+      const int32_t m = z.r[k] < 0 ? -z.r[k] : z.r[k];
+      if (m != 0) return z.f + RB * k + bitlen32((uint32_t)m) + 1;
+    }
+    return -30000;
+  };
+  const int ea = bound(a), eb = bound(b);
+  const int E = ea > eb ? ea : eb, fb = eb > -30000 ? b.f : -30000, fmax = a.f > fb ? a.f : fb;
+  int F = E + 2 - (RB * (WA - 1) + 28);
+  F = F > fmax - (RB - 1) ? F : fmax - (RB - 1);
+  int32_t d[1][WA], t[WA];
+#pragma unroll
+  for (int k = 0; k < WA; ++k) d[0][k] = t[k] = 0;
+  const int pa = F - a.f + RB, pb = F - b.f + RB;
+  if (pa < RB * (W + 1)) shifted_digits<W, WA>(a.r, pa / RB, pa % RB, d[0]);
+  if (eb > -30000 && pb < RB * (W + 1)) shifted_digits<W, WA>(b.r, pb / RB, pb % RB, t);
+#pragma unroll
+  for (int k = 0; k < WA; ++k) d[0][k] -= t[k];
+  carry32<WA>(d[0]);
+  rz<W> z;
+  z.f = F;
+  top_window<WA, W, 1>(d, z.f);
+#pragma unroll
+  for (int k = 0; k < W; ++k) z.r[k] = d[0][WA - W + k];
+  normalize_top<W>(z);
+  return z;
+}
+
 // 1 / sqrt(v) for a positive real v (im = 0): Newton's iteration
 // y <- y (3 - v y^2) / 2 from the double seed; each step doubles the bits.
 template <int W>
 HT_HD fz<W> inv_sqrt(const fz<W>& v, int steps) {
   const double vd = real_to_double<W>(v);
-  fz<W> y = from_real<W>(1.0 / std::sqrt(vd));
-  const fz<W> three = from_real<W>(3.0);
+  const fz<W> seed = from_real<W>(1.0 / std::sqrt(vd)), three = from_real<W>(3.0);
+  rz<W> x, y, c3;
+  x.f = v.f;
+  y.f = seed.f;
+  c3.f = three.f;
+#pragma unroll
+  for (int k = 0; k < W; ++k) {
+    x.r[k] = v.r[k];
+    y.r[k] = seed.r[k];
+    c3.r[k] = three.r[k];
+  }
+#pragma unroll 1
   for (int it = 0; it < steps; ++it) {
-    fz<W> vy2 = mul<W>(v, mul<W>(y, y));
-    fz<W> c = sub<W>(three, vy2);
-    y = mul<W>(y, c);
+    y = mul<W>(y, sub<W>(c3, mul<W>(x, mul<W>(y, y))));
     y.f -= 1;  // halve
   }
-  return y;
+  fz<W> z;
+  z.f = y.f;
+#pragma unroll
+  for (int k = 0; k < W; ++k) {
+    z.r[k] = y.r[k];
+    z.i[k] = 0;
+  }
+  return z;
 }
 
 // ------------------------------------------------------------ least squares
