@@ -77,10 +77,10 @@ __device__ __forceinline__ void int_point(const double* __restrict__ x, int nv, 
 
 // Monomials m0..m1 of one polynomial at the lane's point.  X and lg are
 // indexable by variable (local arrays or shared-memory views); P is scratch
-// for the forward products (max monomial size entries).  Two forms: into the
-// doubles of the outputs (value vrow [2][L][n], gradient jrow [nv][2][L][n]),
-// or into limb strings: the gradient times scale (each entry rounded once
-// from its exact fixed-point product) in zrow, the value as L doubles.
+// for the forward products (max monomial size entries).  int_row_run leaves
+// the exact sums in the row's slots (the tracker goes on from there); int_row
+// rounds them into the doubles of the outputs (value vrow [2][L][n], gradient
+// jrow [nv][2][L][n]).
 struct IntPoly {
   const int32_t* mon_off;
   const uint16_t* pairs;
@@ -121,32 +121,6 @@ __device__ void int_row(const IntPoly& s, const mpi::fz<IntW<L>::W>* __restrict_
     store_slot<L>(ar, ai, Fv[i], (i == nv ? vrow : jrow + (int64_t)i * 2 * L * n) + p, n);
   }
 }
-template <int L, class XA, class LG, class PS>
-__device__ void int_row_fz(const IntPoly& s, const mpi::fz<IntW<L>::W>* __restrict__ cfz, int m0, int m1, const XA& X,
-                           const LG& lg, int nv, int32_t* zrow, int64_t n, int64_t p, double* vre, double* vim, PS* P,
-                           double scale) {
-  constexpr int W = IntW<L>::W, WA = IntW<L>::WA;
-  int Fv[kIntMaxVars + 1];
-  int4 acc[(kIntMaxVars + 1) * RowAcc<L>::Q];
-  RowAcc<L> row{acc, Fv, nv};
-  int_row_run<L>(s, cfz, m0, m1, X, lg, nv, row, Fv, P);
-  int32_t ar[WA], ai[WA];
-  row.load(nv, ar, ai);
-  mpi::fixed_to_doubles<WA, L>(ar, Fv[nv], vre);
-  mpi::fixed_to_doubles<WA, L>(ai, Fv[nv], vim);
-  for (int i = 0; i < nv; ++i) {
-    row.load(i, ar, ai);
-    const mpi::fz<W> z = mpi::fixed_scaled_to_fz<WA, W>(ar, ai, Fv[i], scale);
-    int32_t* q = zrow + (int64_t)i * (2 * W + 1) * n + p;
-    q[0] = z.f;
-#pragma unroll
-    for (int k = 0; k < W; ++k) {
-      q[(1 + k) * n] = z.r[k];
-      q[(1 + W + k) * n] = z.i[k];
-    }
-  }
-}
-
 // Views of a CTA's converted points in shared memory: limb strings padded to
 // NW words, [var][lane][NW] (a multiple of 16 bytes, moved in 128-bit words;
 // the 12- and 20-word strides of DD and QD put the eight lanes of each

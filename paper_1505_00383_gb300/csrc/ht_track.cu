@@ -21,8 +21,10 @@
 // Per-path state lives in device memory in the vertical layout of Section 3
 // ([entry][2][L][m], path index fastest) -- the "work space for multiple
 // paths" of Table tabmemory.
+#include <algorithm>
+
 #include "ht_eval.cuh"
-#include "ht_int_row.cuh"
+#include "ht_int_mgs.cuh"
 #include "ht_internal.h"
 #include "ht_mpi_ops.cuh"
 #include "ht_mlp.cuh"
@@ -387,41 +389,14 @@ __device__ __forceinline__ void stz(double* base, int64_t e, int64_t m, int64_t 
   }
 }
 
-// Storage of A and R for the integer least squares: the vertical doubles
-// (converted on every load and store) or limb strings in [entry][2W+1][m]
-// int32 words (exponent, re limbs, im limbs; loaded and stored as they are).
+// A and R of the integer least squares of more than 32 rows: the vertical
+// doubles, converted on every load and store.
 template <int L>
 struct DblStore {
   double* base;
   int64_t m, p;
   __device__ __forceinline__ mpi::fz<IntW<L>::W> ld(int64_t e) const { return ldz<L>(base, e, m, p); }
   __device__ __forceinline__ void st(int64_t e, const mpi::fz<IntW<L>::W>& z) const { stz<L>(base, e, m, p, z); }
-};
-template <int L>
-struct FzStore {
-  static constexpr int W = IntW<L>::W;
-  int32_t* base;
-  int64_t m, p;
-  __device__ __forceinline__ mpi::fz<W> ld(int64_t e) const {
-    const int32_t* q = base + e * (2 * W + 1) * m + p;
-    mpi::fz<W> z;
-    z.f = q[0];
-#pragma unroll
-    for (int k = 0; k < W; ++k) {
-      z.r[k] = q[(1 + k) * m];
-      z.i[k] = q[(1 + W + k) * m];
-    }
-    return z;
-  }
-  __device__ __forceinline__ void st(int64_t e, const mpi::fz<W>& z) const {
-    int32_t* q = base + e * (2 * W + 1) * m + p;
-    q[0] = z.f;
-#pragma unroll
-    for (int k = 0; k < W; ++k) {
-      q[(1 + k) * m] = z.r[k];
-      q[(1 + W + k) * m] = z.i[k];
-    }
-  }
 };
 
 template <int L, int N, class ST>
@@ -494,6 +469,30 @@ __global__ void __launch_bounds__(32) mgs_kernel(double* A, double* R, double* x
     mgs_team<L>(A, R, x, rows, cols, n_sys, p, p < n_sys, 0, 1);
 }
 
+// Standalone least squares on limb strings of at most 32 rows, one row per
+// lane (ht_int_mgs.cuh): the entries are converted once on loading and once on
+// storing.  R's entries below the diagonal are left as they are.
+constexpr int kMgsWarps = 4;
+template <int L>
+__global__ void __launch_bounds__(32 * kMgsWarps) mgs_rows_kernel(double* A, double* R, double* x, int rows, int cols,
+                                                               int64_t n_sys) {
+  using Z = mpi::fz<IntW<L>::W>;
+  __shared__ __align__(16) int32_t xch[kMgsWarps][RowLanes<L>::WORDS];
+  const int warp = threadIdx.x >> 5, pp = RowLanes<L>::systems(rows), Wc = cols + 1;
+  RowLanes<L> rl(rows, xch[warp]);
+  const int64_t n_chunks = (n_sys + pp - 1) / pp;
+  for (int64_t c = (int64_t)blockIdx.x * kMgsWarps + warp; c < n_chunks; c += (int64_t)gridDim.x * kMgsWarps) {
+    const int64_t p = c * pp + rl.sub;
+    rl.row = rl.sub < pp && p < n_sys;
+    const int i = rl.i;
+    rl.template solve<33>(
+        cols, 1, [&](int j) { return ldz<L>(A, (int64_t)i * Wc + j, n_sys, p); },
+        [&](int j, const Z& z) { stz<L>(A, (int64_t)i * Wc + j, n_sys, p, z); },
+        [&](int j, const Z& z) { stz<L>(R, (int64_t)i * Wc + j, n_sys, p, z); },
+        [&](int, const Z& z) { stz<L>(x, i, n_sys, p, z); });
+  }
+}
+
 // The learned proposal for the paths of one warp (all 32 lanes call it; want
 // marks the lanes whose path starts a learned step): features, the network
 // on the tensor cores, and h e^rho clamped.  Out of line so that the
@@ -553,7 +552,7 @@ __device__ __forceinline__ cx<L> cx_from(const double* re, const double* im) {
 // MAXT: the largest team (8, or 16 for the wide instantiation that serves
 // few groups of double and double-double paths with more warps each, and
 // any group when the autotuner picks 16).
-template <int L, bool LEARN, bool INT, int MAXT = 8>
+template <int L, bool LEARN, bool INT, int MAXT = INT ? 16 : 8>
 __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 2 ? 2 : 1))) track_kernel(TrackArgs a) {
   __shared__ double red[4][MAXT][32];  // per-warp partials: residual, update, point norms; finiteness
   __shared__ double sh_h[32];       // learned step of each lane's path
@@ -566,7 +565,8 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
   // lives in shared memory.
   __shared__ MlpWarpSmem mlp_stage;
   // INT: the group's converted working points ([n][32][NW] words, then
-  // [n][32] log2 moduli), dynamic shared memory sized by the launcher
+  // [n][32] log2 moduli) while the rows are evaluated, the solve's exchange
+  // buffers (one a warp) after; dynamic shared memory sized by the launcher
   extern __shared__ __align__(16) int32_t xs_int[];
   float* lgs_int = reinterpret_cast<float*>(xs_int + a.n * 32 * SmemPoints<L>::NW);
   const int cap = a.prm.max_order + 1;
@@ -577,11 +577,15 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
   const int64_t m = a.m;
   const int count = *a.count_in;
   const int64_t rowA = (int64_t)W * 2 * L * m;  // doubles per row of A
-  // DD and QD with integer evaluation keep A and R as limb strings
-  // ([entry][2W+1][m] words) from the evaluation through the least squares:
-  // no conversions
+  // DD and QD with integer evaluation keep A as limb strings from the
+  // evaluation through the least squares: no conversions
   constexpr bool FZ = INT && L >= 2;
-  const int64_t rowZ = (int64_t)W * (2 * IntW<L>::W + 1) * m;  // words per row of A
+  // (one row per lane: entry j of the rows of a warp's systems is NQ 128-bit
+  // words a lane, [chunk][j][NQ][32]; the CTA's own workspace, which its
+  // groups reuse, stays in L2)
+  constexpr int NQ = mpi::fzs<IntW<L>::W>::NW / 4;
+  const int pp = RowLanes<L>::systems(n), chunks = (32 + pp - 1) / pp;  // systems a warp, warps' worth a group
+  int4* const Acta = reinterpret_cast<int4*>(a.A) + (int64_t)blockIdx.x * chunks * W * NQ * 32;
   PolyView v;
   v.mon_off = a.mon_off;
   v.pairs = a.pairs;
@@ -801,18 +805,31 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
         using ZW = mpi::fz<IntW<L>::W>;
         constexpr int WZ = IntW<L>::W;
         mpi::fzs<IntW<L>::W> P[INT ? kIntMaxTrack : 1];
+        int Fv[kIntMaxTrack + 1];
+        int4 acc[(kIntMaxTrack + 1) * RowAcc<L>::Q];
+        RowAcc<L> row{acc, Fv, n};
         const SmemPoints<L> X{xs_int, lane};
         const SmemLog lg{lgs_int, lane};
+        const IntPoly ip{a.mon_off, a.pairs, a.step_off, a.sweep, a.clg};
         const ZW gz = fz_of<L>(gamma);
         const ZW gsz = fz_of<L>(cscale_r(gamma, r_diff<L>(1.0, tt)));  // gamma (1 - tt)
         const ZW ttz = mpi::from_real<WZ>(tt), one = mpi::from_real<WZ>(1.0);
+        const int ch = lane / pp, sl = (lane - ch * pp) * n;  // this path's chunk and its first lane there
         for (int j = warp; j < n; j += T) {
-          const FzStore<L> Zrow{reinterpret_cast<int32_t*>(a.A) + (int64_t)j * rowZ, m, p};
+          int4* const out = Acta + (int64_t)ch * W * NQ * 32 + sl + j;  // this row's lane of the solve
+          auto put = [&](int c, const ZW& z) {
+            const mpi::fzs<WZ> q(z);
+#pragma unroll
+            for (int k = 0; k < NQ; ++k)
+              out[(c * NQ + k) * 32] = make_int4(q.w[4 * k], q.w[4 * k + 1], q.w[4 * k + 2], q.w[4 * k + 3]);
+          };
+          int_row_run<L>(ip, static_cast<const Z*>(a.cfz), __ldg(a.poly_off + j), __ldg(a.poly_off + j + 1), X, lg, n, row,
+                         Fv, P);
           double vre[L], vim[L];
-          // the row comes out as tt times the gradient, scaled in the exact
-          // fixed-point sums, as the limb strings the least squares reads
-          int_row_fz<L>(IntPoly{a.mon_off, a.pairs, a.step_off, a.sweep, a.clg}, static_cast<const Z*>(a.cfz),
-                        __ldg(a.poly_off + j), __ldg(a.poly_off + j + 1), X, lg, n, Zrow.base, m, p, vre, vim, P, tt);
+          int32_t ar[IntW<L>::WA], ai[IntW<L>::WA];
+          row.load(n, ar, ai);
+          mpi::fixed_to_doubles<IntW<L>::WA, L>(ar, Fv[n], vre);
+          mpi::fixed_to_doubles<IntW<L>::WA, L>(ai, Fv[n], vim);
           const ZW fj = mpi::from_doubles<WZ, L>(vre, vim);
           const int d = __ldg(a.deg + j);
           const ZW xj = X[j];
@@ -820,14 +837,19 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
           for (int e = 0; e < d - 1; ++e) xd1 = e == 0 ? xj : mpi::mul<WZ>(xd1, xj);
           const ZW gval = mpi::sub<WZ>(mpi::mul<WZ>(xd1, xj), one);  // x_j^d - 1
           ZW t2[2] = {mpi::mul<WZ>(gsz, gval), mpi::mul<WZ>(ttz, fj)};
-          const int e_add[2] = {1, 1}, e_neg[2] = {-1, -1};
-          const ZW hj = mpi::sum<WZ, 2>(t2, e_add, 2);
-          const ZW mh = mpi::sum<WZ, 2>(t2, e_neg, 2);
+          const int e_neg[2] = {-1, -1};
+          const ZW hj = mpi::add<WZ>(t2[0], t2[1]);
+          put(n, mpi::sum<WZ, 2>(t2, e_neg, 2));
+          if (nrhs == 2) put(n + 1, mpi::sub<WZ>(mpi::mul<WZ>(gz, gval), fj));  // -dh/dt = gamma g - f
           const int e_d[1] = {d};
           const ZW dg = mpi::mul<WZ>(gsz, mpi::sum<WZ, 1>(&xd1, e_d, 1));  // gamma (1 - tt) d x_j^(d-1)
-          Zrow.st(j, mpi::add<WZ>(Zrow.ld(j), dg));
-          Zrow.st(n, mh);
-          if (nrhs == 2) Zrow.st(n + 1, mpi::sub<WZ>(mpi::mul<WZ>(gz, gval), fj));  // -dh/dt = gamma g - f
+          // the row is tt times the gradient, scaled in the exact fixed-point sums
+          for (int i = 0; i < n; ++i) {
+            row.load(i, ar, ai);
+            ZW z = mpi::fixed_scaled_to_fz<IntW<L>::WA, WZ>(ar, ai, Fv[i], tt);
+            if (i == j) z = mpi::add<WZ>(z, dg);
+            put(i, z);
+          }
           // the residual's modulus from its leading limb; a non-finite
           // coordinate (which limb strings cannot carry) makes it NaN
           double hr, hi;
@@ -861,14 +883,37 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
       __syncthreads();
       // ---- C: least squares J dx = -h by modified Gram-Schmidt
       // DD and QD with integer evaluation solve on the integer pipe, on the
-      // limb strings in A and R (for DD the FP64 MGS had been faster while
-      // every load and store converted: 1.6 s against 3.1 s for the n = 12,
-      // 4,096-path run; without conversions the integer path takes 1.08 s
-      // against 1.43 s)
-      if constexpr (FZ)
-        mgs_team_int<L, kIntMaxTrack>(FzStore<L>{reinterpret_cast<int32_t*>(a.A), m, p},
-                                      FzStore<L>{reinterpret_cast<int32_t*>(a.R), m, p}, a.dx, n, n, m, p, act, warp,
-                                      T, nrhs, a.tdx);
+      // limb strings in A, a row per lane; the warps deal the group's systems
+      // and exchange through the points' shared memory, which this round no
+      // longer reads
+      if constexpr (FZ) {
+        const unsigned live = __ballot_sync(0xffffffffu, act);
+        RowLanes<L> rl(n, xs_int + warp * RowLanes<L>::WORDS);
+        for (int c = warp; c < chunks; c += T) {
+          const int pl = c * pp + rl.sub;  // the system's path in the group
+          if (((live >> (c * pp)) & (pp >= 32 ? ~0u : (1u << pp) - 1u)) == 0) continue;
+          const int64_t ps = __shfl_sync(0xffffffffu, (int)p, min(pl, 31));
+          rl.row = rl.sub < pp && pl < 32 && ((live >> pl) & 1u);
+          const int4* in = Acta + (int64_t)c * W * NQ * 32 + lane;
+          rl.template solve<kIntMaxTrack + 2>(
+              n, nrhs,
+              [&](int j) {
+                mpi::fzs<IntW<L>::W> q;
+#pragma unroll
+                for (int k = 0; k < NQ; ++k) {
+                  const int4 w = in[(j * NQ + k) * 32];
+                  q.w[4 * k] = w.x;
+                  q.w[4 * k + 1] = w.y;
+                  q.w[4 * k + 2] = w.z;
+                  q.w[4 * k + 3] = w.w;
+                }
+                return static_cast<Z>(q);
+              },
+              [](int, const Z&) {}, [](int, const Z&) {},
+              [&](int k, const Z& z) { stz<L>(k == 0 ? a.dx : a.tdx, rl.i, m, ps, z); });
+        }
+        __syncthreads();
+      }
       else
         mgs_team<L>(a.A, a.R, a.dx, n, n, m, p, act, warp, T, nrhs, a.tdx);
       // ---- D: x <- x + dx on this warp's coordinates; partial norms
@@ -1091,7 +1136,11 @@ int launch_start_l(int n, const int32_t* d_deg, int64_t first, int64_t count, do
 template <int L>
 int launch_mgs_l(double* A, double* R, double* x, int rows, int cols, int64_t n_sys, int variant, cudaStream_t st) {
   if (n_sys == 0) return HT_OK;
-  if (variant == 2 && L > 1)
+  if (variant == 2 && L > 1 && rows <= 32) {
+    const int64_t chunks = (n_sys + RowLanes<L>::systems(rows) - 1) / RowLanes<L>::systems(rows);
+    const int64_t grid = std::min<int64_t>((chunks + kMgsWarps - 1) / kMgsWarps, (int64_t)sm_count() * 16);
+    mgs_rows_kernel<L><<<(unsigned)grid, 32 * kMgsWarps, 0, st>>>(A, R, x, rows, cols, n_sys);
+  } else if (variant == 2 && L > 1)
     mgs_kernel<L, L != 1><<<(unsigned)((n_sys + 31) / 32), 32, 0, st>>>(A, R, x, rows, cols, n_sys);
   else
     mgs_kernel<L, false><<<(unsigned)((n_sys + 31) / 32), 32, 0, st>>>(A, R, x, rows, cols, n_sys);
@@ -1100,6 +1149,15 @@ int launch_mgs_l(double* A, double* R, double* x, int rows, int cols, int64_t n_
 }
 
 #if HT_LIMBS == 1
+int64_t track_int_ctas(int64_t groups) { return std::max<int64_t>(1, std::min<int64_t>(groups, 4 * (int64_t)sm_count())); }
+size_t track_int_bytes(int L, int n, int nrhs) {
+  const int pp = RowLanes<2>::systems(n), chunks = (32 + pp - 1) / pp;
+  return (size_t)chunks * (n + nrhs) * 32 * (L == 4 ? sizeof(mpi::fzs<8>) : sizeof(mpi::fzs<5>));
+}
+int track_int_team(int n) {
+  const int pp = RowLanes<2>::systems(n), chunks = (32 + pp - 1) / pp;
+  return (chunks + (chunks + 15) / 16 - 1) / ((chunks + 15) / 16);
+}
 __global__ void __launch_bounds__(256) mlp_image_kernel(MlpSmem* img, const __nv_bfloat16* __restrict__ wbf,
                                                         const float* __restrict__ master) {
   mlp_load(*img, wbf, master);
@@ -1133,9 +1191,7 @@ template <int L>
 int launch_track_l(const TrackArgs& a, int team, int64_t max_groups, cudaStream_t st) {
   const bool learn = a.mlp_img != nullptr;
   const bool in = L > 1 && a.int_eval;  // the double tracker keeps FP64 evaluation
-  // dynamic shared memory of the integer instantiations: the converted points
-  const size_t dsm = in ? smem_points_bytes<L>(a.n) : 0;
-  auto go = [&](auto kern) {
+  auto go = [&](auto kern, size_t dsm) {
     // the kernel's static shared memory counts against the same 48 KB default,
     // so the limit is raised for any dynamic size (n = 32 DD asks for 48 KB)
     if (dsm > 0) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm);
@@ -1144,19 +1200,21 @@ int launch_track_l(const TrackArgs& a, int team, int64_t max_groups, cudaStream_
     if (per_sm < 1) per_sm = 1;
     int64_t grid = (int64_t)sm_count() * per_sm;
     if (grid > max_groups) grid = max_groups;
+    if (in && grid > track_int_ctas(max_groups)) grid = track_int_ctas(max_groups);  // the workspace's CTAs
     if (grid < 1) grid = 1;
     kern<<<(unsigned)grid, 32 * team, dsm, st>>>(a);
   };
-  if (team > 8) {  // wide teams: double and double double (the host only asks for these)
+  if (in) {
+    if constexpr (L > 1) {
+      // the converted points, then the solve's exchange buffers in their place
+      const size_t dsm = std::max(smem_points_bytes<L>(a.n), (size_t)team * RowLanes<L>::WORDS * sizeof(int32_t));
+      learn ? go(track_kernel<L, true, true>, dsm) : go(track_kernel<L, false, true>, dsm);
+    }
+  } else if (team > 8) {  // wide teams: double and double double (the host only asks for these)
     if (L == 4) return set_error(HT_EUNSUPPORTED, "track launch: teams above 8 warps need D or DD");
-    if (learn)
-      in ? go(track_kernel<L, true, L == 2, 16>) : go(track_kernel<L, true, false, 16>);
-    else
-      in ? go(track_kernel<L, false, L == 2, 16>) : go(track_kernel<L, false, false, 16>);
-  } else if (learn) {
-    in ? go(track_kernel<L, true, L != 1>) : go(track_kernel<L, true, false>);
+    learn ? go(track_kernel<L, true, false, 16>, 0) : go(track_kernel<L, false, false, 16>, 0);
   } else {
-    in ? go(track_kernel<L, false, L != 1>) : go(track_kernel<L, false, false>);
+    learn ? go(track_kernel<L, true, false>, 0) : go(track_kernel<L, false, false>, 0);
   }
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? HT_OK : cuda_fail(e, "track launch");

@@ -47,8 +47,8 @@ struct TrackArgs {
   double* xp;  // [n]     working point
   double* hx;  // [cap][n] accepted history, oldest first (cap = max_order + 1)
   double* ht;  // [cap]   their t values
-  double* A;   // [n][n+nrhs] [J | -h (| -dh/dt)], then Q
-  double* R;   // [n][n+nrhs] triangular factor, 1/r_qq on the diagonal
+  double* A;   // [n][n+nrhs] [J | -h (| -dh/dt)], then Q (int_eval: limb strings, a block per CTA)
+  double* R;   // [n][n+nrhs] triangular factor, 1/r_qq on the diagonal (int_eval: none)
   double* dx;  // [n]
   double* tx;  // [cap][n] tangents of the history points (predictor > 0)
   double* tdx; // [n]     tangent solved in the latest Newton round
@@ -89,6 +89,13 @@ struct TrackArgs {
   double rho_min, rho_max;
   double alpha_max;        // learned tangent correction clamp (0: off)
 };
+
+// CTAs of an int_eval launch over at most `groups` groups of paths, and the
+// bytes of the workspace A of each for an L-limb system in n variables.
+int64_t track_int_ctas(int64_t groups);
+size_t track_int_bytes(int L, int n, int nrhs);
+// Warps that share a group's systems evenly in an int_eval launch (at most 16).
+int track_int_team(int n);
 
 template <int L>
 int launch_start_l(int n, const int32_t* d_deg, int64_t first, int64_t count, double* x, cudaStream_t st);
