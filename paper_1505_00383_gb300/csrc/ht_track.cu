@@ -601,15 +601,25 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
   // Groups of 32 active paths are taken from a queue (one counter per
   // launch, zeroed by the compaction before it): a CTA whose groups finish
   // early takes more, instead of a fixed share of them.
+  // DD and QD on the integer pipe spread few paths thinly: a group is as many
+  // paths as give every CTA one (a multiple of a warp's systems in the
+  // least squares), since its rounds shorten with the warps it has to share the
+  // SM with.  In double a group's cost is its instruction count on the FP64
+  // pipe, whatever the lanes in use, so it always takes 32.
+  int G = 32;
+  if constexpr (FZ) {
+    G = (count + (int)gridDim.x - 1) / (int)gridDim.x;
+    G = min(32, (G + pp - 1) / pp * pp);
+  }
   __shared__ int sh_group;
   for (;;) {
     if (threadIdx.x == 0) sh_group = atomicAdd(a.queue, 1);
     __syncthreads();
     const int64_t g = sh_group;
     __syncthreads();  // every thread has read the group before the next take
-    if (g * 32 >= count) break;
-    const int64_t slot = g * 32 + lane;
-    const int64_t p = slot < count ? a.idx_in[slot] : -1;
+    if (g * G >= count) break;
+    const int64_t slot = g * G + lane;
+    const int64_t p = lane < G && slot < count ? a.idx_in[slot] : -1;
     for (int iter = 0; iter < a.iters; ++iter) {
       int8_t stt = p >= 0 ? a.status[p] : (int8_t)1;
       const bool act = stt == 0;
@@ -689,24 +699,11 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
         }
         return r_div(num, den);
       };
-      if (start) {
-        double step = fmin(h, 1.0 - t);
-        t1 = (step >= 1.0 - t) ? 1.0 : t + step;
-        if constexpr (L > 1) {
-          for (int j = warp; j < mm; j += T) {
-            const rl<L> wj = weight(j);
-#pragma unroll
-            for (int l = 0; l < L; ++l) sh_w[j][l][lane] = r_limb(wj, l);
-          }
-        }
-      }
-      // (in double a weight is a few instructions: every warp computes them,
-      // without the barrier)
-      if constexpr (L > 1) __syncthreads();
-      if (start) {
-        // tangent predictors: cubic Hermite on the last two points and their
-        // tangents, Euler on the last one; until a tangent exists, x itself
-        rl<L> ca = r_from<L>(0.0), cb = r_from<L>(0.0), cc = r_from<L>(0.0), cd = r_from<L>(0.0);
+      // tangent predictors: cubic Hermite on the last two points and their
+      // tangents (weights of x0, v0, x1, v1), Euler on the last one (weight of
+      // v1); until a tangent exists, x itself
+      rl<L> ca = r_from<L>(0.0), cb = r_from<L>(0.0), cc = r_from<L>(0.0), cd = r_from<L>(0.0);
+      auto tangent_weights = [&]() {
         if (herm) {  // x0, v0 at s0 = ht[nh-2]; x1, v1 at s1 = ht[nh-1]
           const double s0 = a.ht[(int64_t)(nh - 2) * m + p], s1 = a.ht[(int64_t)(nh - 1) * m + p];
           const rl<L> d = r_diff<L>(s1, s0), u = r_div(r_diff<L>(t1, s0), d);
@@ -718,6 +715,48 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
           cd = r_mul(r_sub(u3, u2), d);                                        // of v1
         } else if (euler) {
           cd = r_diff<L>(t1, a.ht[(int64_t)(nh - 1) * m + p]);
+        }
+      };
+      if (start) {
+        double step = fmin(h, 1.0 - t);
+        t1 = (step >= 1.0 - t) ? 1.0 : t + step;
+        if constexpr (L > 1) {
+          for (int j = warp; j < mm; j += T) {
+            const rl<L> wj = weight(j);
+#pragma unroll
+            for (int l = 0; l < L; ++l) sh_w[j][l][lane] = r_limb(wj, l);
+          }
+          // the tangent predictors' weights (a QD division and a dozen QD
+          // products in FP64) once, by the last warp
+          if (warp == T - 1 && (herm || euler)) {
+            tangent_weights();
+#pragma unroll
+            for (int l = 0; l < L; ++l) {
+              sh_w[0][l][lane] = r_limb(ca, l);
+              sh_w[1][l][lane] = r_limb(cb, l);
+              sh_w[2][l][lane] = r_limb(cc, l);
+              sh_w[3][l][lane] = r_limb(cd, l);
+            }
+          }
+        }
+      }
+      // (in double a weight is a few instructions: every warp computes them,
+      // without the barrier)
+      if constexpr (L > 1) __syncthreads();
+      if (start) {
+        if constexpr (L == 1) {
+          tangent_weights();
+        } else if (herm || euler) {
+          auto get = [&](int k) {
+            double wl[L];
+#pragma unroll
+            for (int l = 0; l < L; ++l) wl[l] = sh_w[k][l][lane];
+            return r_of<L>(wl);
+          };
+          ca = get(0);
+          cb = get(1);
+          cc = get(2);
+          cd = get(3);
         }
         rl<L> w[8];
         for (int j = 0; j < mm; ++j) {
@@ -734,22 +773,29 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
           cx<L> acc = czero<L>();
           bool fz_done = false;
           if constexpr (FZ && L == 4) {
-            // QD extrapolation on the integer pipe: the history points times
-            // their weights as limb-string products, summed exactly and
-            // rounded once (a QD complex-by-real product on the FP64 pipe is
-            // about 200 FP64 instructions)
-            if (!herm && !euler && mm > 0) {
+            // QD predictors on the integer pipe: the history points and
+            // tangents times their weights as limb-string products, summed
+            // exactly and rounded once (a QD complex-by-real product on the
+            // FP64 pipe is about 200 FP64 instructions)
+            const int nt = herm ? 4 : (euler ? 2 : mm);
+            if (nt > 0) {
               constexpr int WZ = IntW<L>::W;
               const double zero4[4] = {0.0, 0.0, 0.0, 0.0};
               mpi::fz<WZ> terms[8];
               int ones[8];
-              for (int j = 0; j < mm; ++j) {
-                const mpi::fz<WZ> wz = mpi::from_doubles<WZ, 4>(w[j].x, zero4);
-                terms[j] = mpi::mul<WZ>(fz_of<L>(ld<L>(a.hx, (int64_t)(base + j) * n + i, m, p)), wz);
+#pragma unroll 1
+              for (int j = 0; j < nt; ++j) {
+                const bool tan = (herm && (j & 1)) || (euler && j == 1);
+                const int q = herm ? nh - 2 + (j >> 1) : (euler ? nh - 1 : base + j);
+                double wl[4];
+#pragma unroll
+                for (int l = 0; l < 4; ++l) wl[l] = euler && j == 0 ? (l == 0 ? 1.0 : 0.0) : sh_w[euler ? 3 : j][l][lane];
+                const mpi::fz<WZ> wz = mpi::from_doubles<WZ, 4>(wl, zero4);
+                terms[j] = mpi::mul<WZ>(fz_of<L>(ld<L>(tan ? a.tx : a.hx, (int64_t)q * n + i, m, p)), wz);
                 ones[j] = 1;
               }
               double re[4], im[4];
-              mpi::to_doubles<WZ, 4>(mpi::sum<WZ, 8>(terms, ones, mm), re, im);
+              mpi::to_doubles<WZ, 4>(mpi::sum<WZ, 8>(terms, ones, nt), re, im);
               acc = cx_from<L>(re, im);
               fz_done = true;
             }
@@ -757,7 +803,8 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
           if (!fz_done)
             for (int j = 0; j < mm; ++j)
               acc = cadd(acc, cscale_r(ld<L>(a.hx, (int64_t)(base + j) * n + i, m, p), w[j]));
-          if (herm) {
+          if (fz_done) {
+          } else if (herm) {
             acc = cscale_r(ld<L>(a.hx, (int64_t)(nh - 2) * n + i, m, p), ca);
             acc = cadd(acc, cscale_r(ld<L>(a.tx, (int64_t)(nh - 2) * n + i, m, p), cb));
             acc = cadd(acc, cscale_r(ld<L>(a.hx, (int64_t)(nh - 1) * n + i, m, p), cc));
@@ -832,17 +879,54 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
           mpi::fixed_to_doubles<IntW<L>::WA, L>(ai, Fv[n], vim);
           const ZW fj = mpi::from_doubles<WZ, L>(vre, vim);
           const int d = __ldg(a.deg + j);
-          const ZW xj = X[j];
-          ZW xd1 = one;  // x_j^(d-1)
-          for (int e = 0; e < d - 1; ++e) xd1 = e == 0 ? xj : mpi::mul<WZ>(xd1, xj);
-          const ZW gval = mpi::sub<WZ>(mpi::mul<WZ>(xd1, xj), one);  // x_j^d - 1
-          ZW t2[2] = {mpi::mul<WZ>(gsz, gval), mpi::mul<WZ>(ttz, fj)};
-          const int e_neg[2] = {-1, -1};
-          const ZW hj = mpi::add<WZ>(t2[0], t2[1]);
-          put(n, mpi::sum<WZ, 2>(t2, e_neg, 2));
-          if (nrhs == 2) put(n + 1, mpi::sub<WZ>(mpi::mul<WZ>(gz, gval), fj));  // -dh/dt = gamma g - f
-          const int e_d[1] = {d};
-          const ZW dg = mpi::mul<WZ>(gsz, mpi::sum<WZ, 1>(&xd1, e_d, 1));  // gamma (1 - tt) d x_j^(d-1)
+          // the start system's terms and the homotopy: xd = x_j^d, xd1 =
+          // x_j^(d-1), gval = xd - 1, hj = gamma (1 - tt) gval + tt fj, dg =
+          // gamma (1 - tt) d xd1, and -dh/dt = gamma gval - fj.  One product
+          // and one sum site each: the strings' code (a product is several
+          // hundred instructions) runs once a row and would miss the
+          // instruction cache at every site.
+          enum { XD1, XD, GV, TG, TF, DG, GG, N_V };
+          mpi::fzs<WZ> v[N_V];
+          v[XD1] = one;
+#pragma unroll 1
+          for (int e = 1; e < d; ++e) v[XD1] = e == 1 ? mpi::fzs<WZ>(X[j]) : mpi::fzs<WZ>(mpi::mul<WZ>(v[XD1], X[j]));
+#pragma unroll 1
+          for (int k = 0; k < 5; ++k) {
+            // products: xd = xd1 x_j; gsz gval; tt fj; gsz (d xd1); gamma gval
+            if (k == 4 && nrhs < 2) break;
+            ZW x, y;
+            int to;
+            if (k == 0) {
+              x = v[XD1];
+              y = X[j];
+              to = XD;
+            } else if (k == 2) {
+              x = ttz;
+              y = fj;
+              to = TF;
+            } else {
+              x = k == 4 ? gz : gsz;
+              y = v[k == 3 ? DG : GV];
+              to = k == 1 ? TG : (k == 3 ? DG : GG);
+            }
+            v[to] = mpi::mul<WZ>(x, y);
+            if (k == 0) {
+              v[GV] = mpi::sub<WZ>(static_cast<ZW>(v[XD]), one);
+              const ZW x1 = v[XD1];
+              const int e_d[1] = {d};
+              v[DG] = mpi::sum<WZ, 1>(&x1, e_d, 1);
+            }
+          }
+          const ZW hj = mpi::add<WZ>(v[TG], v[TF]);
+          ZW mh = hj;  // -hj: the negated sum, rounded as itself
+          {
+            const ZW t2[2] = {v[TG], v[TF]};
+            const int e_neg[2] = {-1, -1};
+            mh = mpi::sum<WZ, 2>(t2, e_neg, 2);
+          }
+          put(n, mh);
+          if (nrhs == 2) put(n + 1, mpi::sub<WZ>(v[GG], fj));  // -dh/dt = gamma g - f
+          const ZW dg = v[DG];
           // the row is tt times the gradient, scaled in the exact fixed-point sums
           for (int i = 0; i < n; ++i) {
             row.load(i, ar, ai);

@@ -1,5 +1,6 @@
 // Host driver of the many-path tracker and the standalone entry points for its
 // stages (start solutions, least squares, compaction).
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -309,7 +310,7 @@ int ht_track_paths_ex(ht_system* s, const int32_t* start_deg, const double* gamm
   // (ht_set_eval_config 0 or 1): A is then limb strings in a block per CTA,
   // and R stays with the lanes
   const bool int_eval = L > 1 && s->d_steps && n <= 32 && (s->eval_variant == -1 || s->eval_variant == 2);
-  const size_t b_A = int_eval ? (size_t)track_int_ctas((m + 31) / 32) * track_int_bytes(L, n, nrhs)
+  const size_t b_A = int_eval ? (size_t)track_int_ctas(std::max((m + 31) / 32, std::min<int64_t>(m, sm_count()))) * track_int_bytes(L, n, nrhs)
                               : (size_t)n * (n + nrhs) * cxb,
                b_R = int_eval ? 0 : (size_t)n * (n + nrhs) * cxb;
   size_t o_xp = take(n * cxb), o_hx = take((size_t)cap * n * cxb), o_ht = take((size_t)cap * m * 8),
@@ -448,7 +449,10 @@ int ht_track_paths_ex(ht_system* s, const int32_t* start_deg, const double* gamm
   drop_graphs(s);
   while (active > 0) {
     int team = pick_team(active);
+    // CTAs a launch can use: groups of 32 paths; on the integer pipe as few
+    // paths as spread over the SMs
     int64_t groups = (active + 31) / 32;
+    if (int_eval) groups = std::max(groups, std::min<int64_t>(active, sm_count()));
     // graph for this (team, iters, rounds, workspace, outputs) configuration
     ht_system::GraphEntry* ge = nullptr;
     for (auto& g : s->graphs)
