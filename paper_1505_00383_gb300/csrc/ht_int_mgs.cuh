@@ -2,11 +2,16 @@
 // lane (device only): the corrector's solve of the DD and QD tracker and of
 // ht_mgs_solve_ex variant 2.
 //
-// A warp serves PP = min(8, 32 / rows) systems, lane (system, row).  A lane
-// holds its row's entry of the pivot column in registers and its row in local
-// memory; a dot product over the rows is one exact fixed-point sum across the
-// system's lanes (row_sum), rounded once, so every lane of the system has the
-// result.  There is no barrier: the warps are independent of each other.
+// A warp has min(8, 32 / rows) slots of `rows` lanes.  They hold the slots / C
+// systems the warp serves, each on C slots: slot c of a system has the columns
+// j = c mod C.  A lane holds its row's entry of the pivot column in registers
+// and its row of its columns in local memory; a dot product over the rows is
+// one exact fixed-point sum across the slot's lanes (row_sum), rounded once,
+// so every lane of the slot has the result.  There is no barrier: the warps
+// are independent of each other.  C = 1 does the least work (a pivot column is
+// normalised on every slot of its system); with C = slots a system takes a
+// C-th of the steps, which is faster while there are warps to spare (DD n =
+// 12, 700 paths on 152 SMs: XX).  The results do not depend on C.
 //
 // Why rows and not whole systems per lane: with a system per lane the columns
 // were dealt to the warps of a CTA, which met at a barrier per column, and
@@ -22,36 +27,41 @@ template <int L>
 struct RowLanes {
   static constexpr int W = IntW<L>::W, WA = W + 1;
   static constexpr int ND = (2 * WA + 3) / 4 * 4;  // exchanged words a lane, 16-byte multiple
-  static constexpr int PP_MAX = 8;                 // systems a warp
-  // Shared memory of one warp: the lanes' digits, then the systems' sums.
-  static constexpr int WORDS = 32 * ND + PP_MAX * 2 * WA * 2;
+  static constexpr int SLOTS_MAX = 8;              // slots a warp
+  // Shared memory of one warp: the lanes' digits, then the slots' sums.
+  static constexpr int WORDS = 32 * ND + SLOTS_MAX * 2 * WA * 2;
   using Z = mpi::fz<W>;
 
-  int rows, i, sub, base, head;  // rows a system; this lane's row, its system in the warp, that system's first lane
-  bool row;                      // the lane has a row of a live system
-  int32_t* dig;                  // shared [32][ND]
-  int64_t* sums;                 // shared [PP_MAX][2 WA]
+  int rows, i, slot, base;        // rows a system; this lane's row, its slot, that slot's first lane
+  int C, sub, cs;                 // slots a system; this lane's system in the warp, its columns are cs mod C
+  bool row;                       // the lane has a row of a live system
+  int32_t* dig;                   // shared [32][ND]
+  int64_t* sums;                  // shared [SLOTS_MAX][2 WA]
 
-  static __host__ __device__ int systems(int rows) {
-    const int pp = 32 / rows;
-    return pp > PP_MAX ? PP_MAX : pp;
+  static __host__ __device__ int slots(int rows) {
+    const int n = 32 / rows;
+    return n > SLOTS_MAX ? SLOTS_MAX : n;
   }
-  __device__ __forceinline__ RowLanes(int rows_, int32_t* xch) : rows(rows_) {
+  // row is false for lanes past the last whole system; the caller clears it
+  // for systems it does not have
+  __device__ __forceinline__ RowLanes(int rows_, int C_, int32_t* xch) : rows(rows_), C(C_) {
     const int lane = threadIdx.x & 31;
-    sub = lane / rows;
-    i = lane - sub * rows;
-    base = sub * rows;
-    head = mpi::bitlen32((uint32_t)rows) > 1 ? mpi::bitlen32((uint32_t)rows) : 1;
-    row = sub < systems(rows);
+    slot = lane / rows;
+    i = lane - slot * rows;
+    base = slot * rows;
+    sub = slot / C;
+    cs = slot - sub * C;
+    row = sub < slots(rows) / C;
     dig = xch;
     sums = reinterpret_cast<int64_t*>(xch + 32 * ND);
   }
 
-  // sum of z over the system's rows: the frame, digits and rounding of mpi::sum
-  __device__ __forceinline__ Z row_sum(const Z& z) const {
+  // sum over the slot's rows of z, or of -z on the lanes with neg, for the
+  // lanes with part (`terms` of them): the frame, digits and rounding of mpi::sum
+  __device__ __forceinline__ Z row_sum(const Z& z, bool part, bool neg, int terms) const {
     const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const int b0 = row ? mpi::bound_exp<W>(z) : -30000;
+    const int lane = threadIdx.x & 31, hb = mpi::bitlen32((uint32_t)terms), head = hb > 1 ? hb : 1;
+    const int b0 = part ? mpi::bound_exp<W>(z) : -30000;
     int E = b0, fm = b0 > -30000 ? z.f : -30000;
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) {
@@ -72,20 +82,24 @@ struct RowLanes {
       mpi::shifted_digits<W, WA>(z.r, sp / mpi::RB, sp % mpi::RB, d);
       mpi::shifted_digits<W, WA>(z.i, sp / mpi::RB, sp % mpi::RB, d + WA);
     }
+    if (neg) {
+#pragma unroll
+      for (int k = 0; k < 2 * WA; ++k) d[k] = -d[k];
+    }
     int4* q = reinterpret_cast<int4*>(dig + lane * ND);
 #pragma unroll
     for (int k = 0; k < ND / 4; ++k) q[k] = make_int4(d[4 * k], d[4 * k + 1], d[4 * k + 2], d[4 * k + 3]);
     __syncwarp();
     if (row)
-      for (int w = i; w < 2 * WA; w += rows) {  // the system's lanes deal the words
+      for (int w = i; w < 2 * WA; w += rows) {  // the slot's lanes deal the words
         int64_t s = 0;
 #pragma unroll 4
         for (int k = 0; k < rows; ++k) s += dig[(base + k) * ND + w];
-        sums[sub * 2 * WA + w] = s;
+        sums[slot * 2 * WA + w] = s;
       }
     __syncwarp();
     int64_t c[2 * WA];
-    const int s0 = row ? sub * 2 * WA : 0;
+    const int s0 = row ? slot * 2 * WA : 0;
 #pragma unroll
     for (int k = 0; k < 2 * WA; ++k) c[k] = sums[s0 + k];
     mpi::carry<WA>(c);
@@ -105,80 +119,94 @@ struct RowLanes {
     return s;
   }
 
+  // z of another lane
+  static __device__ __forceinline__ Z shfl(const Z& z, int src) {
+    Z t;
+    t.f = __shfl_sync(0xffffffffu, z.f, src);
+#pragma unroll
+    for (int k = 0; k < W; ++k) {
+      t.r[k] = __shfl_sync(0xffffffffu, z.r[k], src);
+      t.i[k] = __shfl_sync(0xffffffffu, z.i[k], src);
+    }
+    return t;
+  }
+
   // Least squares of [A | b_0 .. b_{nrhs-1}], cols <= rows <= 32, cols + nrhs
-  // <= MAXC.  load(j) gives this lane's entry of column j, put_q(j, z) takes
-  // its entry of the orthogonal factor (j < cols) or of a reduced right-hand
-  // side, put_r(j, z) the entries j >= i of its row of R (1/r_ii at j = i;
-  // lanes i < cols), put_x(k, z) coordinate i of solution k.  All 32 lanes of
-  // the warp call it.
-  template <int MAXC, class Load, class PutQ, class PutR, class PutX>
-  __device__ __forceinline__ void solve(int cols, int nrhs, Load load, PutQ put_q, PutR put_r, PutX put_x) const {
+  // <= MAXC.  load(j) gives this lane's row's entry of column j, once, for
+  // the lane's columns and column 0; put_q(j, z) takes it in the orthogonal
+  // factor (j < cols) or in a reduced right-hand side; put_r(j, z) the
+  // entries j >= i of row i of R (1/r_ii at j = i; rows i < cols), which
+  // get_r(i, j) returns to any lane of the system; put_x(k, z) coordinate i
+  // of solution k.
+  // Each output is put by one slot of the system.  All 32 lanes of the warp
+  // call it.
+  template <int MAXC, class Load, class PutQ, class PutR, class GetR, class PutX>
+  __device__ __forceinline__ void solve(int cols, int nrhs, Load load, PutQ put_q, PutR put_r, GetR get_r,
+                                        PutX put_x) const {
     const int Wc = cols + nrhs;
-    mpi::fzs<W> a[MAXC], r[MAXC];  // the lane's row of A, and of R
+    mpi::fzs<W> a[MAXC];  // the lane's row of A (its columns)
     Z Q, nxt;
     Q.f = nxt.f = 0;
 #pragma unroll
     for (int k = 0; k < W; ++k) Q.r[k] = Q.i[k] = nxt.r[k] = nxt.i[k] = 0;
     if (row) nxt = load(0);
-    // phase q projects the columns j > q on column q, then normalises column
-    // q + 1 (j = Wc; the first phase, q = -1, only normalises column 0)
+    // phase q projects the columns j > q on column q, C at a time, then
+    // normalises column q + 1 (step Wc; the first phase, q = -1, only
+    // normalises column 0)
     for (int q = -1; q < cols; ++q)
-      for (int j = q < 0 ? Wc : q + 1; j <= Wc; ++j) {
-        const bool pivot = j == Wc;
+      for (int jb = q < 0 ? Wc : (q + 1) / C * C;; jb += C) {
+        const bool pivot = jb >= Wc;
         if (pivot && q + 1 == cols) break;
+        const int j = pivot ? q + 1 : jb + cs;
+        const bool mine = row && j > q && j < Wc;
         Z u, v;
         if (pivot) {
+          if (C > 1 && q >= 0) nxt = shfl(nxt, min(base + ((q + 1) % C - cs) * rows + i, 31));
           u = v = nxt;
         } else {
-          u = Q;
-          v = Q;
-          if (row) v = q == 0 ? load(j) : static_cast<Z>(a[j]);
+          u = v = Q;
+          if (mine) v = q == 0 ? load(j) : static_cast<Z>(a[j]);
         }
-        Z s = row_sum(mpi::mul<W>(mpi::conj<W>(u), v));
+        Z s = row_sum(mpi::mul<W>(mpi::conj<W>(u), v), row, false, rows);
         if (pivot) s = mpi::inv_sqrt<W>(s, mpi::inv_sqrt_steps<W>());
         const Z t = mpi::mul<W>(s, u);
-        const int jr = pivot ? q + 1 : j;
-        if (i == (pivot ? q + 1 : q)) {
-          r[jr] = s;
-          if (row) put_r(jr, s);
-        }
+        if (mine && i == (pivot ? j : q) && (!pivot || cs == 0)) put_r(j, s);
         if (pivot) {
           Q = t;
-          if (row) put_q(jr, t);
-        } else {
-          v = mpi::sub<W>(v, t);
+          if (row && cs == 0) put_q(j, t);
+          break;
+        }
+        v = mpi::sub<W>(v, t);
+        if (mine) {
           a[j] = v;
           if (j == q + 1) nxt = v;
-          if (row && q + 1 == cols) put_q(j, v);
+          if (q + 1 == cols) put_q(j, v);
         }
       }
-    // back substitution: lane j forms x_j from its right-hand side and the
-    // products it has collected (one exact sum), then every lane above
-    // collects its product with x_j
-    for (int k = 0; k < nrhs; ++k)
-      for (int j = cols - 1; j >= 0; --j) {
-        Z x;
-        x.f = 0;
+    __syncwarp();  // R's entries are visible to the system's slots
+    // Back substitution, the right-hand sides dealt to the system's slots: lane
+    // l keeps x_l once it is known, and x_j is the sum over the lanes of
+    // y_j (lane j) and -r_jl x_l (lanes l > j), times 1/r_jj.  (One lane adding
+    // the n - j products by itself took 25,000 clocks a coordinate in QD.)
+    for (int k0 = 0; k0 < nrhs; k0 += C) {
+      const int k = k0 + cs;
+      const bool mine = row && k < nrhs;
+      Z x;
+      x.f = 0;
 #pragma unroll
-        for (int l = 0; l < W; ++l) x.r[l] = x.i[l] = 0;
-        if (i == j && row) {
-          Z S[MAXC];
-          int cnt = 0;
-          S[cnt++] = r[cols + k];
-          for (int l = j + 1; l < cols; ++l) S[cnt++] = a[l];
-          x = mpi::mul<W>(mpi::first_minus_rest<W, MAXC>(S, cnt), static_cast<Z>(r[j]));
+      for (int l = 0; l < W; ++l) x.r[l] = x.i[l] = 0;
+      for (int j = cols - 1; j >= 0; --j) {
+        const bool part = mine && i >= j && i < cols;
+        Z z = x;
+        if (part) z = get_r(j, i == j ? cols + k : i);
+        if (part && i > j) z = mpi::mul<W>(z, x);
+        z = row_sum(z, part, i > j, cols - j);
+        if (part && i == j) {
+          x = mpi::mul<W>(z, get_r(j, j));
           put_x(k, x);
         }
-        if (j == 0) break;
-        const int src = min(base + j, 31);
-        x.f = __shfl_sync(0xffffffffu, x.f, src);
-#pragma unroll
-        for (int l = 0; l < W; ++l) {
-          x.r[l] = __shfl_sync(0xffffffffu, x.r[l], src);
-          x.i[l] = __shfl_sync(0xffffffffu, x.i[l], src);
-        }
-        if (i < j && row) a[j] = mpi::mul<W>(static_cast<Z>(r[j]), x);
       }
+    }
   }
 };
 

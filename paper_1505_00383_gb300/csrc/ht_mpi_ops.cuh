@@ -311,27 +311,17 @@ HT_HD rz<W> sub(const rz<W>& a, const rz<W>& b) {
   return z;
 }
 
-// 1 / sqrt(v) for a positive real v (im = 0): Newton's iteration
-// y <- y (3 - v y^2) / 2 from the double seed; each step doubles the bits.
+// The real part as a real string, and back (im zero).
 template <int W>
-HT_HD fz<W> inv_sqrt(const fz<W>& v, int steps) {
-  const double vd = real_to_double<W>(v);
-  const fz<W> seed = from_real<W>(1.0 / std::sqrt(vd)), three = from_real<W>(3.0);
-  rz<W> x, y, c3;
-  x.f = v.f;
-  y.f = seed.f;
-  c3.f = three.f;
+HT_HD rz<W> real_of(const fz<W>& z) {
+  rz<W> y;
+  y.f = z.f;
 #pragma unroll
-  for (int k = 0; k < W; ++k) {
-    x.r[k] = v.r[k];
-    y.r[k] = seed.r[k];
-    c3.r[k] = three.r[k];
-  }
-#pragma unroll 1
-  for (int it = 0; it < steps; ++it) {
-    y = mul<W>(y, sub<W>(c3, mul<W>(x, mul<W>(y, y))));
-    y.f -= 1;  // halve
-  }
+  for (int k = 0; k < W; ++k) y.r[k] = z.r[k];
+  return y;
+}
+template <int W>
+HT_HD fz<W> complex_of(const rz<W>& y) {
   fz<W> z;
   z.f = y.f;
 #pragma unroll
@@ -340,6 +330,46 @@ HT_HD fz<W> inv_sqrt(const fz<W>& v, int steps) {
     z.i[k] = 0;
   }
   return z;
+}
+
+// 1 / sqrt(v) for a positive real v (im = 0): Newton's iteration
+// y <- y (3 - v y^2) / 2 from the double seed; each step doubles the bits.
+template <int W>
+HT_HD fz<W> inv_sqrt(const fz<W>& v, int steps) {
+  const double vd = real_to_double<W>(v);
+  rz<W> y = real_of<W>(from_real<W>(1.0 / std::sqrt(vd)));
+  const rz<W> x = real_of<W>(v), c3 = real_of<W>(from_real<W>(3.0));
+#pragma unroll 1
+  for (int it = 0; it < steps; ++it) {
+    y = mul<W>(y, sub<W>(c3, mul<W>(x, mul<W>(y, y))));
+    y.f -= 1;  // halve
+  }
+  return complex_of<W>(y);
+}
+
+// a / b for reals, b nonzero: Newton's iteration y <- y (2 - b y) for 1 / b
+// from the double seed (each step doubles the bits), then a y.
+template <int W>
+HT_HD rz<W> quotient(const rz<W>& a, const rz<W>& b, double b_lead) {
+  rz<W> y = real_of<W>(from_real<W>(1.0 / b_lead));
+  const rz<W> two = real_of<W>(from_real<W>(2.0));
+#pragma unroll 1
+  for (int it = 0; it < 3; ++it) y = mul<W>(y, sub<W>(two, mul<W>(b, y)));
+  return mul<W>(a, y);
+}
+// Weights of cubic Hermite interpolation at u in [0, 1] of an interval of
+// length d: of the values and slopes at 0 and at 1, w[0..3] = 2 u^3 - 3 u^2 +
+// 1, (u^3 - 2 u^2 + u) d, 3 u^2 - 2 u^3, (u^3 - u^2) d.
+template <int W>
+HT_HD void hermite_weights(const rz<W>& u, const rz<W>& d, rz<W>* w) {
+  const rz<W> u2 = mul<W>(u, u), u3 = mul<W>(u2, u);
+  const fz<W> t[4] = {complex_of<W>(u3), complex_of<W>(u2), complex_of<W>(u), from_real<W>(1.0)};
+  const int e[4][4] = {{2, -3, 0, 1}, {1, -2, 1, 0}, {-2, 3, 0, 0}, {1, -1, 0, 0}};
+#pragma unroll 1
+  for (int k = 0; k < 4; ++k) {
+    w[k] = real_of<W>(sum<W, 4>(t, e[k], 4));
+    if (k & 1) w[k] = mul<W>(w[k], d);
+  }
 }
 
 // ------------------------------------------------------------ least squares

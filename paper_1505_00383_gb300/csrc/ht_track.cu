@@ -475,11 +475,11 @@ __global__ void __launch_bounds__(32) mgs_kernel(double* A, double* R, double* x
 constexpr int kMgsWarps = 4;
 template <int L>
 __global__ void __launch_bounds__(32 * kMgsWarps) mgs_rows_kernel(double* A, double* R, double* x, int rows, int cols,
-                                                               int64_t n_sys) {
+                                                               int64_t n_sys, int C) {
   using Z = mpi::fz<IntW<L>::W>;
   __shared__ __align__(16) int32_t xch[kMgsWarps][RowLanes<L>::WORDS];
-  const int warp = threadIdx.x >> 5, pp = RowLanes<L>::systems(rows), Wc = cols + 1;
-  RowLanes<L> rl(rows, xch[warp]);
+  const int warp = threadIdx.x >> 5, pp = RowLanes<L>::slots(rows) / C, Wc = cols + 1;
+  RowLanes<L> rl(rows, C, xch[warp]);
   const int64_t n_chunks = (n_sys + pp - 1) / pp;
   for (int64_t c = (int64_t)blockIdx.x * kMgsWarps + warp; c < n_chunks; c += (int64_t)gridDim.x * kMgsWarps) {
     const int64_t p = c * pp + rl.sub;
@@ -489,6 +489,7 @@ __global__ void __launch_bounds__(32 * kMgsWarps) mgs_rows_kernel(double* A, dou
         cols, 1, [&](int j) { return ldz<L>(A, (int64_t)i * Wc + j, n_sys, p); },
         [&](int j, const Z& z) { stz<L>(A, (int64_t)i * Wc + j, n_sys, p, z); },
         [&](int j, const Z& z) { stz<L>(R, (int64_t)i * Wc + j, n_sys, p, z); },
+        [&](int r, int j) { return ldz<L>(R, (int64_t)r * Wc + j, n_sys, p); },
         [&](int, const Z& z) { stz<L>(x, i, n_sys, p, z); });
   }
 }
@@ -580,12 +581,12 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
   // DD and QD with integer evaluation keep A as limb strings from the
   // evaluation through the least squares: no conversions
   constexpr bool FZ = INT && L >= 2;
-  // (one row per lane: entry j of the rows of a warp's systems is NQ 128-bit
-  // words a lane, [chunk][j][NQ][32]; the CTA's own workspace, which its
-  // groups reuse, stays in L2)
+  // (a block per CTA, which its groups reuse, so that it stays in L2: path l
+  // of the group, entry j of a row, NQ 128-bit words: [32][W][NQ][n], row
+  // fastest, as the lanes of the solve read it)
   constexpr int NQ = mpi::fzs<IntW<L>::W>::NW / 4;
-  const int pp = RowLanes<L>::systems(n), chunks = (32 + pp - 1) / pp;  // systems a warp, warps' worth a group
-  int4* const Acta = reinterpret_cast<int4*>(a.A) + (int64_t)blockIdx.x * chunks * W * NQ * 32;
+  const int slots = RowLanes<L>::slots(n);  // of a warp in the solve
+  int4* const Acta = reinterpret_cast<int4*>(a.A) + (int64_t)blockIdx.x * 32 * W * NQ * n;
   PolyView v;
   v.mon_off = a.mon_off;
   v.pairs = a.pairs;
@@ -602,14 +603,12 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
   // launch, zeroed by the compaction before it): a CTA whose groups finish
   // early takes more, instead of a fixed share of them.
   // DD and QD on the integer pipe spread few paths thinly: a group is as many
-  // paths as give every CTA one (a multiple of a warp's systems in the
-  // least squares), since its rounds shorten with the warps it has to share the
-  // SM with.  In double a group's cost is its instruction count on the FP64
+  // paths as give every CTA one, since its rounds shorten with the work the
+  // SM shares.  In double a group's cost is its instruction count on the FP64
   // pipe, whatever the lanes in use, so it always takes 32.
   int G = 32;
   if constexpr (FZ) {
     G = (count + (int)gridDim.x - 1) / (int)gridDim.x;
-    G = min(32, (G + pp - 1) / pp * pp);
   }
   __shared__ int sh_group;
   for (;;) {
@@ -726,9 +725,33 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
 #pragma unroll
             for (int l = 0; l < L; ++l) sh_w[j][l][lane] = r_limb(wj, l);
           }
-          // the tangent predictors' weights (a QD division and a dozen QD
-          // products in FP64) once, by the last warp
-          if (warp == T - 1 && (herm || euler)) {
+          // the tangent predictors' weights once, by the last warp; in QD on
+          // limb strings (a division and a dozen products: 250,000 clocks of
+          // the FP64 pipe's latency)
+          if (FZ && L == 4 && warp == T - 1 && herm) {
+            if constexpr (L == 4) {
+              constexpr int WZ = IntW<L>::W;
+              const double s0 = a.ht[(int64_t)(nh - 2) * m + p], s1 = a.ht[(int64_t)(nh - 1) * m + p];
+              const double zero4[4] = {0.0, 0.0, 0.0, 0.0};
+              auto diff = [&](double x, double y) {
+                const rl<L> d = r_diff<L>(x, y);
+                double wl[4];
+#pragma unroll
+                for (int l = 0; l < 4; ++l) wl[l] = r_limb(d, l);
+                return mpi::real_of<WZ>(mpi::from_doubles<WZ, 4>(wl, zero4));
+              };
+              const mpi::rz<WZ> d = diff(s1, s0);
+              mpi::rz<WZ> w4[4];
+              mpi::hermite_weights<WZ>(mpi::quotient<WZ>(diff(t1, s0), d, s1 - s0), d, w4);
+#pragma unroll 1
+              for (int k = 0; k < 4; ++k) {
+                double wl[4];
+                mpi::fixed_to_doubles<WZ, 4>(w4[k].r, w4[k].f, wl);
+#pragma unroll
+                for (int l = 0; l < 4; ++l) sh_w[k][l][lane] = wl[l];
+              }
+            }
+          } else if (warp == T - 1 && (herm || euler)) {
             tangent_weights();
 #pragma unroll
             for (int l = 0; l < L; ++l) {
@@ -859,16 +882,27 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
         const SmemLog lg{lgs_int, lane};
         const IntPoly ip{a.mon_off, a.pairs, a.step_off, a.sweep, a.clg};
         const ZW gz = fz_of<L>(gamma);
-        const ZW gsz = fz_of<L>(cscale_r(gamma, r_diff<L>(1.0, tt)));  // gamma (1 - tt)
+        ZW gsz;  // gamma (1 - tt); in QD, where 53 x 106 bits fit, as a limb-string product: the same value
+        if constexpr (L == 4) {
+          const rl<L> omt = r_diff<L>(1.0, tt);
+          double wl[L], zero[L];
+#pragma unroll
+          for (int l = 0; l < L; ++l) {
+            wl[l] = r_limb(omt, l);
+            zero[l] = 0.0;
+          }
+          gsz = mpi::mul<WZ>(gz, mpi::from_doubles<WZ, L>(wl, zero));
+        } else {
+          gsz = fz_of<L>(cscale_r(gamma, r_diff<L>(1.0, tt)));
+        }
         const ZW ttz = mpi::from_real<WZ>(tt), one = mpi::from_real<WZ>(1.0);
-        const int ch = lane / pp, sl = (lane - ch * pp) * n;  // this path's chunk and its first lane there
         for (int j = warp; j < n; j += T) {
-          int4* const out = Acta + (int64_t)ch * W * NQ * 32 + sl + j;  // this row's lane of the solve
+          int4* const out = Acta + (int64_t)lane * W * NQ * n + j;  // row j of this path
           auto put = [&](int c, const ZW& z) {
             const mpi::fzs<WZ> q(z);
 #pragma unroll
             for (int k = 0; k < NQ; ++k)
-              out[(c * NQ + k) * 32] = make_int4(q.w[4 * k], q.w[4 * k + 1], q.w[4 * k + 2], q.w[4 * k + 3]);
+              out[(c * NQ + k) * n] = make_int4(q.w[4 * k], q.w[4 * k + 1], q.w[4 * k + 2], q.w[4 * k + 3]);
           };
           int_row_run<L>(ip, static_cast<const Z*>(a.cfz), __ldg(a.poly_off + j), __ldg(a.poly_off + j + 1), X, lg, n, row,
                          Fv, P);
@@ -972,29 +1006,38 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
       // longer reads
       if constexpr (FZ) {
         const unsigned live = __ballot_sync(0xffffffffu, act);
-        RowLanes<L> rl(n, xs_int + warp * RowLanes<L>::WORDS);
+        // columns of a system on C slots while that leaves every warp at most
+        // one system's worth
+        const int C = G <= T ? slots : 1, per = slots / C, chunks = (G + per - 1) / per;
+        RowLanes<L> rl(n, C, xs_int + warp * RowLanes<L>::WORDS);
         for (int c = warp; c < chunks; c += T) {
-          const int pl = c * pp + rl.sub;  // the system's path in the group
-          if (((live >> (c * pp)) & (pp >= 32 ? ~0u : (1u << pp) - 1u)) == 0) continue;
+          const int pl = c * per + rl.sub;  // the system's path in the group
+          if (((live >> (c * per)) & ((1u << per) - 1u)) == 0) continue;
           const int64_t ps = __shfl_sync(0xffffffffu, (int)p, min(pl, 31));
-          rl.row = rl.sub < pp && pl < 32 && ((live >> pl) & 1u);
-          const int4* in = Acta + (int64_t)c * W * NQ * 32 + lane;
-          rl.template solve<kIntMaxTrack + 2>(
-              n, nrhs,
-              [&](int j) {
-                mpi::fzs<IntW<L>::W> q;
+          rl.row = rl.sub < per && pl < 32 && ((live >> pl) & 1u);
+          int4* const blk = Acta + (int64_t)min(pl, 31) * W * NQ * n;
+          auto get = [&](int r, int j) {
+            mpi::fzs<IntW<L>::W> q;
 #pragma unroll
-                for (int k = 0; k < NQ; ++k) {
-                  const int4 w = in[(j * NQ + k) * 32];
-                  q.w[4 * k] = w.x;
-                  q.w[4 * k + 1] = w.y;
-                  q.w[4 * k + 2] = w.z;
-                  q.w[4 * k + 3] = w.w;
-                }
-                return static_cast<Z>(q);
+            for (int k = 0; k < NQ; ++k) {
+              const int4 w = blk[(j * NQ + k) * n + r];
+              q.w[4 * k] = w.x;
+              q.w[4 * k + 1] = w.y;
+              q.w[4 * k + 2] = w.z;
+              q.w[4 * k + 3] = w.w;
+            }
+            return static_cast<Z>(q);
+          };
+          // R's rows take the places of A's, which are read once
+          rl.template solve<kIntMaxTrack + 2>(
+              n, nrhs, [&](int j) { return get(rl.i, j); }, [](int, const Z&) {},
+              [&](int j, const Z& z) {
+                const mpi::fzs<IntW<L>::W> q(z);
+#pragma unroll
+                for (int k = 0; k < NQ; ++k)
+                  blk[(j * NQ + k) * n + rl.i] = make_int4(q.w[4 * k], q.w[4 * k + 1], q.w[4 * k + 2], q.w[4 * k + 3]);
               },
-              [](int, const Z&) {}, [](int, const Z&) {},
-              [&](int k, const Z& z) { stz<L>(k == 0 ? a.dx : a.tdx, rl.i, m, ps, z); });
+              get, [&](int k, const Z& z) { stz<L>(k == 0 ? a.dx : a.tdx, rl.i, m, ps, z); });
         }
         __syncthreads();
       }
@@ -1221,9 +1264,9 @@ template <int L>
 int launch_mgs_l(double* A, double* R, double* x, int rows, int cols, int64_t n_sys, int variant, cudaStream_t st) {
   if (n_sys == 0) return HT_OK;
   if (variant == 2 && L > 1 && rows <= 32) {
-    const int64_t chunks = (n_sys + RowLanes<L>::systems(rows) - 1) / RowLanes<L>::systems(rows);
+    const int64_t chunks = (n_sys + RowLanes<L>::slots(rows) - 1) / RowLanes<L>::slots(rows);
     const int64_t grid = std::min<int64_t>((chunks + kMgsWarps - 1) / kMgsWarps, (int64_t)sm_count() * 16);
-    mgs_rows_kernel<L><<<(unsigned)grid, 32 * kMgsWarps, 0, st>>>(A, R, x, rows, cols, n_sys);
+    mgs_rows_kernel<L><<<(unsigned)grid, 32 * kMgsWarps, 0, st>>>(A, R, x, rows, cols, n_sys, 1);
   } else if (variant == 2 && L > 1)
     mgs_kernel<L, L != 1><<<(unsigned)((n_sys + 31) / 32), 32, 0, st>>>(A, R, x, rows, cols, n_sys);
   else
@@ -1235,12 +1278,7 @@ int launch_mgs_l(double* A, double* R, double* x, int rows, int cols, int64_t n_
 #if HT_LIMBS == 1
 int64_t track_int_ctas(int64_t groups) { return std::max<int64_t>(1, std::min<int64_t>(groups, 4 * (int64_t)sm_count())); }
 size_t track_int_bytes(int L, int n, int nrhs) {
-  const int pp = RowLanes<2>::systems(n), chunks = (32 + pp - 1) / pp;
-  return (size_t)chunks * (n + nrhs) * 32 * (L == 4 ? sizeof(mpi::fzs<8>) : sizeof(mpi::fzs<5>));
-}
-int track_int_team(int n) {
-  const int pp = RowLanes<2>::systems(n), chunks = (32 + pp - 1) / pp;
-  return (chunks + (chunks + 15) / 16 - 1) / ((chunks + 15) / 16);
+  return (size_t)32 * n * (n + nrhs) * (L == 4 ? sizeof(mpi::fzs<8>) : sizeof(mpi::fzs<5>));
 }
 __global__ void __launch_bounds__(256) mlp_image_kernel(MlpSmem* img, const __nv_bfloat16* __restrict__ wbf,
                                                         const float* __restrict__ master) {

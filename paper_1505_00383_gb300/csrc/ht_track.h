@@ -94,8 +94,6 @@ struct TrackArgs {
 // bytes of the workspace A of each for an L-limb system in n variables.
 int64_t track_int_ctas(int64_t groups);
 size_t track_int_bytes(int L, int n, int nrhs);
-// Warps that share a group's systems evenly in an int_eval launch (at most 16).
-int track_int_team(int n);
 
 template <int L>
 int launch_start_l(int n, const int32_t* d_deg, int64_t first, int64_t count, double* x, cudaStream_t st);

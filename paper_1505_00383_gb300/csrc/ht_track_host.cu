@@ -435,7 +435,7 @@ int ht_track_paths_ex(ht_system* s, const int32_t* start_deg, const double* gamm
     if (s->track_team > 0 && s->track_team <= 16) {
       t = s->track_team;
     } else if (int_eval) {
-      return track_int_team(n);
+      return 16;  // the rows of the systems, and in small groups their columns, spread over all
     } else {
       while (t < 8 && 2 * t <= n) t *= 2;
     }
