@@ -34,12 +34,10 @@ struct MlpFwdSmem {
   MlpWarpSmem w[kMlpThreads / 32];
 };
 
-// y = MLP(x) for B samples; if z1 is given, also the pre-activations of both
-// hidden layers (z1, z2 sized for B rounded up to a multiple of 32 rows).
+// y = MLP(x) for B samples.
 __global__ void __launch_bounds__(kMlpThreads) mlp_forward_kernel(const __nv_bfloat16* __restrict__ wbf,
                                                                   const float* __restrict__ master, int64_t B,
-                                                                  const float* __restrict__ x, float* __restrict__ y,
-                                                                  float* __restrict__ z1, float* __restrict__ z2) {
+                                                                  const float* __restrict__ x, float* __restrict__ y) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   MlpFwdSmem& sm = *reinterpret_cast<MlpFwdSmem*>(smem_raw);
   mlp_load(sm.net, wbf, master);
@@ -50,10 +48,7 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_forward_kernel(const __nv_bfl
     const int64_t s = w0 * 32 + lane;
     float xs[MLP_IN], ys[MLP_OUT];
     for (int i = 0; i < MLP_IN; ++i) xs[i] = s < B ? x[s * MLP_IN + i] : 0.0f;
-    if (z1)
-      mlp_forward_warp(sm.net, sm.w[wid], xs, ys, z1 + w0 * 32 * MLP_HID, z2 + w0 * 32 * MLP_HID);
-    else
-      mlp_forward_warp(sm.net, sm.w[wid], xs, ys);
+    mlp_forward_warp(sm.net, sm.w[wid], xs, ys);
     if (s < B) {
       y[s * MLP_OUT + 0] = ys[0];
       y[s * MLP_OUT + 1] = ys[1];
@@ -66,8 +61,13 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_forward_kernel(const __nv_bfl
 // operands in BF16, each laid out for the fragment it feeds: row-major [m][k]
 // for A and [n][k] for B (mma.m16n8k16 .row.col), rows padded to 72 elements
 // so the 8 row groups of a fragment load fall in distinct banks.
-constexpr int kBwdChunk = 64, kBwdThreads = 128, LDC = kBwdChunk + 8, LDH = MLP_HID + 8;
+constexpr int kBwdChunk = 64, kBwdThreads = 256, LDC = kBwdChunk + 8, LDH = MLP_HID + 8;
+constexpr int LDZ = MLP_HID + 1;  // FP32 rows: a thread per sample walks its row without bank conflicts
 struct MlpBwdSmem {
+  MlpSmem net;                        // for the chunk's forward pass
+  MlpWarpSmem w[kBwdChunk / 32];
+  float z1[kBwdChunk * LDZ];          // pre-activations [s][i]
+  float y[kBwdChunk * MLP_OUT];
   __nv_bfloat16 W2T[MLP_HID * LDH];   // [i][o] = W2[o][i]: B operand of dh1 = dz2 W2
   __nv_bfloat16 dz2r[kBwdChunk * LDH];  // [s][o]: A operand of dh1
   __nv_bfloat16 dz2T[MLP_HID * LDC];  // [o][s]: A operand of dW2
@@ -77,10 +77,10 @@ struct MlpBwdSmem {
   __nv_bfloat16 h2T[MLP_HID * LDC];   // [i][s] = bf16(relu(z2)): B operand of dW3
   __nv_bfloat16 xT[MLP_IN * LDC];     // [i][s] = bf16(x): B operand of dW1
   float W3[MLP_OUT * MLP_HID];
-  float dz1f[kBwdChunk * MLP_HID];    // FP32 activation gradients for the bias sums
-  float dz2f[kBwdChunk * MLP_HID];
+  float dz1f[kBwdChunk * LDZ];        // FP32 activation gradients for the bias sums
+  float dz2f[kBwdChunk * LDZ];
   float dyf[kBwdChunk * MLP_OUT];
-  float z2[kBwdChunk * MLP_HID];
+  float z2[kBwdChunk * LDZ];
   unsigned long long mask1[kBwdChunk];  // bit i: z1[s][i] > 0
   float err2[kBwdChunk];
 };
@@ -101,21 +101,33 @@ __device__ __forceinline__ void mma_tile(float* c, const __nv_bfloat16* A, int l
   }
 }
 
-// Chunk c of the batch: dL/dy = 2 (y - target) / B, the activation gradients
-// through both ReLU layers, and the chunk's partial gradient of every
-// parameter (part[c][MLP_NPARAM]) and partial loss (loss_part[c]).  The
-// activations are recomputed from the stored pre-activations exactly as the
-// forward pass rounded them.
+// Chunk c of the batch: the forward pass (32 samples a warp, pre-activations
+// kept in shared memory), dL/dy = 2 (y - target) / B, the activation
+// gradients through both ReLU layers, and the chunk's partial gradient of
+// every parameter (part[c][MLP_NPARAM]) and partial loss (loss_part[c]).  The
+// activations are recomputed from the pre-activations exactly as the forward
+// pass rounded them.  (A batch of 4,096 is 64 CTAs of a few microseconds:
+// launches bound it, so the forward pass is not a kernel of its own.)
 __global__ void __launch_bounds__(kBwdThreads) mlp_backward_kernel(
-    const __nv_bfloat16* __restrict__ wbf, int64_t B, const float* __restrict__ x, const float* __restrict__ y,
-    const float* __restrict__ target, const float* __restrict__ z1, const float* __restrict__ z2,
-    float* __restrict__ part, float* __restrict__ loss_part) {
+    const __nv_bfloat16* __restrict__ wbf, const float* __restrict__ master, int64_t B, const float* __restrict__ x,
+    const float* __restrict__ target, float* __restrict__ part, float* __restrict__ loss_part) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   MlpBwdSmem& sm = *reinterpret_cast<MlpBwdSmem*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
   const int64_t s0 = (int64_t)blockIdx.x * kBwdChunk;
   const int ns = (int)min((int64_t)kBwdChunk, B - s0);
   const __nv_bfloat16 zero = __float2bfloat16(0.0f);
+  // ---- the chunk's forward pass
+  mlp_load(sm.net, wbf, master);
+  __syncthreads();
+  if (warp < kBwdChunk / 32) {
+    const int sl = warp * 32 + lane;
+    float xs[MLP_IN], ys[MLP_OUT];
+    for (int i = 0; i < MLP_IN; ++i) xs[i] = sl < ns ? x[(s0 + sl) * MLP_IN + i] : 0.0f;
+    mlp_forward_warp(sm.net, sm.w[warp], xs, ys, sm.z1 + warp * 32 * LDZ, sm.z2 + warp * 32 * LDZ, LDZ);
+    for (int o = 0; o < MLP_OUT; ++o) sm.y[sl * MLP_OUT + o] = ys[o];
+  }
+  __syncthreads();
   // ---- stage weights and the chunk's activations
   for (int e = tid; e < MLP_HID * MLP_HID; e += kBwdThreads) {
     const int o = e / MLP_HID, i = e % MLP_HID;
@@ -123,13 +135,13 @@ __global__ void __launch_bounds__(kBwdThreads) mlp_backward_kernel(
   }
   for (int e = tid; e < MLP_OUT * MLP_HID; e += kBwdThreads) sm.W3[e] = __bfloat162float(wbf[OFF_W3 + e]);
   for (int e = tid; e < kBwdChunk * MLP_HID; e += kBwdThreads) {
-    const int sl = e / MLP_HID, i = e % MLP_HID;
+    const int sl = e % kBwdChunk, i = e / kBwdChunk;
     const bool live = sl < ns;
-    const float a = live ? z1[(s0 + sl) * MLP_HID + i] : 0.0f;
-    const float b = live ? z2[(s0 + sl) * MLP_HID + i] : 0.0f;
+    const float a = live ? sm.z1[sl * LDZ + i] : 0.0f;
+    const float b = live ? sm.z2[sl * LDZ + i] : 0.0f;
     sm.h1T[i * LDC + sl] = __float2bfloat16(fmaxf(a, 0.0f));
     sm.h2T[i * LDC + sl] = __float2bfloat16(fmaxf(b, 0.0f));
-    sm.z2[sl * MLP_HID + i] = b;
+    if (!live) sm.z2[sl * LDZ + i] = 0.0f;
   }
   for (int e = tid; e < kBwdChunk * MLP_IN; e += kBwdThreads) {
     const int sl = e / MLP_IN, i = e % MLP_IN;
@@ -139,44 +151,50 @@ __global__ void __launch_bounds__(kBwdThreads) mlp_backward_kernel(
   if (tid < kBwdChunk) {  // layer-1 ReLU mask of sample tid
     unsigned long long mk = 0;
     if (tid < ns)
-      for (int i = 0; i < MLP_HID; ++i) mk |= (unsigned long long)(z1[(s0 + tid) * MLP_HID + i] > 0.0f) << i;
+      for (int i = 0; i < MLP_HID; ++i) mk |= (unsigned long long)(sm.z1[tid * LDZ + i] > 0.0f) << i;
     sm.mask1[tid] = mk;
   }
   __syncthreads();
-  // ---- per sample: dy, dh2 = W3^T dy (K = 2, FP32) and the layer-2 mask
-  if (tid < kBwdChunk) {
-    const int sl = tid;
+  // ---- per sample: dy, dh2 = W3^T dy (K = 2, FP32) and the layer-2 mask; the
+  // hidden units of a sample over kBwdThreads / kBwdChunk threads
+  {
+    const int sl = tid % kBwdChunk, part_i = tid / kBwdChunk;
+    constexpr int NI = MLP_HID / (kBwdThreads / kBwdChunk);
     const bool live = sl < ns;
     float d[MLP_OUT], err = 0.0f;
     for (int o = 0; o < MLP_OUT; ++o) {
-      const float e = live ? y[(s0 + sl) * MLP_OUT + o] - target[(s0 + sl) * MLP_OUT + o] : 0.0f;
+      const float e = live ? sm.y[sl * MLP_OUT + o] - target[(s0 + sl) * MLP_OUT + o] : 0.0f;
       err += e * e;
       d[o] = 2.0f * e / (float)B;
-      sm.dyf[sl * MLP_OUT + o] = d[o];
-      sm.dyT[o * LDC + sl] = __float2bfloat16(d[o]);
+      if (part_i == 0) {
+        sm.dyf[sl * MLP_OUT + o] = d[o];
+        sm.dyT[o * LDC + sl] = __float2bfloat16(d[o]);
+      }
     }
-    sm.err2[sl] = err;
-    for (int i = 0; i < MLP_HID; ++i) {
+    if (part_i == 0) sm.err2[sl] = err;
+    for (int i = part_i * NI; i < (part_i + 1) * NI; ++i) {
       float a = 0.0f;
       for (int o = 0; o < MLP_OUT; ++o) a += d[o] * sm.W3[o * MLP_HID + i];
-      const float dz = sm.z2[sl * MLP_HID + i] > 0.0f ? a : 0.0f;
-      sm.dz2f[sl * MLP_HID + i] = dz;
+      const float dz = sm.z2[sl * LDZ + i] > 0.0f ? a : 0.0f;
+      sm.dz2f[sl * LDZ + i] = dz;
       const __nv_bfloat16 q = __float2bfloat16(dz);
       sm.dz2r[sl * LDH + i] = q;
       sm.dz2T[i * LDC + sl] = q;
     }
   }
   __syncthreads();
-  // ---- dh1 = dz2 W2 on the tensor cores (warp w: samples 16w..16w+15), layer-1 mask
-  for (int nt = 0; nt < MLP_HID / 8; ++nt) {
+  // ---- dh1 = dz2 W2 on the tensor cores (warp w: 16 samples from 16 (w mod 4),
+  // every second 8 units from 8 (w / 4)), layer-1 mask
+  const int mw = 16 * (warp % (kBwdChunk / 16));
+  for (int nt = warp / (kBwdChunk / 16); nt < MLP_HID / 8; nt += kBwdThreads / 32 / (kBwdChunk / 16)) {
     float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    mma_tile(c, sm.dz2r, LDH, sm.W2T, LDH, 16 * warp, 8 * nt, MLP_HID / 16);
-    const int r0 = 16 * warp + g, r1 = r0 + 8, col = 8 * nt + 2 * t;
+    mma_tile(c, sm.dz2r, LDH, sm.W2T, LDH, mw, 8 * nt, MLP_HID / 16);
+    const int r0 = mw + g, r1 = r0 + 8, col = 8 * nt + 2 * t;
     const float v[4] = {c[0], c[1], c[2], c[3]};
     const int rows[4] = {r0, r0, r1, r1}, cols[4] = {col, col + 1, col, col + 1};
     for (int q = 0; q < 4; ++q) {
       const float dz = (sm.mask1[rows[q]] >> cols[q]) & 1ull ? v[q] : 0.0f;
-      sm.dz1f[rows[q] * MLP_HID + cols[q]] = dz;
+      sm.dz1f[rows[q] * LDZ + cols[q]] = dz;
       sm.dz1T[cols[q] * LDC + rows[q]] = __float2bfloat16(dz);
     }
   }
@@ -218,8 +236,8 @@ __global__ void __launch_bounds__(kBwdThreads) mlp_backward_kernel(
   if (tid < MLP_HID) {
     float a = 0.0f, b = 0.0f;
     for (int sl = 0; sl < kBwdChunk; ++sl) {
-      a += sm.dz1f[sl * MLP_HID + tid];
-      b += sm.dz2f[sl * MLP_HID + tid];
+      a += sm.dz1f[sl * LDZ + tid];
+      b += sm.dz2f[sl * LDZ + tid];
     }
     out[OFF_B1 + tid] = a;
     out[OFF_B2 + tid] = b;
@@ -235,36 +253,54 @@ __global__ void __launch_bounds__(kBwdThreads) mlp_backward_kernel(
   }
 }
 
-// grad[p] = sum over chunks (in chunk order) of part[c][p]; loss = sum / B.
-__global__ void mlp_grad_reduce_kernel(int n_chunks, int64_t B, const float* __restrict__ part,
-                                       const float* __restrict__ loss_part, float* __restrict__ grad,
-                                       float* __restrict__ loss) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p == 0) {
-    float l = 0.0f;
-    for (int c = 0; c < n_chunks; ++c) l += loss_part[c];
-    *loss = l / (float)B;
+// sum of v[c * stride] over c < n, in order; the loads go ahead of the
+// additions, which wait for each other.
+__device__ __forceinline__ float ordered_sum(const float* __restrict__ v, int n, int64_t stride) {
+  constexpr int U = 16;
+  float a = 0.0f, t[U];
+  for (int c = 0; c < n; c += U) {
+#pragma unroll
+    for (int k = 0; k < U; ++k) t[k] = v[(int64_t)min(c + k, n - 1) * stride];
+#pragma unroll
+    for (int k = 0; k < U; ++k)
+      if (c + k < n) a += t[k];
   }
-  if (p >= MLP_NPARAM) return;
-  float a = 0.0f;
-  for (int c = 0; c < n_chunks; ++c) a += part[(int64_t)c * MLP_NPARAM + p];
-  grad[p] = a;
+  return a;
 }
 
 // Adam (Kingma & Ba 2015) on the FP32 masters, then the BF16 copy.
-__global__ void mlp_adam_kernel(float* __restrict__ w, __nv_bfloat16* __restrict__ wbf, float* __restrict__ m,
-                                float* __restrict__ v, const float* __restrict__ g, float lr, float b1, float b2,
-                                float eps, float c1, float c2) {
+struct AdamStep {
+  float *w, *m, *v;
+  __nv_bfloat16* wbf;
+  float lr, b1, b2, eps, c1, c2;
+  __device__ __forceinline__ void operator()(int p, float gp) const {
+    const float mp = b1 * m[p] + (1.0f - b1) * gp;
+    const float vp = b2 * v[p] + (1.0f - b2) * gp * gp;
+    m[p] = mp;
+    v[p] = vp;
+    const float wp = w[p] - lr * (mp / c1) / (sqrtf(vp / c2) + eps);
+    w[p] = wp;
+    wbf[p] = __float2bfloat16(wp);
+  }
+};
+
+// grad[p] = sum over chunks (in chunk order) of part[c][p]; loss = sum / B;
+// with ADAM, the Adam step on it.
+template <bool ADAM>
+__global__ void mlp_grad_reduce_kernel(int n_chunks, int64_t B, const float* __restrict__ part,
+                                       const float* __restrict__ loss_part, float* __restrict__ grad,
+                                       float* __restrict__ loss, AdamStep adam) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p == MLP_NPARAM) *loss = ordered_sum(loss_part, n_chunks, 1) / (float)B;
   if (p >= MLP_NPARAM) return;
-  const float gp = g[p];
-  const float mp = b1 * m[p] + (1.0f - b1) * gp;
-  const float vp = b2 * v[p] + (1.0f - b2) * gp * gp;
-  m[p] = mp;
-  v[p] = vp;
-  const float wp = w[p] - lr * (mp / c1) / (sqrtf(vp / c2) + eps);
-  w[p] = wp;
-  wbf[p] = __float2bfloat16(wp);
+  const float g = ordered_sum(part + p, n_chunks, MLP_NPARAM);
+  grad[p] = g;
+  if constexpr (ADAM) adam(p, g);
+}
+
+__global__ void mlp_adam_kernel(const float* __restrict__ g, AdamStep adam) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p < MLP_NPARAM) adam(p, g[p]);
 }
 
 __global__ void mlp_to_bf16_kernel(const float* __restrict__ w, __nv_bfloat16* __restrict__ wbf) {
@@ -272,8 +308,7 @@ __global__ void mlp_to_bf16_kernel(const float* __restrict__ w, __nv_bfloat16* _
   if (p < MLP_NPARAM) wbf[p] = __float2bfloat16(w[p]);
 }
 
-static int mlp_fwd_launch(const ht_mlp* net, int64_t B, const float* x, float* y, float* z1, float* z2,
-                          cudaStream_t st) {
+static int mlp_fwd_launch(const ht_mlp* net, int64_t B, const float* x, float* y, cudaStream_t st) {
   const size_t smem = sizeof(MlpFwdSmem);
   static bool attr_set = false;
   if (!attr_set) {
@@ -285,18 +320,16 @@ static int mlp_fwd_launch(const ht_mlp* net, int64_t B, const float* x, float* y
   int64_t cap = (int64_t)sm_count() * 8;
   if (grid > cap) grid = cap;
   if (grid < 1) grid = 1;
-  mlp_forward_kernel<<<(unsigned)grid, kMlpThreads, smem, st>>>(net->wbf, net->master, B, x, y, z1, z2);
+  mlp_forward_kernel<<<(unsigned)grid, kMlpThreads, smem, st>>>(net->wbf, net->master, B, x, y);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? HT_OK : cuda_fail(e, "mlp forward launch");
 }
 
-// Workspace for a batch of B samples (Bp = B rounded up to 32 rows, C chunks
-// of kBwdChunk samples): y [Bp][2]; z1, z2 [Bp][64]; partial gradients
-// [C][MLP_NPARAM]; partial losses [C].
-static int mlp_ws(ht_mlp* net, int64_t B, float** y, float** z1, float** z2, float** part, float** lpart,
-                  cudaStream_t st) {
-  const int64_t Bp = (B + 31) / 32 * 32, C = (B + kBwdChunk - 1) / kBwdChunk;
-  size_t need = ((size_t)Bp * (MLP_OUT + 2 * MLP_HID) + (size_t)C * (MLP_NPARAM + 1)) * sizeof(float);
+// Workspace for batches of up to B samples (C chunks of kBwdChunk) and `losses`
+// batch losses: partial gradients [C][MLP_NPARAM]; partial losses [C]; losses.
+static int mlp_ws(ht_mlp* net, int64_t B, int64_t losses, float** part, float** lpart, float** lbuf, cudaStream_t st) {
+  const int64_t C = (B + kBwdChunk - 1) / kBwdChunk;
+  size_t need = ((size_t)C * (MLP_NPARAM + 1) + (size_t)losses) * sizeof(float);
   if (net->ws_bytes < need) {
     if (net->ws) {
       cudaStreamSynchronize(st);
@@ -312,24 +345,29 @@ static int mlp_ws(ht_mlp* net, int64_t B, float** y, float** z1, float** z2, flo
     net->ws_bytes = need;
   }
   float* f = (float*)net->ws;
-  *y = f;
-  f += Bp * MLP_OUT;
-  *z1 = f;
-  f += Bp * MLP_HID;
-  *z2 = f;
-  f += Bp * MLP_HID;
   *part = f;
   f += C * MLP_NPARAM;
   *lpart = f;
+  f += C;
+  if (lbuf) *lbuf = f;
   return HT_OK;
 }
 
-static int mlp_grad_batch(ht_mlp* net, int64_t B, const float* x, const float* target, cudaStream_t st) {
-  float *y, *z1, *z2, *part, *lpart;
-  int rc = mlp_ws(net, B, &y, &z1, &z2, &part, &lpart, st);
-  if (rc != HT_OK) return rc;
-  rc = mlp_fwd_launch(net, B, x, y, z1, z2, st);
-  if (rc != HT_OK) return rc;
+// The next Adam step of the network at rate lr.
+static AdamStep adam_step(ht_mlp* net, float lr) {
+  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+  ++net->step;
+  // bias corrections 1 - beta^k in double, rounded once: in FP32, 1 - powf
+  // would amplify powf's rounding by beta^k / (1 - beta^k) (about 1000 at k = 1)
+  const float c1 = (float)(1.0 - std::pow((double)b1, (double)net->step));
+  const float c2 = (float)(1.0 - std::pow((double)b2, (double)net->step));
+  return AdamStep{net->master, net->m, net->v, net->wbf, lr, b1, b2, eps, c1, c2};
+}
+
+// Gradient of one batch into net->grad and its loss into *loss; with adam,
+// that Adam step as well.
+static int mlp_grad_batch(ht_mlp* net, int64_t B, const float* x, const float* target, float* part, float* lpart,
+                          float* loss, const AdamStep* adam, cudaStream_t st) {
   const int64_t C = (B + kBwdChunk - 1) / kBwdChunk;
   const size_t smem = sizeof(MlpBwdSmem);
   static bool attr_set = false;
@@ -337,21 +375,18 @@ static int mlp_grad_batch(ht_mlp* net, int64_t B, const float* x, const float* t
     cudaFuncSetAttribute(mlp_backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     attr_set = true;
   }
-  mlp_backward_kernel<<<(unsigned)C, kBwdThreads, smem, st>>>(net->wbf, B, x, y, target, z1, z2, part, lpart);
-  mlp_grad_reduce_kernel<<<(MLP_NPARAM + 127) / 128, 128, 0, st>>>((int)C, B, part, lpart, net->grad, net->loss);
+  mlp_backward_kernel<<<(unsigned)C, kBwdThreads, smem, st>>>(net->wbf, net->master, B, x, target, part, lpart);
+  const unsigned blocks = (MLP_NPARAM + 1 + 127) / 128;
+  if (adam)
+    mlp_grad_reduce_kernel<true><<<blocks, 128, 0, st>>>((int)C, B, part, lpart, net->grad, loss, *adam);
+  else
+    mlp_grad_reduce_kernel<false><<<blocks, 128, 0, st>>>((int)C, B, part, lpart, net->grad, loss, AdamStep());
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? HT_OK : cuda_fail(e, "mlp backward launch");
 }
 
 static int mlp_adam_launch(ht_mlp* net, const float* grad, float lr, cudaStream_t st) {
-  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  ++net->step;
-  // bias corrections 1 - beta^k in double, rounded once: in FP32, 1 - powf
-  // would amplify powf's rounding by beta^k / (1 - beta^k) (about 1000 at k = 1)
-  const float c1 = (float)(1.0 - std::pow((double)b1, (double)net->step));
-  const float c2 = (float)(1.0 - std::pow((double)b2, (double)net->step));
-  mlp_adam_kernel<<<(MLP_NPARAM + 255) / 256, 256, 0, st>>>(net->master, net->wbf, net->m, net->v, grad, lr, b1, b2,
-                                                            eps, c1, c2);
+  mlp_adam_kernel<<<(MLP_NPARAM + 255) / 256, 256, 0, st>>>(grad, adam_step(net, lr));
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? HT_OK : cuda_fail(e, "mlp adam launch");
 }
@@ -426,7 +461,7 @@ int ht_mlp_forward(const ht_mlp* net, int64_t B, const float* x, float* y, void*
   if (B == 0) return HT_OK;
   if (!x || !y || !is_device_ptr(x) || !is_device_ptr(y) || (((uintptr_t)x | (uintptr_t)y) & 3))
     return set_error(HT_EINVAL, "ht_mlp_forward: x and y must be device memory");
-  return mlp_fwd_launch(net, B, x, y, nullptr, nullptr, (cudaStream_t)stream);
+  return mlp_fwd_launch(net, B, x, y, (cudaStream_t)stream);
 }
 
 int ht_mlp_loss_grad(ht_mlp* net, int64_t B, const float* x, const float* target, float* grad, float* loss,
@@ -436,7 +471,9 @@ int ht_mlp_loss_grad(ht_mlp* net, int64_t B, const float* x, const float* target
       (grad && !is_device_ptr(grad)) || (loss && !is_device_ptr(loss)))
     return set_error(HT_EINVAL, "ht_mlp_loss_grad: bad arguments");
   cudaStream_t st = (cudaStream_t)stream;
-  int rc = mlp_grad_batch(net, B, x, target, st);
+  float *part, *lpart;
+  int rc = mlp_ws(net, B, 0, &part, &lpart, nullptr, st);
+  if (rc == HT_OK) rc = mlp_grad_batch(net, B, x, target, part, lpart, net->loss, nullptr, st);
   if (rc != HT_OK) return rc;
   cudaError_t e = cudaSuccess;
   if (grad) e = cudaMemcpyAsync(grad, net->grad, MLP_NPARAM * sizeof(float), cudaMemcpyDeviceToDevice, st);
@@ -451,26 +488,42 @@ int ht_mlp_train(ht_mlp* net, int64_t n, const float* x, const float* target, in
       !is_device_ptr(target))
     return set_error(HT_EINVAL, "ht_mlp_train: bad arguments");
   cudaStream_t st = (cudaStream_t)stream;
-  for (int ep = 0; ep < epochs; ++ep) {
-    double sum = 0.0;
-    int nb = 0;
-    for (int64_t off = 0; off < n; off += batch) {
-      const int64_t B = (off + batch <= n) ? batch : n - off;
-      int rc = mlp_grad_batch(net, B, x + off * MLP_IN, target + off * MLP_OUT, st);
-      if (rc != HT_OK) return rc;
-      rc = mlp_adam_launch(net, net->grad, lr, st);
-      if (rc != HT_OK) return rc;
-      if (epoch_loss) {
-        float l = 0;
-        cudaError_t e = cudaMemcpyAsync(&l, net->loss, sizeof(float), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) return cuda_fail(e, "ht_mlp_train");
-        sum += l;
-        ++nb;
+  // the batches' losses stay on the device and come back up to kLosses at a
+  // time (the host used to wait for each)
+  constexpr int64_t kLosses = 1 << 14;
+  const int64_t nb = n / batch + (n % batch != 0);
+  float *part, *lpart, *lbuf;
+  int rc = mlp_ws(net, batch < n ? batch : n, kLosses, &part, &lpart, &lbuf, st);
+  if (rc != HT_OK) return rc;
+  std::vector<float> hl(kLosses);
+  int64_t kept = 0;  // losses on the device
+  double sum = 0.0;
+  int64_t summed = 0;  // batches of the running epoch in sum
+  int done = 0;        // epochs reported
+  auto flush = [&]() {
+    cudaError_t e = cudaMemcpyAsync(hl.data(), lbuf, kept * sizeof(float), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_fail(e, "ht_mlp_train");
+    for (int64_t k = 0; k < kept; ++k) {
+      sum += hl[k];
+      if (++summed == nb) {
+        epoch_loss[done++] = (float)(sum / (double)nb);
+        sum = 0.0;
+        summed = 0;
       }
     }
-    if (epoch_loss) epoch_loss[ep] = (float)(sum / (nb ? nb : 1));
-  }
+    kept = 0;
+    return (int)HT_OK;
+  };
+  for (int ep = 0; ep < epochs; ++ep)
+    for (int64_t b = 0; b < nb; ++b) {
+      const int64_t off = b * batch, B = n - off < batch ? n - off : batch;
+      const AdamStep adam = adam_step(net, lr);
+      rc = mlp_grad_batch(net, B, x + off * MLP_IN, target + off * MLP_OUT, part, lpart, lbuf + kept, &adam, st);
+      if (rc == HT_OK && epoch_loss && ++kept == kLosses) rc = flush();
+      if (rc != HT_OK) return rc;
+    }
+  if (kept > 0 && (rc = flush()) != HT_OK) return rc;
   cudaError_t e = cudaStreamSynchronize(st);
   return e == cudaSuccess ? HT_OK : cuda_fail(e, "ht_mlp_train");
 }

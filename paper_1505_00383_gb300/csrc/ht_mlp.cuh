@@ -68,10 +68,12 @@ __device__ __forceinline__ void mma_bf16(float* d, const uint32_t* a, uint32_t b
 // Forward pass for the warp's 32 samples.  Each lane passes the features of
 // its own sample (x[16]) and receives its outputs y[2].  If z1_rows is given,
 // the pre-activations of both hidden layers are also written to z1_rows and
-// z2_rows ([32][64] each, row = sample of the warp) for the backward pass.
+// z2_rows ([32][64] each, row = sample of the warp, z_ld floats apart) for the
+// backward pass.
 // All 32 lanes must call it.
 __device__ __forceinline__ void mlp_forward_warp(const MlpSmem& s, MlpWarpSmem& w, const float* x, float* y,
-                                                 float* z1_rows = nullptr, float* z2_rows = nullptr) {
+                                                 float* z1_rows = nullptr, float* z2_rows = nullptr,
+                                                 int z_ld = MLP_HID) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   for (int i = 0; i < MLP_IN; i += 2) *reinterpret_cast<uint32_t*>(&w.X[lane * LDX + i]) = pack_bf16(x[i], x[i + 1]);
   __syncwarp();
@@ -138,14 +140,14 @@ __device__ __forceinline__ void mlp_forward_warp(const MlpSmem& s, MlpWarpSmem& 
     if (z1_rows) {
       for (int j = 0; j < 8; ++j) {
         const int c = 8 * j + 2 * t;
-        z1_rows[(size_t)r0 * MLP_HID + c] = h1[j][0];
-        z1_rows[(size_t)r0 * MLP_HID + c + 1] = h1[j][1];
-        z1_rows[(size_t)r1 * MLP_HID + c] = h1[j][2];
-        z1_rows[(size_t)r1 * MLP_HID + c + 1] = h1[j][3];
-        z2_rows[(size_t)r0 * MLP_HID + c] = h2[j][0];
-        z2_rows[(size_t)r0 * MLP_HID + c + 1] = h2[j][1];
-        z2_rows[(size_t)r1 * MLP_HID + c] = h2[j][2];
-        z2_rows[(size_t)r1 * MLP_HID + c + 1] = h2[j][3];
+        z1_rows[(size_t)r0 * z_ld + c] = h1[j][0];
+        z1_rows[(size_t)r0 * z_ld + c + 1] = h1[j][1];
+        z1_rows[(size_t)r1 * z_ld + c] = h1[j][2];
+        z1_rows[(size_t)r1 * z_ld + c + 1] = h1[j][3];
+        z2_rows[(size_t)r0 * z_ld + c] = h2[j][0];
+        z2_rows[(size_t)r0 * z_ld + c + 1] = h2[j][1];
+        z2_rows[(size_t)r1 * z_ld + c] = h2[j][2];
+        z2_rows[(size_t)r1 * z_ld + c + 1] = h2[j][3];
       }
     }
   }
