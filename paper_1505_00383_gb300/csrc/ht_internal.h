@@ -46,6 +46,7 @@ struct ht_system {
   struct GraphEntry {            // captured rounds of the tracker for one team size
     int team = 0;
     int64_t groups = 0;
+    bool col = false;
     const void* key_a = nullptr;
     const void* key_b = nullptr;
     cudaGraphExec_t exec = nullptr;

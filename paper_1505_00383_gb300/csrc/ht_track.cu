@@ -23,6 +23,7 @@
 // paths" of Table tabmemory.
 #include <algorithm>
 
+#include "ht_col_mgs.cuh"
 #include "ht_eval.cuh"
 #include "ht_int_mgs.cuh"
 #include "ht_internal.h"
@@ -34,8 +35,14 @@ namespace ht {
 
 enum : int8_t { PH_TRACK = 0, PH_POLISH = 1 };
 
-// max over values that lets a NaN through (a NaN norm rejects the step)
-__device__ __forceinline__ double nanmax(double m, double v) { return (v > m || v != v) ? v : m; }
+// max over non-negative values that lets a NaN through (a NaN norm rejects the
+// step).  Their bit patterns are ordered as they are, with NaN above infinity,
+// so the comparison runs on the integer pipe (a double-precision comparison
+// holds the FP64 pipe for 64 clocks).
+__device__ __forceinline__ double nanmax(double m, double v) {
+  const long long a = __double_as_longlong(m), b = __double_as_longlong(v) & 0x7fffffffffffffffLL;
+  return __longlong_as_double(a > b ? a : b);
+}
 
 template <int L>
 __device__ __forceinline__ cx<L> root_of_unity(int d, int k) {
@@ -554,12 +561,12 @@ __device__ __forceinline__ cx<L> cx_from(const double* re, const double* im) {
 // few groups of double and double-double paths with more warps each, and
 // any group when the autotuner picks 16).
 template <int L, bool LEARN, bool INT, int MAXT = INT ? 16 : 8>
-__global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 2 ? 2 : 1))) track_kernel(TrackArgs a) {
+__global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 4 : (L == 2 ? 2 : 1))) track_kernel(TrackArgs a) {
   __shared__ double red[4][MAXT][32];  // per-warp partials: residual, update, point norms; finiteness
   __shared__ double sh_h[32];       // learned step of each lane's path
   __shared__ double sh_alpha[32];   // learned tangent correction of each lane's path
   __shared__ long long sh_slot[32]; // trace record slot of each lane's path (-1: none)
-  __shared__ double sh_w[L > 1 ? 8 : 1][L][32];  // extrapolation weights (DD, QD), [point][limb][lane]
+  __shared__ double sh_w[8][L][32];  // extrapolation weights, [point][limb][lane]
   // The network's weights are read from the device image (L1/L2): staging
   // them in shared memory would enlarge the shared-memory carveout and take
   // L1 capacity from the Newton workspace.  Only warp 0's sample staging
@@ -581,6 +588,8 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
   // DD and QD with integer evaluation keep A as limb strings from the
   // evaluation through the least squares: no conversions
   constexpr bool FZ = INT && L >= 2;
+  // double, few paths: the least squares with a column per lane (ht_col_mgs.cuh)
+  constexpr bool COL = L == 1 && MAXT > 8;
   // (a block per CTA, which its groups reuse, so that it stays in L2: path l
   // of the group, entry j of a row, NQ 128-bit words: [32][W][NQ][n], row
   // fastest, as the lanes of the solve read it)
@@ -606,10 +615,10 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
   // paths as give every CTA one, since its rounds shorten with the work the
   // SM shares.  In double a group's cost is its instruction count on the FP64
   // pipe, whatever the lanes in use, so it always takes 32.
+  // (with a column per lane in the least squares the lanes count there too)
   int G = 32;
-  if constexpr (FZ) {
-    G = (count + (int)gridDim.x - 1) / (int)gridDim.x;
-  }
+  const bool col = COL && a.col_lanes;
+  if (FZ || col) G = min(32, (count + (int)gridDim.x - 1) / (int)gridDim.x);
   __shared__ int sh_group;
   for (;;) {
     if (threadIdx.x == 0) sh_group = atomicAdd(a.queue, 1);
@@ -719,7 +728,7 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
       if (start) {
         double step = fmin(h, 1.0 - t);
         t1 = (step >= 1.0 - t) ? 1.0 : t + step;
-        if constexpr (L > 1) {
+        {
           for (int j = warp; j < mm; j += T) {
             const rl<L> wj = weight(j);
 #pragma unroll
@@ -728,7 +737,8 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
           // the tangent predictors' weights once, by the last warp; in QD on
           // limb strings (a division and a dozen products: 250,000 clocks of
           // the FP64 pipe's latency)
-          if (FZ && L == 4 && warp == T - 1 && herm) {
+          if (L == 1) {
+          } else if (FZ && L == 4 && warp == T - 1 && herm) {
             if constexpr (L == 4) {
               constexpr int WZ = IntW<L>::W;
               const double s0 = a.ht[(int64_t)(nh - 2) * m + p], s1 = a.ht[(int64_t)(nh - 1) * m + p];
@@ -763,9 +773,10 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
           }
         }
       }
-      // (in double a weight is a few instructions: every warp computes them,
-      // without the barrier)
-      if constexpr (L > 1) __syncthreads();
+      // (in double too: a division holds the FP64 pipe for 1,474 clocks, and
+      // with 64 registers dealing takes 16,384 paths of n = 16 from 948 to 923
+      // ms, 4,096 of n = 12 from 200 to 191 ms)
+      __syncthreads();
       if (start) {
         if constexpr (L == 1) {
           tangent_weights();
@@ -783,14 +794,10 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
         }
         rl<L> w[8];
         for (int j = 0; j < mm; ++j) {
-          if constexpr (L > 1) {
-            double wl[L];
+          double wl[L];
 #pragma unroll
-            for (int l = 0; l < L; ++l) wl[l] = sh_w[j][l][lane];
-            w[j] = r_of<L>(wl);
-          } else {
-            w[j] = weight(j);
-          }
+          for (int l = 0; l < L; ++l) wl[l] = sh_w[j][l][lane];
+          w[j] = r_of<L>(wl);
         }
         for (int i = warp; i < n; i += T) {
           cx<L> acc = czero<L>();
@@ -1041,8 +1048,24 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 3 : (L == 
         }
         __syncthreads();
       }
-      else
-        mgs_team<L>(a.A, a.R, a.dx, n, n, m, p, act, warp, T, nrhs, a.tdx);
+      if constexpr (COL) {
+        if (col) {
+          const unsigned live = __ballot_sync(0xffffffffu, act);
+          const int per = ColLanes::systems(n, nrhs), chunks = (G + per - 1) / per;
+          double2* sh = reinterpret_cast<double2*>(xs_int) + warp * ColLanes::words(n, nrhs);
+          for (int c = warp; c < chunks; c += T) {  // at most ColLanes::WARPS chunks
+            const int pl = c * per + min(lane / ColLanes::lanes(n, nrhs), per - 1);
+            const int64_t ps = __shfl_sync(0xffffffffu, (int)p, min(pl, 31));
+            ColLanes::solve(
+                n, nrhs, pl < 32 && ((live >> pl) & 1u), sh,
+                [&](int i, int j) { return ld<1>(a.A, (int64_t)i * W + j, m, ps); },
+                [&](int k, int i, const cx<1>& z) { st<1>(k == 0 ? a.dx : a.tdx, i, m, ps, z); });
+          }
+          __syncthreads();
+        }
+      }
+      if constexpr (!FZ)
+        if (!col) mgs_team<L>(a.A, a.R, a.dx, n, n, m, p, act, warp, T, nrhs, a.tdx);
       // ---- D: x <- x + dx on this warp's coordinates; partial norms
       double pdx = 0.0, pxp = 0.0;
       if (act) {
@@ -1276,6 +1299,9 @@ int launch_mgs_l(double* A, double* R, double* x, int rows, int cols, int64_t n_
 }
 
 #if HT_LIMBS == 1
+int64_t track_col_paths(int n, int nrhs) {
+  return n > ColLanes::N ? 0 : (int64_t)sm_count() * ColLanes::WARPS * ColLanes::systems(n, nrhs);
+}
 int64_t track_int_ctas(int64_t groups) { return std::max<int64_t>(1, std::min<int64_t>(groups, 4 * (int64_t)sm_count())); }
 size_t track_int_bytes(int L, int n, int nrhs) {
   return (size_t)32 * n * (n + nrhs) * (L == 4 ? sizeof(mpi::fzs<8>) : sizeof(mpi::fzs<5>));
@@ -1332,9 +1358,16 @@ int launch_track_l(const TrackArgs& a, int team, int64_t max_groups, cudaStream_
       const size_t dsm = std::max(smem_points_bytes<L>(a.n), (size_t)team * RowLanes<L>::WORDS * sizeof(int32_t));
       learn ? go(track_kernel<L, true, true>, dsm) : go(track_kernel<L, false, true>, dsm);
     }
-  } else if (team > 8) {  // wide teams: double and double double (the host only asks for these)
-    if (L == 4) return set_error(HT_EUNSUPPORTED, "track launch: teams above 8 warps need D or DD");
-    learn ? go(track_kernel<L, true, false, 16>, 0) : go(track_kernel<L, false, false, 16>, 0);
+  } else if (team > 8 || a.col_lanes || (L <= 2 && max_groups <= sm_count())) {
+    // wide teams, and groups that have an SM each (no use for the other
+    // kernel's 64 registers): double and double double
+    if constexpr (L == 4) {
+      return set_error(HT_EUNSUPPORTED, "track launch: teams above 8 warps need D or DD");
+    } else {
+      const size_t dsm =
+          a.col_lanes ? (size_t)ColLanes::WARPS * ColLanes::words(a.n, a.prm.predictor > 0 ? 2 : 1) * sizeof(double2) : 0;
+      learn ? go(track_kernel<L, true, false, 16>, dsm) : go(track_kernel<L, false, false, 16>, dsm);
+    }
   } else {
     learn ? go(track_kernel<L, true, false>, 0) : go(track_kernel<L, false, false>, 0);
   }

@@ -42,6 +42,7 @@ struct TrackArgs {
   int n;
   int64_t m;
   int iters;
+  int col_lanes;  // double, few paths: least squares with a column per lane
   TrackPrm prm;
   double* x;   // [n]     accepted point (the caller's x_end)
   double* xp;  // [n]     working point
@@ -94,6 +95,8 @@ struct TrackArgs {
 // bytes of the workspace A of each for an L-limb system in n variables.
 int64_t track_int_ctas(int64_t groups);
 size_t track_int_bytes(int L, int n, int nrhs);
+// Active paths up to which the double tracker solves with a column per lane (0: never).
+int64_t track_col_paths(int n, int nrhs);
 
 template <int L>
 int launch_start_l(int n, const int32_t* d_deg, int64_t first, int64_t count, double* x, cudaStream_t st);

@@ -434,6 +434,8 @@ int ht_track_paths_ex(ht_system* s, const int32_t* start_deg, const double* gamm
     int t = 1;
     if (s->track_team > 0 && s->track_team <= 16) {
       t = s->track_team;
+    } else if (L == 1 && active <= track_col_paths(n, nrhs)) {
+      return std::max(4, std::min(16, n));  // a warp per polynomial, four at least for the solve
     } else if (int_eval) {
       return 16;  // the rows of the systems, and in small groups their columns, spread over all
     } else {
@@ -450,13 +452,15 @@ int ht_track_paths_ex(ht_system* s, const int32_t* start_deg, const double* gamm
   while (active > 0) {
     int team = pick_team(active);
     // CTAs a launch can use: groups of 32 paths; on the integer pipe as few
-    // paths as spread over the SMs
+    // paths as spread over the SMs, and in double with a column per lane
     int64_t groups = (active + 31) / 32;
-    if (int_eval) groups = std::max(groups, std::min<int64_t>(active, sm_count()));
+    const bool col = L == 1 && active <= track_col_paths(n, nrhs);
+    if (int_eval || col) groups = std::max(groups, std::min<int64_t>(active, sm_count()));
     // graph for this (team, iters, rounds, workspace, outputs) configuration
     ht_system::GraphEntry* ge = nullptr;
     for (auto& g : s->graphs)
-      if (g.team == team && g.key_a == (const void*)x_end && g.key_b == (const void*)status && g.groups >= groups) ge = &g;
+      if (g.team == team && g.key_a == (const void*)x_end && g.key_b == (const void*)status && g.groups >= groups && g.col == col)
+        ge = &g;
     if (!ge) {
       cudaGraph_t graph;
       cudaStream_t cs;
@@ -474,6 +478,7 @@ int ht_track_paths_ex(ht_system* s, const int32_t* start_deg, const double* gamm
         ar.count_in = cnt[r & 1];
         ar.queue = queue[r & 1];
         ar.iters = iters;
+        ar.col_lanes = col;
         crc = by_limbs(L, [&](auto c) { return launch_track_l<decltype(c)::value>(ar, team, groups, cs); });
         if (crc == HT_OK)
           crc = launch_compact(idx[r & 1], cnt[r & 1], status, idx[(r + 1) & 1], cnt[(r + 1) & 1], cs,
@@ -493,6 +498,7 @@ int ht_track_paths_ex(ht_system* s, const int32_t* start_deg, const double* gamm
       ht_system::GraphEntry g;
       g.team = team;
       g.groups = groups;
+      g.col = col;
       g.key_a = x_end;
       g.key_b = status;
       ee = cudaGraphInstantiate(&g.exec, graph, 0);
