@@ -17,7 +17,7 @@
 namespace ht {
 
 struct ColLanes {
-  static constexpr int N = 16;      // largest n
+  static constexpr int MAX = 16;    // largest n
   static constexpr int WARPS = 4;   // warps of a CTA that solve (one per sub-partition)
 
   static __host__ __device__ int lanes(int n, int nrhs) { return n + nrhs - 1; }
@@ -30,8 +30,10 @@ struct ColLanes {
 
   // All 32 lanes call it.  load(i, j): entry (i, j) of [A | b] of this lane's
   // system; put(k, i, z): coordinate i of solution k (called by one lane);
-  // live: this lane's system exists.
-  template <class Load, class Put>
+  // live: this lane's system exists.  n <= N: the loops over the rows are
+  // unrolled N times, and a row past n still holds the FP64 pipe (predicated
+  // off: n = 6 with N = 16 took 106,000 clocks, as many per column as n = 16).
+  template <int N, class Load, class Put>
   static __device__ __forceinline__ void solve(int n, int nrhs, bool live, double2* sh, Load load, Put put) {
     const int lane = threadIdx.x & 31, lp = lanes(n, nrhs), sys = min(lane / lp, systems(n, nrhs) - 1), W = n + nrhs;
     const int c = lane - (lane / lp) * lp;
@@ -117,6 +119,21 @@ struct ColLanes {
       }
     }
     __syncwarp();  // the shared memory may be reused
+  }
+  template <class Load, class Put>
+  static __device__ __forceinline__ void solve_any(int n, int nrhs, bool live, double2* sh, Load load, Put put) {
+    if (n <= 4)
+      solve<4>(n, nrhs, live, sh, load, put);
+    else if (n <= 6)
+      solve<6>(n, nrhs, live, sh, load, put);
+    else if (n <= 8)
+      solve<8>(n, nrhs, live, sh, load, put);
+    else if (n <= 10)
+      solve<10>(n, nrhs, live, sh, load, put);
+    else if (n <= 12)
+      solve<12>(n, nrhs, live, sh, load, put);
+    else
+      solve<MAX>(n, nrhs, live, sh, load, put);
   }
 };
 

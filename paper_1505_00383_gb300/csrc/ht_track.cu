@@ -1056,7 +1056,7 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 4 : (L == 
           for (int c = warp; c < chunks; c += T) {  // at most ColLanes::WARPS chunks
             const int pl = c * per + min(lane / ColLanes::lanes(n, nrhs), per - 1);
             const int64_t ps = __shfl_sync(0xffffffffu, (int)p, min(pl, 31));
-            ColLanes::solve(
+            ColLanes::solve_any(
                 n, nrhs, pl < 32 && ((live >> pl) & 1u), sh,
                 [&](int i, int j) { return ld<1>(a.A, (int64_t)i * W + j, m, ps); },
                 [&](int k, int i, const cx<1>& z) { st<1>(k == 0 ? a.dx : a.tdx, i, m, ps, z); });
@@ -1300,7 +1300,7 @@ int launch_mgs_l(double* A, double* R, double* x, int rows, int cols, int64_t n_
 
 #if HT_LIMBS == 1
 int64_t track_col_paths(int n, int nrhs) {
-  return n > ColLanes::N ? 0 : (int64_t)sm_count() * ColLanes::WARPS * ColLanes::systems(n, nrhs);
+  return n > ColLanes::MAX ? 0 : (int64_t)sm_count() * ColLanes::WARPS * ColLanes::systems(n, nrhs);
 }
 int64_t track_int_ctas(int64_t groups) { return std::max<int64_t>(1, std::min<int64_t>(groups, 4 * (int64_t)sm_count())); }
 size_t track_int_bytes(int L, int n, int nrhs) {
