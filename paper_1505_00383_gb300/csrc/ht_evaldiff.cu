@@ -171,8 +171,12 @@ __global__ void __launch_bounds__(512) evaldiff_split_kernel(EvalArgs a, const i
               const int ex = (int)(w[i] >> 24);
               if (ex <= 1)
                 acc = cadd(acc, v[i]);
+              else if (ex == 2)
+                acc = caxpy(acc, 2.0, v[i]);
+              else if (ex == 3)
+                acc = caxpy(acc, 3.0, v[i]);
               else
-                acc = jacc<1>(acc, (double)ex, v[i]);
+                acc = caxpy(acc, (double)ex, v[i]);
             }
             t = min(t + U, te);
           }
