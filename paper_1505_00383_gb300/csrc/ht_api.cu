@@ -181,7 +181,9 @@ int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8
     std::vector<uint32_t> steps;
     std::vector<int32_t> step_off;
     if (n_vars <= 64) {
+      step_off.reserve(s->M + 1);
       step_off.assign(1, 0);
+      steps.reserve(4 * s->n_pairs + s->M);
       for (int64_t m = 0; m < s->M; ++m) {
         mpi::sweep_steps(s->h_pairs.data() + s->h_mon_off[m], s->h_mon_off[m + 1] - s->h_mon_off[m], steps);
         step_off.push_back((int32_t)steps.size());
@@ -197,6 +199,8 @@ int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8
     }
     if (limbs == 1 && s->max_slots < (1 << 24) && s->n_pairs + s->M < (1LL << 31)) {
       std::vector<std::vector<uint32_t>> of(n_vars + 1);
+      terms.reserve(s->n_pairs + s->M);
+      term_off.reserve((size_t)n_polys * (n_vars + 1) + 1);
       term_off.assign(1, 0);
       for (int j = 0; j < n_polys; ++j) {
         for (auto& o : of) o.clear();
@@ -214,25 +218,32 @@ int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8
     }
     const size_t b_hz = up(hz.size()), b_hl = up(hl.size() * sizeof(float)), b_so = up(step_off.size() * 4),
                  b_st = up(steps.size() * 4), b_to = up(term_off.size() * 4);
-    void* blk = nullptr;
-    e = cudaMalloc(&blk, b_hz + b_hl + b_so + b_st + b_to + terms.size() * 4);
+    // one upload: coefficients | log2 moduli | steps' offsets | steps | terms' offsets | terms
+    const size_t o_hl = b_hz, o_so = o_hl + b_hl, o_st = o_so + b_so, o_to = o_st + b_st, o_te = o_to + b_to;
+    std::vector<unsigned char> host(o_te + up(terms.size() * 4));
+    auto put = [&](size_t off, const void* p, size_t bytes) {
+      if (bytes) std::memcpy(&host[off], p, bytes);
+    };
+    put(0, hz.data(), hz.size());
+    put(o_hl, hl.data(), hl.size() * sizeof(float));
+    put(o_so, step_off.data(), step_off.size() * 4);
+    put(o_st, steps.data(), steps.size() * 4);
+    put(o_to, term_off.data(), term_off.size() * 4);
+    put(o_te, terms.data(), terms.size() * 4);
+    char* blk = nullptr;
+    e = cudaMalloc((void**)&blk, host.size());
     if (e == cudaSuccess) {
       s->d_coef_fz = blk;
-      s->d_coef_lg = (float*)((char*)blk + b_hz);
-      e = cudaMemcpy(s->d_coef_fz, hz.data(), hz.size(), cudaMemcpyHostToDevice);
-      if (e == cudaSuccess) e = cudaMemcpy(s->d_coef_lg, hl.data(), hl.size() * sizeof(float), cudaMemcpyHostToDevice);
-    }
-    if (e == cudaSuccess && !steps.empty()) {
-      s->d_step_off = (int32_t*)((char*)blk + b_hz + b_hl);
-      s->d_steps = (uint32_t*)((char*)blk + b_hz + b_hl + b_so);
-      e = cudaMemcpy(s->d_step_off, step_off.data(), step_off.size() * 4, cudaMemcpyHostToDevice);
-      if (e == cudaSuccess) e = cudaMemcpy(s->d_steps, steps.data(), steps.size() * 4, cudaMemcpyHostToDevice);
-    }
-    if (e == cudaSuccess && !terms.empty()) {
-      s->d_term_off = (int32_t*)((char*)blk + b_hz + b_hl + b_so + b_st);
-      s->d_terms = (uint32_t*)((char*)blk + b_hz + b_hl + b_so + b_st + b_to);
-      e = cudaMemcpy(s->d_term_off, term_off.data(), term_off.size() * 4, cudaMemcpyHostToDevice);
-      if (e == cudaSuccess) e = cudaMemcpy(s->d_terms, terms.data(), terms.size() * 4, cudaMemcpyHostToDevice);
+      s->d_coef_lg = (float*)(blk + o_hl);
+      if (!steps.empty()) {
+        s->d_step_off = (int32_t*)(blk + o_so);
+        s->d_steps = (uint32_t*)(blk + o_st);
+      }
+      if (!terms.empty()) {
+        s->d_term_off = (int32_t*)(blk + o_to);
+        s->d_terms = (uint32_t*)(blk + o_te);
+      }
+      e = cudaMemcpy(blk, host.data(), host.size(), cudaMemcpyHostToDevice);
     }
     if (e != cudaSuccess) {
       cudaGetLastError();

@@ -559,8 +559,8 @@ __device__ __forceinline__ cx<L> cx_from(const double* re, const double* im) {
 // per-output fixed-point frames), the rest of the round in FP64 arithmetic.
 // MAXT: the largest team (8, or 16 for the wide instantiation that serves
 // few groups of double and double-double paths with more warps each, and
-// any group when the autotuner picks 16).
-template <int L, bool LEARN, bool INT, int MAXT = INT ? 16 : 8>
+// any group when the autotuner picks 16; track_int_warps on the integer pipe).
+template <int L, bool LEARN, bool INT, int MAXT = INT ? track_int_warps(L) : 8>
 __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 4 : (L == 2 ? 2 : 1))) track_kernel(TrackArgs a) {
   __shared__ double red[4][MAXT][32];  // per-warp partials: residual, update, point norms; finiteness
   __shared__ double sh_h[32];       // learned step of each lane's path

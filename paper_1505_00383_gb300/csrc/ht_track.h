@@ -91,6 +91,11 @@ struct TrackArgs {
   double alpha_max;        // learned tangent correction clamp (0: off)
 };
 
+// Warps of an int_eval CTA (one CTA an SM).  They deal a group's polynomials
+// and systems, so more help until the registers spill: QD with 12 warps of 168
+// registers against 16 of 128: n = 10, 4,096 paths 597 -> 570 ms.
+constexpr int track_int_warps(int L) { return L == 4 ? 12 : 16; }
+
 // CTAs of an int_eval launch over at most `groups` groups of paths, and the
 // bytes of the workspace A of each for an L-limb system in n variables.
 int64_t track_int_ctas(int64_t groups);

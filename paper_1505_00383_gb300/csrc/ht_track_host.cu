@@ -418,26 +418,28 @@ int ht_track_paths_ex(ht_system* s, const int32_t* start_deg, const double* gamm
   // read of the active count, captured once per team size as a CUDA graph.
   const int iters = P.iters_per_launch > 0 ? P.iters_per_launch : (s->track_iters > 0 ? s->track_iters : 4);
   const int rounds = P.rounds_per_sync > 0 ? P.rounds_per_sync : 8;
-  // Team size: the largest power of two up to 8 warps and n.  More warps per
-  // group means fewer groups in flight for the same FP64 issue rate, so the
-  // per-path workspace (A and R, 2 n (n + 1) complex entries per path) of the
-  // resident groups stays in L2; on the n = 16 double workload 8 warps beat 1
-  // warp by 1.7x and 4 warps by 4 %.
-  // While fewer groups are active than there are SMs (a small batch, or the
-  // tail of any run), a double or double-double group with more than 8 MGS
-  // columns gets 16 warps: every SM then runs at most one group, and the
-  // wider team shortens that group's round (fewer columns and polynomials per
-  // warp).  QD (200+ registers a thread) keeps 8.
+  // Team size in double: the largest power of two up to 8 warps and n.  More
+  // warps per group means fewer groups in flight for the same FP64 issue rate,
+  // so the per-path workspace (A and R, 2 n (n + 1) complex entries per path) of
+  // the resident groups stays in L2; on the n = 16 double workload 8 warps beat
+  // 1 warp by 1.7x and 4 warps by 4 %.  While few paths are active (a column
+  // per lane in the least squares) a warp per polynomial; while fewer groups
+  // are active than there are SMs, a double group with more than 8 columns
+  // gets 16 warps (every SM then runs at most one group).  On the integer pipe
+  // always the kernel's most (track_int_warps).
   const bool wide_ok = L <= 2 && n + 1 > 8;
   auto pick_team = [&](int64_t active) {
-    if (P.team_warps > 0) return P.team_warps;
+    // QD accepts teams of up to 8; on the integer pipe the widest is the
+    // kernel's 12 warps
+    const int widest = int_eval && L == 4 ? track_int_warps(L) : 8;
+    if (P.team_warps > 0) return P.team_warps == 8 ? widest : P.team_warps;
     int t = 1;
     if (s->track_team > 0 && s->track_team <= 16) {
-      t = s->track_team;
+      t = s->track_team == 8 ? widest : s->track_team;
     } else if (L == 1 && active <= track_col_paths(n, nrhs)) {
       return std::max(4, std::min(16, n));  // a warp per polynomial, four at least for the solve
     } else if (int_eval) {
-      return 16;  // the rows of the systems, and in small groups their columns, spread over all
+      return track_int_warps(L);  // the rows of the systems, and in small groups their columns, spread over all
     } else {
       while (t < 8 && 2 * t <= n) t *= 2;
     }
