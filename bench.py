@@ -184,7 +184,7 @@ def _traffic(L):
 def _track_sha():
     h = hashlib.sha256()
     for f in ("ht_track.cu", "ht_track.h", "ht_eval.cuh", "ht_int_row.cuh", "ht_mp.cuh", "ht_mpi.cuh", "ht_mpi_eval.cuh",
-              "ht_mpi_ops.cuh", "ht_mlp.cuh"):
+              "ht_mpi_ops.cuh", "ht_mlp.cuh", "ht_int_mgs.cuh", "ht_col_mgs.cuh"):
         h.update(open(os.path.join(ROOT, "paper_1505_00383_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 

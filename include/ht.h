@@ -165,8 +165,8 @@ int ht_eval_diff_unfused(ht_system* sys, int64_t n_pts, const double* x, double*
  *            variant 2, 128 (or 0, 64) runs one unit of 32 points and one
  *            polynomial per warp with the lane's point in local memory, and
  *            256 runs work items of 32 points and a group of polynomials per
- *            CTA (one polynomial per warp: 16-warp CTAs for systems of at
- *            least 16 polynomials, else 8) with the points in shared memory
+ *            CTA (one polynomial per warp, or with few points a polynomial's
+ *            monomials over several warps) with the points in shared memory
  *            (the same bits either way)
  * Variants 0, 1 and 3 perform the same operations in the same order, so their
  * results are bitwise identical; variant 2 meets the same accuracy bound
@@ -321,7 +321,8 @@ int ht_mgs_solve(int limbs, int rows, int cols, int64_t n_sys, double* Ab, doubl
  *              as a radix-2^29 limb string, every dot product and norm is one
  *              exact fixed-point sum of its products rounded once, 1/r_qq
  *              comes from Newton's iteration for 1/sqrt; results are written
- *              back as doubles (the leading 53-bit pieces of each value).
+ *              back as doubles (the leading 53-bit pieces of each value), at
+ *              the end for up to 32 rows and after every column for more.
  * The tracker uses variant 2 for QD systems unless ht_set_eval_config chose
  * an FP64 variant.  Errors as ht_mgs_solve; HT_EUNSUPPORTED for
  * variant 2 with limbs 1 or more than 64 rows.

@@ -28,6 +28,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <mutex>
 
 #include "ht_eval.cuh"
 #include "ht_internal.h"
@@ -431,9 +432,12 @@ __global__ void __launch_bounds__(512, 1) evaldiff_intsplit_kernel(EvalArgs a, I
 }
 
 // Raise a kernel's dynamic shared-memory limit (per device) only when a larger
-// system needs more, not on every launch.
+// system needs more, not on every launch; one thread at a time, so that the
+// limit never falls.
 template <class K>
 static void raise_smem(K kern, size_t smem, size_t* set) {
+  static std::mutex lock;
+  std::lock_guard<std::mutex> guard(lock);
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64 || smem > set[dev]) {

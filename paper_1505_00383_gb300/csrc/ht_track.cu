@@ -1,15 +1,20 @@
 // Many-path predictor-corrector tracking of gamma (1 - t) g(x) + t f(x) = 0
 // (Section 2 of Verschelde & Yu 2015), with g_i = x_i^d_i - 1.
 //
-// Execution model.  A CTA serves a group of 32 paths (one per lane) with T
-// warps; warp r is "team member" r for all 32 paths.  Every warp executes the
-// same instruction stream for its 32 paths (the SIMT picture of Table
-// tabsimtprecor), and the work of one Newton step is split over the T warps:
+// Execution model.  A CTA serves a group of up to 32 paths (one per lane) with
+// T warps.  Every warp executes the same instruction stream for the group's
+// paths (the SIMT picture of Table tabsimtprecor), and the work of one Newton
+// step is split over the T warps:
 //   * evaluation: warp r evaluates the polynomials j = r, r + T, ...;
-//   * modified Gram-Schmidt: warp r owns the columns j = r, r + T, ... of the
-//     augmented matrix [J | -h]; the owner of column q normalises it, then
-//     every warp projects its later columns (no cross-warp reductions: each
-//     dot product runs down a whole column in one warp);
+//   * least squares, by one of three layouts with the same operations and bits
+//     per arithmetic:
+//     - double, many paths (mgs_team): a system per lane; the columns of the
+//       augmented matrix [J | -h] are dealt to the warps, whose barrier is per
+//       column; the FP64 pipe is the limit and every lane of it is used;
+//     - double, few paths (ht_col_mgs.cuh): a column per lane, the systems
+//       dealt to the warps; a group is then active / SMs paths;
+//     - DD and QD on the integer pipe (ht_int_mgs.cuh): a row per lane, the
+//       systems dealt to the warps; groups likewise;
 //   * prediction and the Newton update: warp r owns coordinates r, r + T, ...
 // One kernel launch runs `iters` Newton steps of every path of its groups; a
 // path's step (predict, 1..newton_max evaluate-correct rounds, accept or
@@ -366,12 +371,12 @@ __device__ void mgs_team(double* A, double* R, double* x, int rows, int cols, in
   __syncthreads();
 }
 
-// The same least squares on the integer pipe (DD, QD): entries are read as
-// limb strings (from stored limb strings, or by exact conversion of stored
-// doubles), every dot product and norm is one exact fixed-point sum of its
-// products rounded once, 1/r_qq comes from Newton's iteration for 1/sqrt, and
-// results are stored back in the same form; the solution is stored as
-// doubles.  The column owner loads and normalises column q; the other warps
+// The same least squares on the integer pipe for more than 32 rows
+// (ht_mgs_solve_ex; up to 32 rows take the row layout of ht_int_mgs.cuh):
+// entries are limb strings by exact conversion of the stored doubles, every
+// dot product and norm is one exact fixed-point sum of its products rounded
+// once, 1/r_qq comes from Newton's iteration for 1/sqrt, and results are
+// stored back as doubles.  The column owner loads and normalises column q; the other warps
 // reload it after the barrier.  Layouts and R's diagonal (1/r_qq) as above.
 template <int L>
 __device__ __forceinline__ mpi::fz<IntW<L>::W> ldz(const double* base, int64_t e, int64_t m, int64_t p) {
@@ -442,8 +447,7 @@ __device__ void mgs_team_int(const ST& A, const ST& R, double* x, int rows, int 
         for (int i = 0; i < rows; ++i) A.st((int64_t)i * Wc + j, col[i]);
         if (j == q + 1 && j < cols) {
           // the pivot column from its stored values, as the owner's reload
-          // would give (for stored doubles the limb strings of the doubles
-          // just written; stored limb strings come back as they were)
+          // would give (the limb strings of the doubles just written)
           for (int i = 0; i < rows; ++i) col[i] = A.ld((int64_t)i * Wc + j);
           normalise(j, col);
         }
@@ -1053,7 +1057,8 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 4 : (L == 
           const unsigned live = __ballot_sync(0xffffffffu, act);
           const int per = ColLanes::systems(n, nrhs), chunks = (G + per - 1) / per;
           double2* sh = reinterpret_cast<double2*>(xs_int) + warp * ColLanes::words(n, nrhs);
-          for (int c = warp; c < chunks; c += T) {  // at most ColLanes::WARPS chunks
+          // (the host keeps the chunks to ColLanes::WARPS, the warps with a buffer)
+          for (int c = warp; warp < ColLanes::WARPS && c < chunks; c += min(T, ColLanes::WARPS)) {
             const int pl = c * per + min(lane / ColLanes::lanes(n, nrhs), per - 1);
             const int64_t ps = __shfl_sync(0xffffffffu, (int)p, min(pl, 31));
             ColLanes::solve_any(
