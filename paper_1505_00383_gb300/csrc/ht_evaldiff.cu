@@ -229,9 +229,8 @@ static int launch_v(const EvalArgs& a, int threads, cudaStream_t st) {
 //   2. bounds every term of polynomial j -- log2|c| + sum a log2|x| for the
 //      value, minus log2|x_v| plus log2 a_v for a derivative -- and fixes one
 //      accumulator frame above the largest bound plus log2 of the term count;
-//   3. accumulates value and Jacobian row as fixed-point limbs: the row lives
-//      in place in the output (2L doubles hold exactly 2 x 2L int32 limbs);
-//   4. converts the accumulators to L doubles.
+//   3. accumulates value and Jacobian row as fixed-point limbs in local memory;
+//   4. converts the accumulators to L doubles and writes the outputs.
 template <int L>
 __global__ void __launch_bounds__(128, 4) evaldiff_int_kernel(EvalArgs a, IntPoly ip,
                                                            const mpi::fz<IntW<L>::W>* __restrict__ cfz) {
@@ -514,7 +513,7 @@ static int launch_int(const EvalArgs& a, const ht_system* s, int threads, cudaSt
 // A cluster of C CTAs per unit: the largest of 1, 2, 4, 8 that the SMs and
 // the monomials have room for (10 points, the call: 10 polynomials of 10
 // monomials 77 us on one warp each, 30 us with C = 1, 25 us with 4; 16 of 246
-// monomials 709, 205 and, with 8, 105 us).  Returns false if the system needs
+// monomials 709, 205 and, with 8, 71 us).  Returns false if the system needs
 // more shared memory.
 static bool launch_split(const EvalArgs& a, const ht_system* s, cudaStream_t st, int* rc) {
   const int64_t sms = sm_count();

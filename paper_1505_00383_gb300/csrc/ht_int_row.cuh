@@ -1,8 +1,8 @@
 // One polynomial's value and gradient row on the integer pipe, for one point
-// per lane (device only): the per-output frames, the reverse-mode sweep of
-// ht_mpi_eval.cuh with the row's fixed-point accumulators in place in the
-// caller's output row, and the conversion of every output to L doubles.  The
-// evaluation kernel and the tracker both call it.
+// per lane (device only): the per-output frames, the sweep's steps of
+// ht_mpi_eval.cuh with the row's fixed-point accumulators in local memory, and
+// the conversion of every output to L doubles.  The evaluation kernels and the
+// tracker both use it.
 #pragma once
 #include "ht_mpi_eval.cuh"
 #include "ht_mpi_ops.cuh"
