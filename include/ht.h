@@ -171,7 +171,9 @@ int ht_eval_diff_unfused(ht_system* sys, int64_t n_pts, const double* x, double*
  * Variants 0, 1 and 3 perform the same operations in the same order, so their
  * results are bitwise identical; variant 2 meets the same accuracy bound
  * (a small multiple of 2^(-53 L) times the sum of the moduli of the terms of
- * each output) with its own rounding.
+ * each output) with its own rounding.  In DD its sums hold 115 bits, which
+ * limits an output of n terms to about n^2 2^-112 of its largest term (n =
+ * 246: 2^-96).
  * The choice also applies inside ht_track_paths for DD and QD systems with
  * n <= 32: by default (and with variant 2) the tracker runs its Newton round
  * on the integer pipe: f and its Jacobian rows, the homotopy terms and the

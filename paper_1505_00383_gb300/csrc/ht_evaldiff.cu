@@ -279,9 +279,9 @@ __device__ __forceinline__ void stage_points(const double* __restrict__ x, int n
 template <int L>
 constexpr int kBlkWarps = L == 4 ? 16 : 32;
 // Row slots that pass through shared memory at a time in the split kernel
-// (2 KB a warp).
+// (4 KB a warp).
 template <int L>
-constexpr int kSplitSlots = 8 / L;
+constexpr int kSplitSlots = 8 / RowAcc<L>::Q;
 
 // Block organisation of the same unit: a CTA takes a block of 32 points and
 // a group of polynomials (as many as it has warps: one each).  The block's
@@ -404,9 +404,9 @@ __global__ void __launch_bounds__(512, 1) evaldiff_intsplit_kernel(EvalArgs a, I
       for (int r = s; r < R; r += S) {
         const int i = i0 + r;
         if (!work || i >= n_slots || p >= n) continue;
-        int64_t c[2 * WA];
+        int64_t c[4 * Q];
 #pragma unroll
-        for (int k = 0; k < 2 * WA; ++k) c[k] = 0;
+        for (int k = 0; k < 4 * Q; ++k) c[k] = 0;
         for (int q = 0; q < S; ++q)
 #pragma unroll
           for (int k = 0; k < Q; ++k) {
@@ -472,7 +472,7 @@ static int launch_int(const EvalArgs& a, const ht_system* s, int threads, cudaSt
       }
     }
     const size_t smem_split = xbytes + (size_t)(S * G) * 32 *
-                                           std::max<size_t>((a.nv + 1) * sizeof(float), kSplitSlots<L> * 2 * IntW<L>::WA * 4);
+                                           std::max<size_t>((a.nv + 1) * sizeof(float), kSplitSlots<L> * RowAcc<L>::Q * sizeof(int4));
     if (S > 1 && smem_split <= 220 * 1024) {
       static size_t set[64] = {0};
       raise_smem(evaldiff_intsplit_kernel<L>, smem_split, set);

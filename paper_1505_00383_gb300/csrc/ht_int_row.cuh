@@ -14,10 +14,10 @@ constexpr int kIntMaxVars = 64;
 
 // The fixed-point accumulators of one polynomial's outputs at the lane's
 // point: slot i the derivative by x_i, slot nv the value, each 2 WA limbs
-// (re, im) in local memory, moved in 128-bit words.
+// (re, im) in local memory, moved in 128-bit words (padded to whole ones).
 template <int L>
 struct RowAcc {
-  static constexpr int W = IntW<L>::W, WA = IntW<L>::WA, Q = WA / 2;  // int4 words per slot
+  static constexpr int W = IntW<L>::W, WA = IntW<L>::WA, Q = (2 * WA + 3) / 4;  // int4 words per slot
   int4* a;        // [(nv + 1) Q]
   const int* Fv;  // frames of the slots
   int nv;
@@ -27,7 +27,7 @@ struct RowAcc {
     for (int k = 0; k < Q; ++k) a[i * Q + k] = make_int4(0, 0, 0, 0);
   }
   __device__ __forceinline__ void load(int i, int32_t* ar, int32_t* ai) const {
-    int32_t w[2 * WA];
+    int32_t w[4 * Q];
 #pragma unroll
     for (int k = 0; k < Q; ++k) {
       const int4 q = a[i * Q + k];
@@ -47,12 +47,14 @@ struct RowAcc {
     int32_t ar[WA], ai[WA];
     load(i, ar, ai);
     mpi::acc_add_fast<W, WA>(ar, ai, d, e, Fv[i]);
-    int32_t w[2 * WA];
+    int32_t w[4 * Q];
 #pragma unroll
     for (int k = 0; k < WA; ++k) {
       w[k] = ar[k];
       w[WA + k] = ai[k];
     }
+#pragma unroll
+    for (int k = 2 * WA; k < 4 * Q; ++k) w[k] = 0;
 #pragma unroll
     for (int k = 0; k < Q; ++k) a[i * Q + k] = make_int4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
   }
