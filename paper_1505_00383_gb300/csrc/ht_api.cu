@@ -3,6 +3,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 
 #include <cmath>
@@ -58,6 +59,31 @@ int sm_count() {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
   return n > 0 ? n : 1;
+}
+
+void raise_smem(const void* kernel, size_t bytes) {
+  // limits set so far; kernels or devices past the table's end ask the driver
+  constexpr int KERNELS = 32, DEVICES = 64;
+  static std::mutex lock;
+  static const void* known[KERNELS];
+  static size_t limit[KERNELS][DEVICES];
+  int dev = 0, k = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> guard(lock);
+  while (k < KERNELS && known[k] && known[k] != kernel) ++k;
+  const bool kept = k < KERNELS && dev >= 0 && dev < DEVICES;
+  size_t now = 0;
+  if (kept) {
+    known[k] = kernel;
+    now = limit[k][dev];
+  } else {
+    cudaFuncAttributes at;
+    if (cudaFuncGetAttributes(&at, kernel) == cudaSuccess) now = (size_t)at.maxDynamicSharedSizeBytes;
+  }
+  if (bytes <= now) return;
+  // (a refused limit surfaces in the launch)
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess && kept)
+    limit[k][dev] = bytes;
 }
 
 }  // namespace ht

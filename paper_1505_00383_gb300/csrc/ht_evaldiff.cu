@@ -28,7 +28,6 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "ht_eval.cuh"
 #include "ht_internal.h"
@@ -430,21 +429,6 @@ __global__ void __launch_bounds__(512, 1) evaldiff_intsplit_kernel(EvalArgs a, I
   }
 }
 
-// Raise a kernel's dynamic shared-memory limit (per device) only when a larger
-// system needs more, not on every launch; one thread at a time, so that the
-// limit never falls.
-template <class K>
-static void raise_smem(K kern, size_t smem, size_t* set) {
-  static std::mutex lock;
-  std::lock_guard<std::mutex> guard(lock);
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64 || smem > set[dev]) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (dev >= 0 && dev < 64) set[dev] = smem;
-  }
-}
-
 template <int L>
 static int launch_int(const EvalArgs& a, const ht_system* s, int threads, cudaStream_t st) {
   const auto* cf = reinterpret_cast<const mpi::fz<IntW<L>::W>*>(s->d_coef_fz);
@@ -474,8 +458,7 @@ static int launch_int(const EvalArgs& a, const ht_system* s, int threads, cudaSt
     const size_t smem_split = xbytes + (size_t)(S * G) * 32 *
                                            std::max<size_t>((a.nv + 1) * sizeof(float), kSplitSlots<L> * RowAcc<L>::Q * sizeof(int4));
     if (S > 1 && smem_split <= 220 * 1024) {
-      static size_t set[64] = {0};
-      raise_smem(evaldiff_intsplit_kernel<L>, smem_split, set);
+      raise_smem((const void*)evaldiff_intsplit_kernel<L>, smem_split);
       int per_sm = 0;
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, evaldiff_intsplit_kernel<L>, 32 * S * G, smem_split);
       if (per_sm < 1) per_sm = 1;
@@ -486,8 +469,7 @@ static int launch_int(const EvalArgs& a, const ht_system* s, int threads, cudaSt
       // as few groups of polynomials as the largest CTA allows, of equal size
       const int groups = (a.np + kBlkWarps<L> - 1) / kBlkWarps<L>;
       const int cta = 32 * ((a.np + groups - 1) / groups);
-      static size_t set[64] = {0};
-      raise_smem(evaldiff_intblk_kernel<L>, xbytes, set);
+      raise_smem((const void*)evaldiff_intblk_kernel<L>, xbytes);
       int per_sm = 0;
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, evaldiff_intblk_kernel<L>, cta, xbytes);
       if (per_sm < 1) per_sm = 1;
@@ -523,8 +505,7 @@ static bool launch_split(const EvalArgs& a, const ht_system* s, cudaStream_t st,
   const int n_slots = std::min(192, (s->max_slots + C - 1) / C + s->max_k);
   const size_t smem = split_smem(a.nv, n_slots);
   if (smem > 220 * 1024) return false;
-  static size_t set[64] = {0};
-  raise_smem(evaldiff_split_kernel, smem, set);
+  raise_smem((const void*)evaldiff_split_kernel, smem);
   // 16 warps, fewer when a part has fewer monomials and outputs
   const int warps = std::max(1, std::min(16, std::max(a.max_terms, a.nv + 1)));
   int per_sm = 0;

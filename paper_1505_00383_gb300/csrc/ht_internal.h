@@ -69,6 +69,11 @@ void clear_error();
 // True when p is device (or managed) memory of the current device.
 bool is_device_ptr(const void* p);
 int sm_count();
+// Let a kernel's launches on the current device use `bytes` of dynamic shared
+// memory.  The limit belongs to the kernel, which any thread may launch for
+// systems of any size, so it is only ever raised, under a lock: a smaller
+// request between another thread's request and its launch must not lower it.
+void raise_smem(const void* kernel, size_t bytes);
 
 // Polynomials j0 .. j1 - 1 at n_pts points: val and jac receive them from
 // their row 0 (val [j1 - j0][2][L][n_pts], jac [j1 - j0][nv][2][L][n_pts]).

@@ -310,11 +310,7 @@ __global__ void mlp_to_bf16_kernel(const float* __restrict__ w, __nv_bfloat16* _
 
 static int mlp_fwd_launch(const ht_mlp* net, int64_t B, const float* x, float* y, cudaStream_t st) {
   const size_t smem = sizeof(MlpFwdSmem);
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(mlp_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr_set = true;
-  }
+  raise_smem((const void*)mlp_forward_kernel, smem);
   int64_t warps = (B + 31) / 32;
   int64_t grid = (warps + 3) / 4;
   int64_t cap = (int64_t)sm_count() * 8;
@@ -370,11 +366,7 @@ static int mlp_grad_batch(ht_mlp* net, int64_t B, const float* x, const float* t
                           float* loss, const AdamStep* adam, cudaStream_t st) {
   const int64_t C = (B + kBwdChunk - 1) / kBwdChunk;
   const size_t smem = sizeof(MlpBwdSmem);
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(mlp_backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr_set = true;
-  }
+  raise_smem((const void*)mlp_backward_kernel, smem);
   mlp_backward_kernel<<<(unsigned)C, kBwdThreads, smem, st>>>(net->wbf, net->master, B, x, target, part, lpart);
   const unsigned blocks = (MLP_NPARAM + 1 + 127) / 128;
   if (adam)

@@ -1347,7 +1347,7 @@ int launch_track_l(const TrackArgs& a, int team, int64_t max_groups, cudaStream_
   auto go = [&](auto kern, size_t dsm) {
     // the kernel's static shared memory counts against the same 48 KB default,
     // so the limit is raised for any dynamic size (n = 32 DD asks for 48 KB)
-    if (dsm > 0) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm);
+    if (dsm > 0) raise_smem((const void*)kern, dsm);
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * team, dsm);
     if (per_sm < 1) per_sm = 1;
