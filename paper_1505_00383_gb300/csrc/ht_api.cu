@@ -214,6 +214,13 @@ int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8
         mpi::sweep_steps(s->h_pairs.data() + s->h_mon_off[m], s->h_mon_off[m + 1] - s->h_mon_off[m], steps);
         step_off.push_back((int32_t)steps.size());
       }
+      s->shape.nv = n_vars;
+      s->shape.np = n_polys;
+      s->shape.max_terms = s->max_terms;
+      s->shape.mean_steps = (double)steps.size() / n_polys;
+      for (int j = 0; j < n_polys; ++j)
+        s->shape.max_steps =
+            std::max<int64_t>(s->shape.max_steps, step_off[s->h_poly_off[j + 1]] - step_off[s->h_poly_off[j]]);
     }
     // double: the terms of every output
     std::vector<uint32_t> terms;

@@ -436,25 +436,10 @@ static int launch_int(const EvalArgs& a, const ht_system* s, int threads, cudaSt
   if (threads == 256) {  // block organisation (points in shared memory)
     const int64_t n_blocks = (a.v.npts + 31) / 32, sms = sm_count();
     const size_t xbytes = smem_points_bytes<L>(a.nv);
-    // Warps per polynomial: with up to 16 warps a CTA takes G polynomials on S
-    // warps each.  Of all S the one with the least time is taken, in units of
-    // one warp's pass over a polynomial: waves of CTAs over the SMs times 1/S,
-    // plus 1/20 a wave for the bounds' and slots' exchange.  A large batch
-    // has many waves whatever S, so it stays unsplit; at 999 points of the
-    // 16-polynomial system S = 4 fills the chip in one wave, and at 3,000
-    // points S = 8 cuts the last wave's idle part (4.4 -> 3.0 ms in QD).
-    int S = 1, G = 1;
-    double best = 1e300;
-    for (int c = 1; c <= 16 && c <= a.max_terms; ++c) {
-      const int most = std::min(a.np, 16 / c), groups = (a.np + most - 1) / most, g = (a.np + groups - 1) / groups;
-      const int64_t slots = sms * (16 / (c * g));
-      const double t = (double)((n_blocks * groups + slots - 1) / slots) * (1.0 / c + (c > 1 ? 0.05 : 0.0));
-      if (t < best * 0.98) {
-        best = t;
-        S = c;
-        G = g;
-      }
-    }
+    EvalShape shape = s->shape;
+    shape.np = a.np;  // of this range of polynomials
+    const EvalSplit split = eval_split(shape, L, n_blocks, sms);
+    const int S = split.S, G = split.G;
     const size_t smem_split = xbytes + (size_t)(S * G) * 32 *
                                            std::max<size_t>((a.nv + 1) * sizeof(float), kSplitSlots<L> * RowAcc<L>::Q * sizeof(int4));
     if (S > 1 && smem_split <= 220 * 1024) {

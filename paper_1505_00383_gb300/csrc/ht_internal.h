@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "ht.h"
+#include "ht_split.h"
 
 // The "instructions" of Table tabmemory: monomial supports and coefficients,
 // stored once on the device and read by all paths.
@@ -13,6 +14,7 @@ struct ht_system {
   int nv = 0, np = 0, limbs = 0, device = 0;
   int64_t M = 0, n_pairs = 0;
   int max_k = 0, max_exp = 0, max_deg = 0, max_terms = 0;
+  ht::EvalShape shape;           // sizes the integer evaluation's split depends on
   int eval_variant = -1;         // 0 unrolled, 1 compact FP64 bodies, 2 integer limbs, -1 default
   int eval_threads = 0;          // CTA size of the evaluation kernel, 0 = default (128)
   int track_team = 0;            // tuned tracker team size and rounds per launch (0: defaults)

@@ -1,0 +1,24 @@
+// Host build of the integer evaluation's split rule (csrc/ht_split.h).
+#include "../paper_1505_00383_gb300/csrc/ht_mpi_eval.cuh"
+#include "../paper_1505_00383_gb300/csrc/ht_split.h"
+
+extern "C" {
+
+int64_t split_steps(const uint16_t* pairs, int k) {
+  std::vector<uint32_t> st;
+  ht::mpi::sweep_steps(pairs, k, st);
+  return (int64_t)st.size();
+}
+
+int split_pick(int nv, int np, int max_terms, int64_t max_steps, double mean_steps, int limbs, int64_t n_blocks,
+               int64_t sms) {
+  ht::EvalShape e;
+  e.nv = nv;
+  e.np = np;
+  e.max_terms = max_terms;
+  e.max_steps = max_steps;
+  e.mean_steps = mean_steps;
+  const ht::EvalSplit s = ht::eval_split(e, limbs, n_blocks, sms);
+  return s.S * 100 + s.G;
+}
+}
