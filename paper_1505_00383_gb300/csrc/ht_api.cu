@@ -105,8 +105,8 @@ int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8
   if (!n_terms || !exps || !coef) return set_error(HT_EINVAL, "ht_create_system: NULL array");
   ht_system* s = new (std::nothrow) ht_system();
   if (!s) return set_error(HT_ENOMEM, "ht_create_system: host allocation");
-  s->nv = n_vars;
-  s->np = n_polys;
+  s->nv = s->shape.nv = n_vars;
+  s->np = s->shape.np = n_polys;
   s->limbs = limbs;
   cudaGetDevice(&s->device);
   s->h_poly_off.assign(n_polys + 1, 0);
@@ -116,7 +116,7 @@ int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8
       return set_error(HT_EINVAL, "ht_create_system: n_terms[%d]=%d < 1", j, n_terms[j]);
     }
     s->h_poly_off[j + 1] = s->h_poly_off[j] + n_terms[j];
-    if (n_terms[j] > s->max_terms) s->max_terms = n_terms[j];
+    s->shape.max_terms = std::max(s->shape.max_terms, (int)n_terms[j]);
   }
   s->M = s->h_poly_off[n_polys];
   s->n_terms.assign(n_terms, n_terms + n_polys);
@@ -214,9 +214,6 @@ int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8
         mpi::sweep_steps(s->h_pairs.data() + s->h_mon_off[m], s->h_mon_off[m + 1] - s->h_mon_off[m], steps);
         step_off.push_back((int32_t)steps.size());
       }
-      s->shape.nv = n_vars;
-      s->shape.np = n_polys;
-      s->shape.max_terms = s->max_terms;
       s->shape.mean_steps = (double)steps.size() / n_polys;
       for (int j = 0; j < n_polys; ++j)
         s->shape.max_steps =
@@ -225,12 +222,23 @@ int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8
     // double: the terms of every output
     std::vector<uint32_t> terms;
     std::vector<int32_t> term_off;
+    int64_t products = 0;
     for (int j = 0; j < n_polys; ++j) {
       const int64_t b = s->h_poly_off[j], e2 = s->h_poly_off[j + 1];
-      const int64_t slots = (e2 - b) + s->h_mon_off[e2] - s->h_mon_off[b];
-      s->max_slots = (int)std::max<int64_t>(s->max_slots, std::min<int64_t>(slots, 1 << 30));
+      int64_t slots = 0, prod = 0;  // a value and k derivatives; x^(a-1) factors and 3 k - 3 products of the sweep
+      for (int64_t m = b; m < e2; ++m) {
+        const int k = s->h_mon_off[m + 1] - s->h_mon_off[m];
+        slots += k + 1;
+        prod += k >= 2 ? 3 * k - 3 : k;
+        for (int32_t r = s->h_mon_off[m]; r < s->h_mon_off[m + 1]; ++r) prod += (s->h_pairs[r] >> 8) - 1;
+      }
+      s->shape.max_slots = std::max(s->shape.max_slots, slots);
+      s->shape.max_products = std::max(s->shape.max_products, prod);
+      products += prod;
     }
-    if (limbs == 1 && s->max_slots < (1 << 24) && s->n_pairs + s->M < (1LL << 31)) {
+    s->shape.mean_slots = (double)(s->n_pairs + s->M) / n_polys;
+    s->shape.mean_products = (double)products / n_polys;
+    if (limbs == 1 && s->shape.max_slots < (1 << 24) && s->n_pairs + s->M < (1LL << 31)) {
       std::vector<std::vector<uint32_t>> of(n_vars + 1);
       terms.reserve(s->n_pairs + s->M);
       term_off.reserve((size_t)n_polys * (n_vars + 1) + 1);

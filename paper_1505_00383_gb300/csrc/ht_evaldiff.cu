@@ -43,7 +43,6 @@ struct EvalArgs {
   double* val;
   double* jac;
   int64_t n_units;
-  int max_terms;  // largest number of monomials of a polynomial
 };
 
 template <int L, bool LOOP>
@@ -480,19 +479,23 @@ static int launch_int(const EvalArgs& a, const ht_system* s, int threads, cudaSt
 // A cluster of C CTAs per unit: the largest of 1, 2, 4, 8 that the SMs and
 // the monomials have room for (10 points, the call: 10 polynomials of 10
 // monomials 77 us on one warp each, 30 us with C = 1, 25 us with 4; 16 of 246
-// monomials 709, 205 and, with 8, 71 us).  Returns false if the system needs
-// more shared memory.
+// monomials 709, 205 and, with 8, 71 us).  Returns false where one warp per
+// unit is faster, or if the system needs more shared memory.
 static bool launch_split(const EvalArgs& a, const ht_system* s, cudaStream_t st, int* rc) {
-  const int64_t sms = sm_count();
+  const int64_t sms = sm_count(), max_terms = s->shape.max_terms, max_slots = s->shape.max_slots;
   int C = 8;
-  while (C > 1 && (a.n_units * C > sms || C * 2 > a.max_terms)) C /= 2;
+  while (C > 1 && (a.n_units * C > sms || C * 2 > max_terms)) C /= 2;
+  // 16 warps, fewer when a part has fewer monomials and outputs
+  const int warps = (int)std::max<int64_t>(1, std::min<int64_t>(16, std::max<int64_t>(max_terms, a.nv + 1)));
   // slots for a CTA's part of a polynomial, up to 96 KB of them (two CTAs a SM)
-  const int n_slots = std::min(192, (s->max_slots + C - 1) / C + s->max_k);
+  const int n_slots = (int)std::min<int64_t>(192, (max_slots + C - 1) / C + s->max_k);
   const size_t smem = split_smem(a.nv, n_slots);
   if (smem > 220 * 1024) return false;
+  if (C == 1) {
+    const int64_t q = std::min<int64_t>(max_slots, n_slots - s->max_k);  // a chunk, as the kernel cuts it
+    if (!double_split_pays(s->shape, a.n_units, sms, warps, (max_slots + q - 1) / q)) return false;
+  }
   raise_smem((const void*)evaldiff_split_kernel, smem);
-  // 16 warps, fewer when a part has fewer monomials and outputs
-  const int warps = std::max(1, std::min(16, std::max(a.max_terms, a.nv + 1)));
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, evaldiff_split_kernel, 32 * warps, smem);
   if (per_sm < 1) per_sm = 1;
@@ -531,16 +534,12 @@ int launch_evaldiff_l(const ht_system* s, int64_t n_pts, int j0, int j1, const d
   a.val = val;
   a.jac = jac;
   a.n_units = ((n_pts + 31) / 32) * a.np;
-  a.max_terms = s->max_terms;
   const int threads = s->eval_threads > 0 ? s->eval_threads : 128;
   if (s->eval_variant == 2 && s->d_steps && s->nv <= kIntMaxVars && s->max_k <= 64)
     return launch_int<L>(a, s, threads, st);
   const bool loop = s->eval_variant != 0;  // default: compact bodies
 #if HT_LIMBS == 1
-  // few units: two per SM sub-partition is where one warp per polynomial
-  // catches up (nash8 shape: 0.39 -> 0.18 ms at 1,000 points, 0.50 and 0.49
-  // ms at 3,000)
-  if (loop && s->d_terms && a.n_units <= 8 * (int64_t)sm_count()) {
+  if (loop && s->d_terms) {  // few units: polynomials over the warps of a CTA or cluster
     int rc;
     if (launch_split(a, s, st, &rc)) return rc;
   }

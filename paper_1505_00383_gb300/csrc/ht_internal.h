@@ -13,8 +13,8 @@
 struct ht_system {
   int nv = 0, np = 0, limbs = 0, device = 0;
   int64_t M = 0, n_pairs = 0;
-  int max_k = 0, max_exp = 0, max_deg = 0, max_terms = 0;
-  ht::EvalShape shape;           // sizes the integer evaluation's split depends on
+  int max_k = 0, max_exp = 0, max_deg = 0;
+  ht::EvalShape shape;           // sizes the evaluation's splits depend on
   int eval_variant = -1;         // 0 unrolled, 1 compact FP64 bodies, 2 integer limbs, -1 default
   int eval_threads = 0;          // CTA size of the evaluation kernel, 0 = default (128)
   int track_team = 0;            // tuned tracker team size and rounds per launch (0: defaults)
@@ -38,7 +38,6 @@ struct ht_system {
   // of the polynomial (a monomial's value, then its derivatives) | exponent << 24
   int32_t* d_term_off = nullptr; // [np (nv + 1) + 1]
   uint32_t* d_terms = nullptr;   // NULL for a polynomial of 2^24 slots and more
-  int max_slots = 0;             // largest number of slots of a polynomial
   void* d_ws = nullptr;          // workspace for the host-buffer entry points
   size_t ws_bytes = 0;
   cudaStream_t host_streams[2] = {nullptr, nullptr};  // pipelined host-buffer evaluation

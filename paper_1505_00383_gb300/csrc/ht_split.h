@@ -1,5 +1,5 @@
-// How many warps share a polynomial in the integer evaluation (host only,
-// plain C++ so that the host tests can build it).
+// How many warps share a polynomial in the evaluation (host only, plain C++ so
+// that the host tests can build it).
 #pragma once
 #include <algorithm>
 #include <cmath>
@@ -13,6 +13,9 @@ struct EvalShape {
   int max_terms = 0;      // monomials of the longest polynomial
   int64_t max_steps = 0;  // sweep steps of the longest polynomial
   double mean_steps = 0;  // and of an average one
+  // double: complex products of the sweep, and terms of all outputs
+  int64_t max_products = 0, max_slots = 0;
+  double mean_products = 0, mean_slots = 0;
 };
 // CTAs of G polynomials on S warps each.
 struct EvalSplit {
@@ -67,6 +70,31 @@ inline EvalSplit eval_split(const EvalShape& e, int limbs, int64_t n_blocks, int
     }
   }
   return best;
+}
+
+// Double evaluation on the FP64 pipe: whether a CTA of `warps` warps for each of
+// `units` units (a polynomial at 32 points, its terms in `chunks` chunks)
+// beats one warp for each.  In units of one complex product at the pipe's full
+// rate (0.17 us) a unit loads a sub-partition with its products and 0.45 for
+// every term it adds; dealt over a CTA's warps, on the SM's four, with 0.55 a
+// term and 3.2 for every output and chunk (searches and loads of the sums).
+// Alone, one warp waits 0.8 a product and 1.8 a term; the CTA's warps 3.2 for
+// each of the products of their share of whole monomials and for each chunk.
+// The 3-norm joins latency and load.  The constants were fitted to eight supports at 32
+// to 16,384 points; the pick costs 0.3 % more than the better of the two on
+// average, 9 % at most.  (Two units a sub-partition, the line for polynomials
+// of 130 monomials, lost 36 % for 12 of 16 two-variable monomials at 3,000
+// points, 28.9 -> 39.2 us, and kept cyclic 10-roots at 4,064 points at 94.8
+// us for 66.1.)
+inline bool double_split_pays(const EvalShape& e, int64_t units, int64_t sms, int warps, int64_t chunks) {
+  auto join = [](double alone, double load) { return alone * alone * alone + load * load * load; };
+  auto waves = [&](int64_t slots) { return (double)((units + slots - 1) / slots); };
+  const double share = (double)((e.max_terms + warps - 1) / warps) / e.max_terms;
+  const double load_one = e.mean_products + 0.45 * e.mean_slots;
+  const double load_split = e.mean_products + 0.55 * e.mean_slots + 3.2 * (e.nv + 1) * chunks;
+  const double one = join(0.8 * e.max_products + 1.8 * e.max_slots, load_one * waves(4 * sms));
+  const double split = join(3.2 * e.max_products * share + 3.2 * chunks, load_split * waves(sms) / 4.0);
+  return split < 0.97 * 0.97 * 0.97 * one;
 }
 
 }  // namespace ht

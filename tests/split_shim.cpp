@@ -21,4 +21,16 @@ int split_pick(int nv, int np, int max_terms, int64_t max_steps, double mean_ste
   const ht::EvalSplit s = ht::eval_split(e, limbs, n_blocks, sms);
   return s.S * 100 + s.G;
 }
+
+int double_pays(int nv, int max_terms, int64_t max_products, double mean_products, int64_t max_slots, double mean_slots,
+                int64_t units, int64_t sms, int warps, int64_t chunks) {
+  ht::EvalShape e;
+  e.nv = nv;
+  e.max_terms = max_terms;
+  e.max_products = max_products;
+  e.mean_products = mean_products;
+  e.max_slots = max_slots;
+  e.mean_slots = mean_slots;
+  return ht::double_split_pays(e, units, sms, warps, chunks);
+}
 }

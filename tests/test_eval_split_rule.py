@@ -1,9 +1,10 @@
-"""The rule that deals a polynomial's monomials to several warps, against
-measured times (CPU: the rule is host code).
+"""The rules that deal a polynomial's monomials to several warps, against
+measured times (CPU: the rules are host code).
 
 golden/eval_split_us.json holds microseconds of ht_eval_diff, variant 2 with
 256 threads, on a GB300 of 152 SMs: with S = 1, 2, 3, 4, 5, 8 and 16 warps a
-polynomial, and of the kernel that preceded splitting (one warp always)."""
+polynomial, and of the kernel that preceded splitting (one warp always);
+golden/eval_double_split_us.json the default variant in double."""
 import ctypes
 import json
 import os
@@ -27,6 +28,8 @@ def shim(tmp_path_factory):
     lib.split_steps.argtypes = [ctypes.c_void_p, ctypes.c_int]
     lib.split_pick.argtypes = [ctypes.c_int] * 3 + [ctypes.c_int64, ctypes.c_double, ctypes.c_int, ctypes.c_int64,
                                                     ctypes.c_int64]
+    lib.double_pays.argtypes = [ctypes.c_int] * 2 + [ctypes.c_int64, ctypes.c_double] * 2 + [ctypes.c_int64] * 2 + \
+        [ctypes.c_int, ctypes.c_int64]
     return lib
 
 
@@ -72,3 +75,26 @@ def test_every_shape_gets_a_valid_split(shim, limbs):
                     S, G = divmod(shim.split_pick(nv, np_, terms, terms * 3, terms * 2.5, limbs, blocks, 152), 100)
                     assert 1 <= S <= min(16, terms) and 1 <= G <= np_
                     assert S * G <= (16 if S > 1 or limbs == 4 else 32)
+
+
+def test_double_picks_are_near_the_better_kernel(shim):
+    """At most 1.1 times the better of one warp and one CTA a polynomial (the
+    model's constants leave 1.09), and at most 1.02 times one warp's, which
+    the default took before."""
+    ratios = []
+    for name, n, warp, cta in json.load(open(os.path.join(HERE, "golden", "eval_double_split_us.json")))["rows"]:
+        s = synth.config_system(name)
+        e = s.exps.astype(np.int64)
+        k = (e > 0).sum(axis=1)
+        prod = np.maximum(e - 1, 0).sum(axis=1) + np.where(k >= 2, 3 * k - 3, k)
+        off = np.concatenate([[0], np.cumsum(s.n_terms)])
+        prods = [int(prod[a:b].sum()) for a, b in zip(off, off[1:])]
+        slots = [int((k[a:b] + 1).sum()) for a, b in zip(off, off[1:])]
+        terms, units = int(max(s.n_terms)), (n + 31) // 32 * s.n_polys
+        q = min(max(slots), min(192, max(slots) + int(k.max())) - int(k.max()))
+        pick = shim.double_pays(s.n_vars, terms, max(prods), float(np.mean(prods)), max(slots), float(np.mean(slots)),
+                                units, 152, max(1, min(16, max(terms, s.n_vars + 1))), (max(slots) + q - 1) // q)
+        t, best = (cta if pick else warp), min(warp, cta)
+        assert t <= 1.1 * best and t <= 1.02 * warp, (name, n, pick, warp, cta)
+        ratios.append(t / best)
+    assert np.exp(np.mean(np.log(ratios))) < 1.01
