@@ -564,7 +564,11 @@ __device__ __forceinline__ cx<L> cx_from(const double* re, const double* im) {
 // MAXT: the largest team (8, or 16 for the wide instantiation that serves
 // few groups of double and double-double paths with more warps each, and
 // any group when the autotuner picks 16; track_int_warps on the integer pipe).
-template <int L, bool LEARN, bool INT, int MAXT = INT ? track_int_warps(L) : 8>
+// COL (double, few paths): the least squares with a column per lane
+// (ht_col_mgs.cuh).  A kernel of its own: its six unrolled bodies spill at 128
+// registers, which cost groups that solve with a system per lane 5 to 20 %
+// (n = 16, 1,500 paths, one-warp teams: 324 -> 376 ms in a shared kernel).
+template <int L, bool LEARN, bool INT, int MAXT = INT ? track_int_warps(L) : 8, bool COL = false>
 __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 4 : (L == 2 ? 2 : 1))) track_kernel(TrackArgs a) {
   __shared__ double red[4][MAXT][32];  // per-warp partials: residual, update, point norms; finiteness
   __shared__ double sh_h[32];       // learned step of each lane's path
@@ -592,8 +596,6 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 4 : (L == 
   // DD and QD with integer evaluation keep A as limb strings from the
   // evaluation through the least squares: no conversions
   constexpr bool FZ = INT && L >= 2;
-  // double, few paths: the least squares with a column per lane (ht_col_mgs.cuh)
-  constexpr bool COL = L == 1 && MAXT > 8;
   // (a block per CTA, which its groups reuse, so that it stays in L2: path l
   // of the group, entry j of a row, NQ 128-bit words: [32][W][NQ][n], row
   // fastest, as the lanes of the solve read it)
@@ -621,8 +623,7 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 4 : (L == 
   // pipe, whatever the lanes in use, so it always takes 32.
   // (with a column per lane in the least squares the lanes count there too)
   int G = 32;
-  const bool col = COL && a.col_lanes;
-  if (FZ || col) G = min(32, (count + (int)gridDim.x - 1) / (int)gridDim.x);
+  if (FZ || COL) G = min(32, (count + (int)gridDim.x - 1) / (int)gridDim.x);
   __shared__ int sh_group;
   for (;;) {
     if (threadIdx.x == 0) sh_group = atomicAdd(a.queue, 1);
@@ -1053,24 +1054,21 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 4 : (L == 
         __syncthreads();
       }
       if constexpr (COL) {
-        if (col) {
-          const unsigned live = __ballot_sync(0xffffffffu, act);
-          const int per = ColLanes::systems(n, nrhs), chunks = (G + per - 1) / per;
-          double2* sh = reinterpret_cast<double2*>(xs_int) + warp * ColLanes::words(n, nrhs);
-          // (the host keeps the chunks to ColLanes::WARPS, the warps with a buffer)
-          for (int c = warp; warp < ColLanes::WARPS && c < chunks; c += min(T, ColLanes::WARPS)) {
-            const int pl = c * per + min(lane / ColLanes::lanes(n, nrhs), per - 1);
-            const int64_t ps = __shfl_sync(0xffffffffu, (int)p, min(pl, 31));
-            ColLanes::solve_any(
-                n, nrhs, pl < 32 && ((live >> pl) & 1u), sh,
-                [&](int i, int j) { return ld<1>(a.A, (int64_t)i * W + j, m, ps); },
-                [&](int k, int i, const cx<1>& z) { st<1>(k == 0 ? a.dx : a.tdx, i, m, ps, z); });
-          }
-          __syncthreads();
+        const unsigned live = __ballot_sync(0xffffffffu, act);
+        const int per = ColLanes::systems(n, nrhs), chunks = (G + per - 1) / per;
+        double2* sh = reinterpret_cast<double2*>(xs_int) + warp * ColLanes::words(n, nrhs);
+        // (the host keeps the chunks to ColLanes::WARPS, the warps with a buffer)
+        for (int c = warp; warp < ColLanes::WARPS && c < chunks; c += min(T, ColLanes::WARPS)) {
+          const int pl = c * per + min(lane / ColLanes::lanes(n, nrhs), per - 1);
+          const int64_t ps = __shfl_sync(0xffffffffu, (int)p, min(pl, 31));
+          ColLanes::solve_any(
+              n, nrhs, pl < 32 && ((live >> pl) & 1u), sh,
+              [&](int i, int j) { return ld<1>(a.A, (int64_t)i * W + j, m, ps); },
+              [&](int k, int i, const cx<1>& z) { st<1>(k == 0 ? a.dx : a.tdx, i, m, ps, z); });
         }
+        __syncthreads();
       }
-      if constexpr (!FZ)
-        if (!col) mgs_team<L>(a.A, a.R, a.dx, n, n, m, p, act, warp, T, nrhs, a.tdx);
+      if constexpr (!FZ && !COL) mgs_team<L>(a.A, a.R, a.dx, n, n, m, p, act, warp, T, nrhs, a.tdx);
       // ---- D: x <- x + dx on this warp's coordinates; partial norms
       double pdx = 0.0, pxp = 0.0;
       if (act) {
@@ -1363,16 +1361,18 @@ int launch_track_l(const TrackArgs& a, int team, int64_t max_groups, cudaStream_
       const size_t dsm = std::max(smem_points_bytes<L>(a.n), (size_t)team * RowLanes<L>::WORDS * sizeof(int32_t));
       learn ? go(track_kernel<L, true, true>, dsm) : go(track_kernel<L, false, true>, dsm);
     }
-  } else if (team > 8 || a.col_lanes || (L <= 2 && max_groups <= sm_count())) {
+  } else if (a.col_lanes) {
+    if constexpr (L == 1) {
+      const size_t dsm = (size_t)ColLanes::WARPS * ColLanes::words(a.n, a.prm.predictor > 0 ? 2 : 1) * sizeof(double2);
+      learn ? go(track_kernel<L, true, false, 16, true>, dsm) : go(track_kernel<L, false, false, 16, true>, dsm);
+    }
+  } else if (team > 8 || (L <= 2 && max_groups <= sm_count())) {
     // wide teams, and groups that have an SM each (no use for the other
     // kernel's 64 registers): double and double double
-    if constexpr (L == 4) {
+    if constexpr (L == 4)
       return set_error(HT_EUNSUPPORTED, "track launch: teams above 8 warps need D or DD");
-    } else {
-      const size_t dsm =
-          a.col_lanes ? (size_t)ColLanes::WARPS * ColLanes::words(a.n, a.prm.predictor > 0 ? 2 : 1) * sizeof(double2) : 0;
-      learn ? go(track_kernel<L, true, false, 16>, dsm) : go(track_kernel<L, false, false, 16>, dsm);
-    }
+    else
+      learn ? go(track_kernel<L, true, false, 16>, 0) : go(track_kernel<L, false, false, 16>, 0);
   } else {
     learn ? go(track_kernel<L, true, false>, 0) : go(track_kernel<L, false, false>, 0);
   }

@@ -1,0 +1,63 @@
+"""The double tracker's least squares in its three layouts -- a column per lane
+(few paths), a system per lane in the wide kernel (up to one group of 32 an SM)
+and in the 8-warp kernel (more) -- and for every team size.  All perform the
+same operations in the same order, so no layout may show in a result.  The
+numbers of paths come from the SM count, so that each run takes the layout that
+it names whatever the chip."""
+import numpy as np
+import pytest
+
+import synth
+from test_gpu_track import ht, track_gpu  # noqa: F401  (ht: the module's fixture)
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _column_paths(n, nrhs):
+    """Paths up to which the tracker solves with a column per lane."""
+    return torch.cuda.get_device_properties(0).multi_processor_count * 4 * (32 // (n + nrhs - 1)) if n <= 16 else 0
+
+
+def _run(ht, s, m, first=0, **over):  # noqa: F811
+    out = track_gpu(ht, s, 1, m, first=first, h_min=1e-4, **over)
+    return [np.asarray(out[k]) for k in ("x_end", "status", "t_end", "steps")]
+
+
+@pytest.mark.parametrize("nrhs", [1, 2])
+@pytest.mark.parametrize("n", list(range(2, 17)))
+def test_columns_per_lane_match_systems_per_lane(ht, n, nrhs):  # noqa: F811
+    """n = 2 to 16 (every unrolled body of the column layout, at and below its
+    size): the first paths of a run too large for the column layout, tracked
+    by a system per lane until few are left, and by themselves in the column
+    layout from the first round.  Six steps a path, so that the large run's
+    paths are all still active when its layout is chosen."""
+    limit = _column_paths(n, nrhs)
+    many, few = limit + 33, min(limit, 37)
+    s = synth.total_degree_system(700 + n, n, 2 if n > 3 else 5, 6 if n == 2 else 8)
+    over = dict(predictor=2 if nrhs == 2 else 0, max_steps=6, iters_per_launch=1, rounds_per_sync=2)
+    whole = _run(ht, s, many, **over)
+    part = _run(ht, s, few, **over)
+    for a, b in zip(whole, part):
+        assert np.array_equal(a[..., :few], b, equal_nan=True)
+    part = _run(ht, s, few, first=many - few, **over)
+    for a, b in zip(whole, part):
+        assert np.array_equal(a[..., -few:], b, equal_nan=True)
+    assert np.min(whole[3]) >= 1
+
+
+@pytest.mark.parametrize("n,predictor", [(6, 0), (6, 2), (16, 0), (16, 2), (19, 0)])
+def test_team_sizes_with_a_system_per_lane(ht, n, predictor):  # noqa: F811
+    """Teams of 1 to 16 warps where a system stays on its lane: in the wide
+    kernel (at most a group an SM), the same bits as the automatic choice, and
+    in the 8-warp kernel (more groups than SMs)."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    limit = _column_paths(n, 2 if predictor else 1)
+    s = synth.total_degree_system(720 + n, n, 2, 8)
+    for m, teams in ((limit + 5, (1, 2, 4, 8, 16)), (32 * sms + 7, (1, 4, 8))):
+        assert m > limit
+        over = dict(predictor=predictor, max_steps=4, iters_per_launch=1, rounds_per_sync=2)
+        base = _run(ht, s, m, **over)
+        for tw in teams:
+            for a, b in zip(base, _run(ht, s, m, team_warps=tw, **over)):
+                assert np.array_equal(a, b, equal_nan=True), (m, tw)
