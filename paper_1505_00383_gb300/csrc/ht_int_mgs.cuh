@@ -2,7 +2,7 @@
 // lane (device only): the corrector's solve of the DD and QD tracker and of
 // ht_mgs_solve_ex variant 2.
 //
-// A warp has min(8, 32 / rows) slots of `rows` lanes.  They hold the slots / C
+// A warp has 32 / rows slots of `rows` lanes.  They hold the slots / C
 // systems the warp serves, each on C slots: slot c of a system has the columns
 // j = c mod C.  A lane holds its row's entry of the pivot column in registers
 // and its row of its columns in local memory; a dot product over the rows is
@@ -33,21 +33,17 @@ template <int L>
 struct RowLanes {
   static constexpr int W = IntW<L>::W, WA = W + 1;
   static constexpr int ND = (2 * WA + 3) / 4 * 4;  // exchanged words a lane, 16-byte multiple
-  static constexpr int SLOTS_MAX = 8;              // slots a warp
-  // Shared memory of one warp: the lanes' digits, then the slots' sums.
-  static constexpr int WORDS = 32 * ND + SLOTS_MAX * 2 * WA * 2;
   using Z = mpi::fz<W>;
 
   int rows, i, slot, base;        // rows a system; this lane's row, its slot, that slot's first lane
   int C, sub, cs;                 // slots a system; this lane's system in the warp, its columns are cs mod C
   bool row;                       // the lane has a row of a live system
   int32_t* dig;                   // shared [32][ND]
-  int64_t* sums;                  // shared [SLOTS_MAX][2 WA]
+  int64_t* sums;                  // shared [slots][2 WA]
 
-  static __host__ __device__ int slots(int rows) {
-    const int n = 32 / rows;
-    return n > SLOTS_MAX ? SLOTS_MAX : n;
-  }
+  static __host__ __device__ int slots(int rows) { return 32 / rows; }
+  // Words of shared memory of one warp: the lanes' digits, then the slots' sums.
+  static __host__ __device__ int words(int rows) { return 32 * ND + slots(rows) * 2 * WA * 2; }
   // row is false for lanes past the last whole system; the caller clears it
   // for systems it does not have
   __device__ __forceinline__ RowLanes(int rows_, int C_, int32_t* xch) : rows(rows_), C(C_) {

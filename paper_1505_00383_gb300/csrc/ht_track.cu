@@ -482,15 +482,17 @@ __global__ void __launch_bounds__(32) mgs_kernel(double* A, double* R, double* x
 
 // Standalone least squares on limb strings of at most 32 rows, one row per
 // lane (ht_int_mgs.cuh): the entries are converted once on loading and once on
-// storing.  R's entries below the diagonal are left as they are.
+// storing.  R's entries below the diagonal are left as they are.  C is 1 (a
+// launch argument all the same: with the constant, the code that the compiler
+// lays out takes 16,384 QD systems of 10 x 10 from 4.06 to 4.17 ms).
 constexpr int kMgsWarps = 4;
 template <int L>
 __global__ void __launch_bounds__(32 * kMgsWarps) mgs_rows_kernel(double* A, double* R, double* x, int rows, int cols,
                                                                int64_t n_sys, int C) {
   using Z = mpi::fz<IntW<L>::W>;
-  __shared__ __align__(16) int32_t xch[kMgsWarps][RowLanes<L>::WORDS];
+  extern __shared__ __align__(16) int32_t xch_mgs[];  // [kMgsWarps][words]
   const int warp = threadIdx.x >> 5, pp = RowLanes<L>::slots(rows) / C, Wc = cols + 1;
-  RowLanes<L> rl(rows, C, xch[warp]);
+  RowLanes<L> rl(rows, C, xch_mgs + warp * RowLanes<L>::words(rows));
   const int64_t n_chunks = (n_sys + pp - 1) / pp;
   for (int64_t c = (int64_t)blockIdx.x * kMgsWarps + warp; c < n_chunks; c += (int64_t)gridDim.x * kMgsWarps) {
     const int64_t p = c * pp + rl.sub;
@@ -623,7 +625,13 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 4 : (L == 
   // pipe, whatever the lanes in use, so it always takes 32.
   // (with a column per lane in the least squares the lanes count there too)
   int G = 32;
-  if (FZ || COL) G = min(32, (count + (int)gridDim.x - 1) / (int)gridDim.x);
+  if (FZ || COL) {
+    // (where a warp solves one system at a time the round is the number of
+    // paths: equal groups, rather than 32 and what is left, in every pass over
+    // the CTAs; n = 17 DD, 6,000 paths in 30 steps: 354 -> 298 ms)
+    const int ctas = (int)gridDim.x, passes = FZ && slots == 1 ? max(1, (count + 32 * ctas - 1) / (32 * ctas)) : 1;
+    G = min(32, (count + ctas * passes - 1) / (ctas * passes));
+  }
   __shared__ int sh_group;
   for (;;) {
     if (threadIdx.x == 0) sh_group = atomicAdd(a.queue, 1);
@@ -1021,10 +1029,11 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 4 : (L == 
         // columns of a system on C slots while that leaves every warp at most
         // one system's worth
         const int C = G <= T ? slots : 1, per = slots / C, chunks = (G + per - 1) / per;
-        RowLanes<L> rl(n, C, xs_int + warp * RowLanes<L>::WORDS);
+        RowLanes<L> rl(n, C, xs_int + warp * RowLanes<L>::words(n));
+        const unsigned mine = per < 32 ? (1u << per) - 1u : ~0u;  // a chunk's paths
         for (int c = warp; c < chunks; c += T) {
           const int pl = c * per + rl.sub;  // the system's path in the group
-          if (((live >> (c * per)) & ((1u << per) - 1u)) == 0) continue;
+          if (((live >> (c * per)) & mine) == 0) continue;
           const int64_t ps = __shfl_sync(0xffffffffu, (int)p, min(pl, 31));
           rl.row = rl.sub < per && pl < 32 && ((live >> pl) & 1u);
           int4* const blk = Acta + (int64_t)min(pl, 31) * W * NQ * n;
@@ -1289,14 +1298,19 @@ int launch_start_l(int n, const int32_t* d_deg, int64_t first, int64_t count, do
 template <int L>
 int launch_mgs_l(double* A, double* R, double* x, int rows, int cols, int64_t n_sys, int variant, cudaStream_t st) {
   if (n_sys == 0) return HT_OK;
-  if (variant == 2 && L > 1 && rows <= 32) {
-    const int64_t chunks = (n_sys + RowLanes<L>::slots(rows) - 1) / RowLanes<L>::slots(rows);
-    const int64_t grid = std::min<int64_t>((chunks + kMgsWarps - 1) / kMgsWarps, (int64_t)sm_count() * 16);
-    mgs_rows_kernel<L><<<(unsigned)grid, 32 * kMgsWarps, 0, st>>>(A, R, x, rows, cols, n_sys, 1);
-  } else if (variant == 2 && L > 1)
-    mgs_kernel<L, L != 1><<<(unsigned)((n_sys + 31) / 32), 32, 0, st>>>(A, R, x, rows, cols, n_sys);
-  else
-    mgs_kernel<L, false><<<(unsigned)((n_sys + 31) / 32), 32, 0, st>>>(A, R, x, rows, cols, n_sys);
+  bool done = false;
+  if constexpr (L > 1) {
+    done = variant == 2;
+    if (done && rows <= 32) {
+      const int64_t chunks = (n_sys + RowLanes<L>::slots(rows) - 1) / RowLanes<L>::slots(rows);
+      const int64_t grid = std::min<int64_t>((chunks + kMgsWarps - 1) / kMgsWarps, (int64_t)sm_count() * 16);
+      const size_t smem = (size_t)kMgsWarps * RowLanes<L>::words(rows) * sizeof(int32_t);  // at most 28 KB
+      mgs_rows_kernel<L><<<(unsigned)grid, 32 * kMgsWarps, smem, st>>>(A, R, x, rows, cols, n_sys, 1);
+    } else if (done) {
+      mgs_kernel<L, true><<<(unsigned)((n_sys + 31) / 32), 32, 0, st>>>(A, R, x, rows, cols, n_sys);
+    }
+  }
+  if (!done) mgs_kernel<L, false><<<(unsigned)((n_sys + 31) / 32), 32, 0, st>>>(A, R, x, rows, cols, n_sys);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? HT_OK : cuda_fail(e, "mgs launch");
 }
@@ -1305,7 +1319,11 @@ int launch_mgs_l(double* A, double* R, double* x, int rows, int cols, int64_t n_
 int64_t track_col_paths(int n, int nrhs) {
   return n > ColLanes::MAX ? 0 : (int64_t)sm_count() * ColLanes::WARPS * ColLanes::systems(n, nrhs);
 }
-int64_t track_int_ctas(int64_t groups) { return std::max<int64_t>(1, std::min<int64_t>(groups, 4 * (int64_t)sm_count())); }
+int64_t track_int_ctas(int64_t groups, int n) {
+  // four an SM (teams of four warps and more), and for n = 1 and 2 as many as their smaller teams fit
+  const int per_sm = std::max(4, 16 / n);
+  return std::max<int64_t>(1, std::min<int64_t>(groups, (int64_t)per_sm * sm_count()));
+}
 size_t track_int_bytes(int L, int n, int nrhs) {
   return (size_t)32 * n * (n + nrhs) * (L == 4 ? sizeof(mpi::fzs<8>) : sizeof(mpi::fzs<5>));
 }
@@ -1351,14 +1369,14 @@ int launch_track_l(const TrackArgs& a, int team, int64_t max_groups, cudaStream_
     if (per_sm < 1) per_sm = 1;
     int64_t grid = (int64_t)sm_count() * per_sm;
     if (grid > max_groups) grid = max_groups;
-    if (in && grid > track_int_ctas(max_groups)) grid = track_int_ctas(max_groups);  // the workspace's CTAs
+    if (in) grid = std::min(grid, track_int_ctas(max_groups, a.n));  // the workspace's CTAs
     if (grid < 1) grid = 1;
     kern<<<(unsigned)grid, 32 * team, dsm, st>>>(a);
   };
   if (in) {
     if constexpr (L > 1) {
       // the converted points, then the solve's exchange buffers in their place
-      const size_t dsm = std::max(smem_points_bytes<L>(a.n), (size_t)team * RowLanes<L>::WORDS * sizeof(int32_t));
+      const size_t dsm = std::max(smem_points_bytes<L>(a.n), (size_t)team * RowLanes<L>::words(a.n) * sizeof(int32_t));
       learn ? go(track_kernel<L, true, true>, dsm) : go(track_kernel<L, false, true>, dsm);
     }
   } else if (a.col_lanes) {

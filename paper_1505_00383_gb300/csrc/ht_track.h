@@ -95,10 +95,18 @@ struct TrackArgs {
 // and systems, so more help until the registers spill: QD with 12 warps of 168
 // registers against 16 of 128: n = 10, 4,096 paths 597 -> 570 ms.
 constexpr int track_int_warps(int L) { return L == 4 ? 12 : 16; }
+// Warps that have work in a group of 32 paths: its polynomials, and its systems
+// at 32 / n a warp.  With more groups than SMs a wider CTA only keeps the next
+// group's warps off the SM (n = 1 and 3, DD, 20,000 paths in 30 steps: 12.8 and
+// 42.5 ms with 16 warps each, 5.4 and 20.3 with 4).
+constexpr int track_int_busy_warps(int L, int n) {
+  const int per = 32 / n, chunks = (32 + per - 1) / per, want = n > chunks ? n : chunks;
+  return want < track_int_warps(L) ? want : track_int_warps(L);
+}
 
 // CTAs of an int_eval launch over at most `groups` groups of paths, and the
 // bytes of the workspace A of each for an L-limb system in n variables.
-int64_t track_int_ctas(int64_t groups);
+int64_t track_int_ctas(int64_t groups, int n);
 size_t track_int_bytes(int L, int n, int nrhs);
 // Active paths up to which the double tracker solves with a column per lane (0: never).
 int64_t track_col_paths(int n, int nrhs);

@@ -310,7 +310,7 @@ int ht_track_paths_ex(ht_system* s, const int32_t* start_deg, const double* gamm
   // (ht_set_eval_config 0 or 1): A is then limb strings in a block per CTA,
   // and R stays with the lanes
   const bool int_eval = L > 1 && s->d_steps && n <= 32 && (s->eval_variant == -1 || s->eval_variant == 2);
-  const size_t b_A = int_eval ? (size_t)track_int_ctas(std::max((m + 31) / 32, std::min<int64_t>(m, sm_count()))) * track_int_bytes(L, n, nrhs)
+  const size_t b_A = int_eval ? (size_t)track_int_ctas(std::max((m + 31) / 32, std::min<int64_t>(m, sm_count())), n) * track_int_bytes(L, n, nrhs)
                               : (size_t)n * (n + nrhs) * cxb,
                b_R = int_eval ? 0 : (size_t)n * (n + nrhs) * cxb;
   size_t o_xp = take(n * cxb), o_hx = take((size_t)cap * n * cxb), o_ht = take((size_t)cap * m * 8),
@@ -426,7 +426,8 @@ int ht_track_paths_ex(ht_system* s, const int32_t* start_deg, const double* gamm
   // per lane in the least squares) a warp per polynomial; while fewer groups
   // are active than there are SMs, a double group with more than 8 columns
   // gets 16 warps (every SM then runs at most one group).  On the integer pipe
-  // always the kernel's most (track_int_warps).
+  // the kernel's most (track_int_warps), or with more groups than SMs the warps
+  // that have work (track_int_busy_warps).
   const bool wide_ok = L <= 2 && n + 1 > 8;
   auto pick_team = [&](int64_t active) {
     // QD accepts teams of up to 8; on the integer pipe the widest is the
@@ -439,7 +440,9 @@ int ht_track_paths_ex(ht_system* s, const int32_t* start_deg, const double* gamm
     } else if (L == 1 && active <= track_col_paths(n, nrhs)) {
       return std::max(4, std::min(16, n));  // a warp per polynomial, four at least for the solve
     } else if (int_eval) {
-      return track_int_warps(L);  // the rows of the systems, and in small groups their columns, spread over all
+      // up to a group an SM: the rows of its systems, and in small groups
+      // their columns, spread over all; else the warps that have work
+      return (active + 31) / 32 <= sm_count() ? track_int_warps(L) : track_int_busy_warps(L, n);
     } else {
       while (t < 8 && 2 * t <= n) t *= 2;
     }

@@ -61,3 +61,21 @@ def test_team_sizes_with_a_system_per_lane(ht, n, predictor):  # noqa: F811
         for tw in teams:
             for a, b in zip(base, _run(ht, s, m, team_warps=tw, **over)):
                 assert np.array_equal(a, b, equal_nan=True), (m, tw)
+
+
+@pytest.mark.parametrize("predictor", [0, 2])
+@pytest.mark.parametrize("L,n", [(2, 1), (2, 2), (2, 3), (2, 5), (2, 17), (4, 1), (4, 2), (4, 3), (4, 9), (4, 17)])
+def test_integer_groups_of_more_paths_than_sms_hold(ht, L, n, predictor):  # noqa: F811
+    """DD and QD with more groups than SMs: teams of the warps that have work,
+    32 to 1 systems a warp in the solve, groups of equal size where a warp
+    takes one; against few paths (the widest teams, columns over slots)."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    s = synth.total_degree_system(740 + n, n, 2 if n > 3 else 5, 6 if n > 1 else 4)
+    over = dict(h_min=1e-4, predictor=predictor, max_steps=4, iters_per_launch=1, rounds_per_sync=2)
+    many, few = 32 * sms + 77, 41
+    keys = ("x_end", "status", "t_end", "steps")
+    whole = track_gpu(ht, s, L, many, **over)
+    for first in (0, many - few):
+        part = track_gpu(ht, s, L, few, first=first, **over)
+        for k in keys:
+            assert np.array_equal(np.asarray(whole[k])[..., first:first + few], np.asarray(part[k]), equal_nan=True), k
