@@ -71,8 +71,8 @@ const char* ht_last_error(void);
  *   limbs    HT_D, HT_DD or HT_QD: the precision evaluations use
  *   out      receives the handle; release it with ht_destroy_system
  * Uses the current CUDA device.  Errors: HT_EINVAL for bad shapes or values,
- * HT_EUNSUPPORTED for a monomial with more than 64 variables, HT_ENOMEM,
- * HT_ECUDA.
+ * HT_EUNSUPPORTED for a monomial with more than 64 variables or 2^31 and more
+ * monomials or variables in them, HT_ENOMEM, HT_ECUDA.
  */
 int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8_t* exps,
                      const double* coef, int limbs, ht_system** out);
@@ -152,7 +152,7 @@ int ht_eval_diff_unfused(ht_system* sys, int64_t n_pts, const double* x, double*
  *            2 integer limbs: the complex products on the integer pipe in
  *              radix-2^29 limbs, sums in an exact fixed-point frame per
  *              output (systems with at most 64 variables; HT_EUNSUPPORTED
- *              otherwise),
+ *              otherwise; a system of 2^31 and more products runs as 1),
  *            3 the three kernels of ht_eval_diff_unfused (coeff, mon, sum
  *              over a workspace): work spread over monomials and points,
  *              which suits few points; the first call allocates the

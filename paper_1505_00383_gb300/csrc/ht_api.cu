@@ -3,6 +3,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <string>
 
@@ -90,31 +91,33 @@ void raise_smem(const void* kernel, size_t bytes) {
 
 using namespace ht;
 
-extern "C" {
+struct SystemDeleter {
+  void operator()(ht_system* s) const {
+    if (s->d_block) cudaFree(s->d_block);
+    if (s->d_coef_fz) cudaFree(s->d_coef_fz);
+    delete s;
+  }
+};
 
-const char* ht_last_error(void) { return g_err.c_str(); }
-
-int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8_t* exps, const double* coef,
-                     int limbs, ht_system** out) {
-  clear_error();
-  if (!out) return set_error(HT_EINVAL, "ht_create_system: out is NULL");
-  *out = nullptr;
+// ht_create_system but for the exceptions of its containers.
+static int create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8_t* exps, const double* coef,
+                         int limbs, ht_system** out) {
   if (n_vars < 1 || n_vars > 255) return set_error(HT_EINVAL, "ht_create_system: n_vars=%d not in 1..255", n_vars);
   if (n_polys < 1) return set_error(HT_EINVAL, "ht_create_system: n_polys=%d < 1", n_polys);
   if (limbs != 1 && limbs != 2 && limbs != 4) return set_error(HT_EINVAL, "ht_create_system: limbs=%d", limbs);
   if (!n_terms || !exps || !coef) return set_error(HT_EINVAL, "ht_create_system: NULL array");
-  ht_system* s = new (std::nothrow) ht_system();
-  if (!s) return set_error(HT_ENOMEM, "ht_create_system: host allocation");
+  std::unique_ptr<ht_system, SystemDeleter> s(new ht_system());
+  const int64_t most = INT32_MAX;  // of monomials, and of their variables: the offsets are 32-bit
+  int64_t terms_of_all = 0;
   s->nv = s->shape.nv = n_vars;
   s->np = s->shape.np = n_polys;
   s->limbs = limbs;
   cudaGetDevice(&s->device);
   s->h_poly_off.assign(n_polys + 1, 0);
   for (int j = 0; j < n_polys; ++j) {
-    if (n_terms[j] < 1) {
-      delete s;
-      return set_error(HT_EINVAL, "ht_create_system: n_terms[%d]=%d < 1", j, n_terms[j]);
-    }
+    if (n_terms[j] < 1) return set_error(HT_EINVAL, "ht_create_system: n_terms[%d]=%d < 1", j, n_terms[j]);
+    terms_of_all += n_terms[j];
+    if (terms_of_all > most) return set_error(HT_EUNSUPPORTED, "ht_create_system: more than %lld monomials", (long long)most);
     s->h_poly_off[j + 1] = s->h_poly_off[j] + n_terms[j];
     s->shape.max_terms = std::max(s->shape.max_terms, (int)n_terms[j]);
   }
@@ -123,14 +126,12 @@ int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8
   s->exps.assign(exps, exps + s->M * n_vars);
   s->coef.assign(coef, coef + s->M * 2 * limbs);
   s->h_mon_off.assign(s->M + 1, 0);
+  int64_t n_steps = 0;
   for (int64_t m = 0; m < s->M; ++m) {
     int k = 0, deg = 0;
     for (int i = 0; i < n_vars; ++i) {
       int a = exps[m * n_vars + i];
-      if (a < 0) {
-        delete s;
-        return set_error(HT_EINVAL, "ht_create_system: negative exponent at monomial %lld", (long long)m);
-      }
+      if (a < 0) return set_error(HT_EINVAL, "ht_create_system: negative exponent at monomial %lld", (long long)m);
       if (a > 0) {
         s->h_pairs.push_back((uint16_t)(i | (a << 8)));
         ++k;
@@ -140,15 +141,14 @@ int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8
     }
     for (int c = 0; c < 2 * limbs; ++c) {
       double v = coef[m * 2 * limbs + c];
-      if (!(v == v) || v - v != 0.0) {
-        delete s;
+      if (!(v == v) || v - v != 0.0)
         return set_error(HT_EINVAL, "ht_create_system: coefficient of monomial %lld is not finite", (long long)m);
-      }
     }
-    if (k > 64) {
-      delete s;
+    if (k > 64)
       return set_error(HT_EUNSUPPORTED, "ht_create_system: monomial %lld has %d variables (max 64)", (long long)m, k);
-    }
+    if ((int64_t)s->h_pairs.size() > most)
+      return set_error(HT_EUNSUPPORTED, "ht_create_system: more than %lld variables in all monomials", (long long)most);
+    n_steps += mpi::sweep_step_count(s->h_pairs.data() + s->h_mon_off[m], k);
     if (k > s->max_k) s->max_k = k;
     if (deg > s->max_deg) s->max_deg = deg;
     s->h_mon_off[m + 1] = (int32_t)s->h_pairs.size();
@@ -163,7 +163,7 @@ int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8
   size_t total = up(b_coef) + up(b_poly) + up(b_mon) + up(b_pairs);
   cudaError_t e = cudaMalloc(&s->d_block, total);
   if (e != cudaSuccess) {
-    delete s;
+    s->d_block = nullptr;
     cudaGetLastError();
     return set_error(HT_ENOMEM, "ht_create_system: cudaMalloc(%zu): %s", total, cudaGetErrorString(e));
   }
@@ -177,11 +177,7 @@ int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8
   if (e == cudaSuccess) e = cudaMemcpy(s->d_mon_off, s->h_mon_off.data(), b_mon, cudaMemcpyHostToDevice);
   if (e == cudaSuccess && s->n_pairs)
     e = cudaMemcpy(s->d_pairs, s->h_pairs.data(), s->n_pairs * sizeof(uint16_t), cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) {
-    cudaFree(s->d_block);
-    delete s;
-    return cuda_fail(e, "ht_create_system: upload");
-  }
+  if (e != cudaSuccess) return cuda_fail(e, "ht_create_system: upload");
   // integer-format coefficients for the integer evaluation variant
   {
     const size_t zsz = limbs == 1 ? sizeof(mpi::fz<3>) : (limbs == 2 ? sizeof(mpi::fz<5>) : sizeof(mpi::fz<8>));
@@ -203,13 +199,15 @@ int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8
       const double mod = std::hypot(re[0], im[0]);
       hl[m] = mod == 0.0 ? -1000.0f : (float)std::log2(mod);
     }
-    // the sweep steps of every monomial (the integer variant takes at most 64 variables)
+    // the sweep steps of every monomial (the integer variant takes at most 64
+    // variables; a system of more steps than the offsets reach runs on the
+    // FP64 bodies instead)
     std::vector<uint32_t> steps;
     std::vector<int32_t> step_off;
-    if (n_vars <= 64) {
+    if (n_vars <= 64 && mpi::offsets_fit(n_steps)) {
       step_off.reserve(s->M + 1);
       step_off.assign(1, 0);
-      steps.reserve(4 * s->n_pairs + s->M);
+      steps.reserve(n_steps);
       for (int64_t m = 0; m < s->M; ++m) {
         mpi::sweep_steps(s->h_pairs.data() + s->h_mon_off[m], s->h_mon_off[m + 1] - s->h_mon_off[m], steps);
         step_off.push_back((int32_t)steps.size());
@@ -238,7 +236,8 @@ int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8
     }
     s->shape.mean_slots = (double)(s->n_pairs + s->M) / n_polys;
     s->shape.mean_products = (double)products / n_polys;
-    if (limbs == 1 && s->shape.max_slots < (1 << 24) && s->n_pairs + s->M < (1LL << 31)) {
+    if (limbs == 1 && s->shape.max_slots < (1 << 24) && mpi::offsets_fit(s->n_pairs + s->M) &&
+        mpi::offsets_fit((int64_t)n_polys * (n_vars + 1))) {
       std::vector<std::vector<uint32_t>> of(n_vars + 1);
       terms.reserve(s->n_pairs + s->M);
       term_off.reserve((size_t)n_polys * (n_vars + 1) + 1);
@@ -288,14 +287,27 @@ int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8
     }
     if (e != cudaSuccess) {
       cudaGetLastError();
-      if (s->d_coef_fz) cudaFree(s->d_coef_fz);
-      cudaFree(s->d_block);
-      delete s;
       return set_error(HT_ENOMEM, "ht_create_system: integer coefficients");
     }
   }
-  *out = s;
+  *out = s.release();
   return HT_OK;
+}
+
+extern "C" {
+
+const char* ht_last_error(void) { return g_err.c_str(); }
+
+int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8_t* exps, const double* coef,
+                     int limbs, ht_system** out) {
+  clear_error();
+  if (!out) return set_error(HT_EINVAL, "ht_create_system: out is NULL");
+  *out = nullptr;
+  try {
+    return create_system(n_vars, n_polys, n_terms, exps, coef, limbs, out);
+  } catch (const std::exception&) {  // a container that could not grow
+    return set_error(HT_ENOMEM, "ht_create_system: host allocation");
+  }
 }
 
 int ht_destroy_system(ht_system* s) {

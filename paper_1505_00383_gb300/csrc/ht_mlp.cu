@@ -8,7 +8,8 @@
 // masters.  The network's role in tracking is described in ht_track.cu.
 #include <cmath>
 #include <cstring>
-#include <vector>
+#include <memory>
+#include <new>
 
 #include "ht_internal.h"
 #include "ht_mlp.cuh"
@@ -487,13 +488,14 @@ int ht_mlp_train(ht_mlp* net, int64_t n, const float* x, const float* target, in
   float *part, *lpart, *lbuf;
   int rc = mlp_ws(net, batch < n ? batch : n, kLosses, &part, &lpart, &lbuf, st);
   if (rc != HT_OK) return rc;
-  std::vector<float> hl(kLosses);
+  std::unique_ptr<float[]> hl(new (std::nothrow) float[kLosses]);
+  if (!hl) return set_error(HT_ENOMEM, "ht_mlp_train: host allocation");
   int64_t kept = 0;  // losses on the device
   double sum = 0.0;
   int64_t summed = 0;  // batches of the running epoch in sum
   int done = 0;        // epochs reported
   auto flush = [&]() {
-    cudaError_t e = cudaMemcpyAsync(hl.data(), lbuf, kept * sizeof(float), cudaMemcpyDeviceToHost, st);
+    cudaError_t e = cudaMemcpyAsync(hl.get(), lbuf, kept * sizeof(float), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "ht_mlp_train");
     for (int64_t k = 0; k < kept; ++k) {

@@ -3,6 +3,7 @@
 // tests run it as is).  The reverse-mode sweep is the one of ht_eval.cuh.
 #pragma once
 #include <cmath>
+#include <cstdint>
 #include <vector>
 
 #include "ht_mpi.cuh"
@@ -111,6 +112,15 @@ inline uint32_t make(uint32_t kind, int var, int p, bool store, bool add, int sl
          (uint32_t)e << 25;
 }
 }  // namespace step
+
+// Number of steps of a monomial with the k variables pr (variable | exponent << 8).
+inline int64_t sweep_step_count(const uint16_t* pr, int k) {
+  int64_t n = 1 + 2 * k + (k > 2 ? k - 2 : 0);
+  for (int r = 0; r < k; ++r) n += (pr[r] >> 8) - 1;
+  return n;
+}
+// The lists' offsets are 32-bit.
+inline bool offsets_fit(int64_t entries) { return entries <= INT32_MAX; }
 
 // Append the steps of a monomial with the k <= 64 variables pr (variable | exponent << 8).
 template <class Out>

@@ -1,4 +1,4 @@
-// Host build of the integer evaluation's split rule (csrc/ht_split.h).
+// Host build of the evaluation's split rules (csrc/ht_split.h) and step lists.
 #include "../paper_1505_00383_gb300/csrc/ht_mpi_eval.cuh"
 #include "../paper_1505_00383_gb300/csrc/ht_split.h"
 
@@ -9,6 +9,10 @@ int64_t split_steps(const uint16_t* pairs, int k) {
   ht::mpi::sweep_steps(pairs, k, st);
   return (int64_t)st.size();
 }
+
+int64_t split_step_count(const uint16_t* pairs, int k) { return ht::mpi::sweep_step_count(pairs, k); }
+
+int split_offsets_fit(int64_t n) { return ht::mpi::offsets_fit(n); }
 
 int split_pick(int nv, int np, int max_terms, int64_t max_steps, double mean_steps, int limbs, int64_t n_blocks,
                int64_t sms) {

@@ -28,6 +28,9 @@ def shim(tmp_path_factory):
     lib.split_steps.argtypes = [ctypes.c_void_p, ctypes.c_int]
     lib.split_pick.argtypes = [ctypes.c_int] * 3 + [ctypes.c_int64, ctypes.c_double, ctypes.c_int, ctypes.c_int64,
                                                     ctypes.c_int64]
+    lib.split_step_count.restype = ctypes.c_int64
+    lib.split_step_count.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    lib.split_offsets_fit.argtypes = [ctypes.c_int64]
     lib.double_pays.argtypes = [ctypes.c_int] * 2 + [ctypes.c_int64, ctypes.c_double] * 2 + [ctypes.c_int64] * 2 + \
         [ctypes.c_int, ctypes.c_int64]
     return lib
@@ -98,3 +101,20 @@ def test_double_picks_are_near_the_better_kernel(shim):
         assert t <= 1.1 * best and t <= 1.02 * warp, (name, n, pick, warp, cta)
         ratios.append(t / best)
     assert np.exp(np.mean(np.log(ratios))) < 1.01
+
+
+def test_step_lists_are_counted_before_they_are_built(shim):
+    """The count that decides whether a system's step list fits 32-bit offsets
+    is the list's length; 64 variables of exponent 127 reach 2^31 steps at
+    260,144 monomials, whose 16.6 million variables fit by themselves."""
+    rng = np.random.default_rng(3)
+    for k in (0, 1, 2, 3, 17, 64):
+        for top in (1, 2, 127):
+            v = np.sort(rng.permutation(64)[:k]).astype(np.int64)
+            pr = np.ascontiguousarray(v | (rng.integers(1, top + 1, k) << 8), dtype=np.uint16)
+            assert shim.split_step_count(pr.ctypes.data, k) == shim.split_steps(pr.ctypes.data, k)
+    pr = np.ascontiguousarray(np.arange(64) | (127 << 8), dtype=np.uint16)
+    per = shim.split_step_count(pr.ctypes.data, 64)
+    assert per == 1 + 64 * 126 + 128 + 62
+    assert shim.split_offsets_fit(260143 * per) and not shim.split_offsets_fit(260144 * per)
+    assert shim.split_offsets_fit(2 ** 31 - 1) and not shim.split_offsets_fit(2 ** 31)
