@@ -70,10 +70,10 @@ const char* ht_last_error(void);
  *   coef     host [M][2][limbs]: complex coefficients (re limbs, im limbs)
  *   limbs    HT_D, HT_DD or HT_QD: the precision evaluations use
  *   out      receives the handle; release it with ht_destroy_system
- * Builds the step and term lists of the evaluation kernels, about 9 bytes a
- * variable of a monomial on the device and 0.1 to 0.4 ms for the systems of
- * the benchmarks.  Uses the current CUDA device.  Errors: HT_EINVAL for bad shapes or values,
- * HT_EUNSUPPORTED for a monomial with more than 64 variables or 2^31 and more
+ * Builds the step and term lists of the evaluation kernels, about 16 bytes a
+ * variable of a monomial on the device (0.1 to 0.4 ms for the systems of the
+ * benchmarks).  Uses the current CUDA device.  Errors: HT_EINVAL for bad
+ * shapes or values, HT_EUNSUPPORTED for a monomial with more than 64 variables or 2^31 and more
  * monomials or variables in them, HT_ENOMEM, HT_ECUDA.
  */
 int ht_create_system(int n_vars, int n_polys, const int32_t* n_terms, const int8_t* exps,

@@ -599,11 +599,11 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 4 : (L == 
   // evaluation through the least squares: no conversions
   constexpr bool FZ = INT && L >= 2;
   // (a block per CTA, which its groups reuse, so that it stays in L2: path l
-  // of the group, entry j of a row, NQ 128-bit words: [32][W][NQ][n], row
+  // of the group, entry j of a row, NQ 128-bit words: [group_max][W][NQ][n], row
   // fastest, as the lanes of the solve read it)
   constexpr int NQ = mpi::fzs<IntW<L>::W>::NW / 4;
   const int slots = RowLanes<L>::slots(n);  // of a warp in the solve
-  int4* const Acta = reinterpret_cast<int4*>(a.A) + (int64_t)blockIdx.x * 32 * W * NQ * n;
+  int4* const Acta = reinterpret_cast<int4*>(a.A) + (int64_t)blockIdx.x * a.group_max * W * NQ * n;
   PolyView v;
   v.mon_off = a.mon_off;
   v.pairs = a.pairs;
@@ -1324,8 +1324,8 @@ int64_t track_int_ctas(int64_t groups, int n) {
   const int per_sm = std::max(4, 16 / n);
   return std::max<int64_t>(1, std::min<int64_t>(groups, (int64_t)per_sm * sm_count()));
 }
-size_t track_int_bytes(int L, int n, int nrhs) {
-  return (size_t)32 * n * (n + nrhs) * (L == 4 ? sizeof(mpi::fzs<8>) : sizeof(mpi::fzs<5>));
+size_t track_int_bytes(int L, int n, int nrhs, int paths) {
+  return (size_t)paths * n * (n + nrhs) * (L == 4 ? sizeof(mpi::fzs<8>) : sizeof(mpi::fzs<5>));
 }
 __global__ void __launch_bounds__(256) mlp_image_kernel(MlpSmem* img, const __nv_bfloat16* __restrict__ wbf,
                                                         const float* __restrict__ master) {

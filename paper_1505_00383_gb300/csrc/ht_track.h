@@ -37,6 +37,7 @@ struct TrackArgs {
   const int32_t* step_off;  // the integer evaluation's sweep steps
   const uint32_t* sweep;
   int int_eval;        // DD/QD: evaluate f on the integer pipe
+  int group_max;       // int_eval: paths that a CTA's block of A holds
   const int32_t* deg;  // start system degrees [n]
   double gamma_re, gamma_im;
   int n;
@@ -105,9 +106,10 @@ constexpr int track_int_busy_warps(int L, int n) {
 }
 
 // CTAs of an int_eval launch over at most `groups` groups of paths, and the
-// bytes of the workspace A of each for an L-limb system in n variables.
+// bytes of the workspace A of each for an L-limb system in n variables and
+// groups of `paths`.
 int64_t track_int_ctas(int64_t groups, int n);
-size_t track_int_bytes(int L, int n, int nrhs);
+size_t track_int_bytes(int L, int n, int nrhs, int paths);
 // Active paths up to which the double tracker solves with a column per lane (0: never).
 int64_t track_col_paths(int n, int nrhs);
 

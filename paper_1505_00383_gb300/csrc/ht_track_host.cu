@@ -308,9 +308,12 @@ int ht_track_paths_ex(ht_system* s, const int32_t* start_deg, const double* gamm
   // DD and QD (n <= 32) evaluate f and solve the Newton systems on the
   // integer pipe unless an FP64 variant was chosen for this system
   // (ht_set_eval_config 0 or 1): A is then limb strings in a block per CTA,
-  // and R stays with the lanes
+  // and R's rows take the places of A's.  A launch over `active` paths has at
+  // least min(active, SMs) CTAs, so no group exceeds group_max.
   const bool int_eval = L > 1 && s->d_steps && n <= 32 && (s->eval_variant == -1 || s->eval_variant == 2);
-  const size_t b_A = int_eval ? (size_t)track_int_ctas(std::max((m + 31) / 32, std::min<int64_t>(m, sm_count())), n) * track_int_bytes(L, n, nrhs)
+  const int64_t spread = std::min<int64_t>(m, sm_count());
+  const int group_max = (int)std::min<int64_t>(32, (m + spread - 1) / spread);
+  const size_t b_A = int_eval ? (size_t)track_int_ctas(std::max((m + 31) / 32, spread), n) * track_int_bytes(L, n, nrhs, group_max)
                               : (size_t)n * (n + nrhs) * cxb,
                b_R = int_eval ? 0 : (size_t)n * (n + nrhs) * cxb;
   size_t o_xp = take(n * cxb), o_hx = take((size_t)cap * n * cxb), o_ht = take((size_t)cap * m * 8),
@@ -335,6 +338,7 @@ int ht_track_paths_ex(ht_system* s, const int32_t* start_deg, const double* gamm
   a.step_off = s->d_step_off;
   a.sweep = s->d_steps;
   a.int_eval = int_eval;
+  a.group_max = group_max;
   a.deg = (const int32_t*)(w + o_deg);
   a.gamma_re = gamma[0];
   a.gamma_im = gamma[1];

@@ -79,3 +79,24 @@ def test_integer_groups_of_more_paths_than_sms_hold(ht, L, n, predictor):  # noq
         part = track_gpu(ht, s, L, few, first=first, **over)
         for k in keys:
             assert np.array_equal(np.asarray(whole[k])[..., first:first + few], np.asarray(part[k]), equal_nan=True), k
+
+
+def test_integer_workspace_follows_the_number_of_paths(ht):  # noqa: F811
+    """QD, n = 24, one path an SM: the matrices of those paths (48 KB each) and
+    not of 32 paths a CTA (1.5 MB each, 233 MB on 152 SMs); 48 KB and its state of
+    about 5 KB a path stay below 128 KB a path."""
+    m = torch.cuda.get_device_properties(0).multi_processor_count
+    s = synth.total_degree_system(760, 24, 2, 6)
+    hs = ht.system_from(s, 4)
+    x = torch.zeros((24, 2, 4, m), dtype=torch.float64, device="cuda")
+    st = torch.zeros((m,), dtype=torch.int8, device="cuda")
+    t = torch.zeros((m,), dtype=torch.float64, device="cuda")
+    prm = ht.ht_default_params(4, max_steps=1)
+    # the kernels' local memory is allocated on their first launch
+    warm = ht.system_from(s, 4)
+    ht.ht_track_paths(warm, s.degrees(), (0.6, 0.8), m, 0, None, prm, x, st, t)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    ht.ht_track_paths(hs, s.degrees(), (0.6, 0.8), m, 0, None, prm, x, st, t)
+    torch.cuda.synchronize()
+    assert before - torch.cuda.mem_get_info()[0] <= m * (128 << 10) + (4 << 20)
