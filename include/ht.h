@@ -483,8 +483,9 @@ int ht_track_refined(ht_system* lo, ht_system* hi, const int32_t* start_deg, con
 /*
  * ht_tune_track -- autotuner for ht_track_paths on this system: tracks the
  * first n_paths paths (from the start solutions) once per candidate launch
- * shape -- team_warps in {1, 2, 4, 8} (up to n; also 16 for D and DD with n >= 8) and iters_per_launch in
- * {2, 4, 8}, p's other settings unchanged (p may be NULL: defaults) -- keeps
+ * shape -- team_warps in {1, 2, 4, 8} (up to n; also 16 for D and DD with n >=
+ * 8, and 0, the automatic choice, for DD and QD on the integer pipe) and
+ * iters_per_launch in {2, 4, 8}, p's other settings unchanged (p may be NULL: defaults) -- keeps
  * the fastest (wall time of the call) in the system, where it replaces the
  * built-in choice whenever a call's params leave team_warps or
  * iters_per_launch at 0, and reports it (output pointers may be NULL).  The

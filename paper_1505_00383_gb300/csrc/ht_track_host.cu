@@ -438,11 +438,12 @@ int ht_track_paths_ex(ht_system* s, const int32_t* start_deg, const double* gamm
     // kernel's 12 warps
     const int widest = int_eval && L == 4 ? track_int_warps(L) : 8;
     if (P.team_warps > 0) return P.team_warps == 8 ? widest : P.team_warps;
+    // (before a tuned size, which was chosen for the bulk of the paths)
+    if (L == 1 && active <= track_col_paths(n, nrhs))
+      return std::max(4, std::min(16, n));  // a warp per polynomial, four at least for the solve
     int t = 1;
     if (s->track_team > 0 && s->track_team <= 16) {
       t = s->track_team == 8 ? widest : s->track_team;
-    } else if (L == 1 && active <= track_col_paths(n, nrhs)) {
-      return std::max(4, std::min(16, n));  // a warp per polynomial, four at least for the solve
     } else if (int_eval) {
       // up to a group an SM: the rows of its systems, and in small groups
       // their columns, spread over all; else the warps that have work
@@ -582,8 +583,13 @@ int ht_tune_track(ht_system* s, const int32_t* start_deg, const double* gamma, i
   const int saved_team = s->track_team, saved_iters = s->track_iters;
   double best = 1e300;
   int bt_team = 0, bt_iters = 0, rc = HT_OK;
-  const int teams[5] = {1, 2, 4, 8, 16}, its[3] = {2, 4, 8};
-  for (int a = 0; a < 5 && rc == HT_OK; ++a) {
+  // On the integer pipe also 0, the automatic choice: it changes with the
+  // number of active paths, and no fixed team up to n warps reaches the 12 or
+  // 16 that it gives small systems (n = 5, DD, 40 paths: 11.5 ms, 14.8 with 4).
+  const bool int_eval = L > 1 && s->d_steps && n <= 32 && (s->eval_variant == -1 || s->eval_variant == 2);
+  const int teams[6] = {0, 1, 2, 4, 8, 16}, its[3] = {2, 4, 8};
+  s->track_team = s->track_iters = 0;
+  for (int a = int_eval ? 0 : 1; a < 6 && rc == HT_OK; ++a) {
     if (teams[a] > 1 && teams[a] > n) continue;
     if (teams[a] > 8 && (L == 4 || n + 1 <= 8)) continue;  // wide teams: D and DD with more than 8 columns
     for (int b = 0; b < 3 && rc == HT_OK; ++b) {

@@ -4,19 +4,32 @@
 rounds per launch) on a sample of paths and keeps the fastest in the system
 object.  This module remembers that choice across processes, keyed by what
 it depends on: the number of variables, the number of terms, the largest
-degree, the precision, whether the learned step runs, whether DD/QD
+degree, the precision, the library's sources (a shape tuned on other kernels
+says nothing about these), whether the learned step runs, whether DD/QD
 evaluation runs on the integer pipe, and the GPU (the kernels of the learned
 and integer modes use other shared memory and registers, so their best shape
-differs).  The cache is a plain JSON object {key: {"team_warps": t,
+differs).  A team of 0 warps is the automatic choice.  The cache is a plain JSON object {key: {"team_warps": t,
 "iters_per_launch": k, "ms": ms}} at a path the caller chooses.
 """
 from __future__ import annotations
 
+import functools
+import hashlib
 import json
 import os
 import tempfile
 
-from . import ht
+from . import _build, ht
+
+
+@functools.lru_cache(maxsize=None)
+def kernels_id() -> str:
+    """Short hash of the library's sources."""
+    h = hashlib.sha256()
+    for f in sorted(os.listdir(_build.CSRC)):
+        with open(os.path.join(_build.CSRC, f), "rb") as src:
+            h.update(f.encode() + b"\0" + src.read())
+    return h.hexdigest()[:12]
 
 
 def cache_key(system, limbs: int, device_name: str, learned: bool = False, int_eval: bool | None = None) -> str:
@@ -25,8 +38,9 @@ def cache_key(system, limbs: int, device_name: str, learned: bool = False, int_e
     if int_eval is None:
         int_eval = limbs > 1 and system.n_vars <= 32
     deg = int(system.exps.astype(int).sum(axis=1).max())
-    return "n=%d;terms=%d;deg=%d;limbs=%d;learned=%d;int=%d;gpu=%s" % (
-        system.n_vars, int(sum(system.n_terms)), deg, limbs, int(bool(learned)), int(bool(int_eval)), device_name)
+    return "n=%d;terms=%d;deg=%d;limbs=%d;kernels=%s;learned=%d;int=%d;gpu=%s" % (
+        system.n_vars, int(sum(system.n_terms)), deg, limbs, kernels_id(), int(bool(learned)), int(bool(int_eval)),
+        device_name)
 
 
 def _load(path):
