@@ -357,7 +357,7 @@ HT_HD rz<W> quotient(const rz<W>& a, const rz<W>& b, double b_lead) {
   for (int it = 0; it < 3; ++it) y = mul<W>(y, sub<W>(two, mul<W>(b, y)));
   return mul<W>(a, y);
 }
-// Weights of cubic Hermite interpolation at u in [0, 1] of an interval of
+// Weights of cubic Hermite interpolation at u (past 1 when it extrapolates) of an interval of
 // length d: of the values and slopes at 0 and at 1, w[0..3] = 2 u^3 - 3 u^2 +
 // 1, (u^3 - 2 u^2 + u) d, 3 u^2 - 2 u^3, (u^3 - u^2) d.
 template <int W>
