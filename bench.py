@@ -5,7 +5,8 @@ double -- one step is one pass over the batch in all three precisions.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
-Prints one JSON line.  ``value`` is whole-job eval-diff points per second, a
+Prints one JSON line (everything measured goes to stderr, and to a file with
+--details).  ``value`` is whole-job eval-diff points per second, a
 point counting once when it has been evaluated (values and full Jacobian) in
 all three precisions.  For N > 1 (torchrun) every rank evaluates its own batch
 (weak scaling, no collective on the data path).  ``--impl reference`` times
@@ -107,7 +108,47 @@ def _args():
                    help="skip the mixed-precision (double tracking, double double refinement) comparison")
     p.add_argument("--no-paper-sweep", action="store_true",
                    help="skip the evaluation sweep of the stand-ins shaped like the paper's applications")
+    p.add_argument("--details", default="", help="file that receives everything measured, as JSON")
     return p.parse_args()
+
+
+LINE_MAX = 2800
+
+
+def _rounded(v):
+    """Floats to six significant digits, all the way down."""
+    if isinstance(v, float):
+        return float("%.6g" % v)
+    if isinstance(v, dict):
+        return {k: _rounded(x) for k, x in v.items()}
+    if isinstance(v, (list, tuple)):
+        return [_rounded(x) for x in v]
+    return v
+
+
+def result_line(full):
+    """The printed line: the result, its configuration, the end-to-end figure with
+    its fastest and slowest pass, the roofline, and one figure for each tracking
+    workload.  Optional parts are dropped from the back if it were too long."""
+    d = dict(full)
+    for k in ("tuned", "unfused_ablation", "paper_shapes", "peaks"):
+        d.pop(k, None)
+    d["per_precision"] = {k: {q: v[q] for q in ("ms", "pts_per_s", "variant", "imad_frac", "fp64_frac") if q in v}
+                          for k, v in full["per_precision"].items()}
+    if full.get("e2e") and "ms_per_precision" in full["e2e"]:
+        d["e2e"] = {k: v for k, v in full["e2e"].items() if k != "ms_per_precision"}
+        d["e2e"]["ms_min_max"] = {k: [min(v), max(v)] for k, v in full["e2e"]["ms_per_precision"].items()}
+    if full.get("cpu_baseline"):
+        d["cpu_baseline"] = {k: v for k, v in full["cpu_baseline"].items() if k != "single_thread"}
+    keep = ("paths_per_s", "plain_paths_per_s", "learned_paths_per_s", "mixed_paths_per_s", "speedup")
+    d["tracking"] = {k: {q: v[q] for q in keep if q in v} for k, v in (full.get("tracking") or {}).items()}
+    d = _rounded(d)
+    for k in (None, "tracking", "wall_s_timed_region", "cpu_baseline", "per_precision"):
+        d.pop(k, None)
+        line = json.dumps(d)
+        if len(line) <= LINE_MAX:
+            break
+    return line
 
 
 class Clocks:
@@ -792,7 +833,7 @@ def run_ours(a):
                                  "sample": "%d D + %d DD + %d QD points, one thread (the paper's one-core "
                                            "comparison)" % (budget1[1], budget1[2], budget1[4])}}
     if rank == 0:
-        print(json.dumps({
+        full = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": a.steps,
             "warmup": a.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "f64 (D, DD, QD limbs)", "data": "synthetic",
@@ -800,10 +841,17 @@ def run_ours(a):
                        "monomial_vars": "2-8", "exponents": "1-3", "n_pts_per_gpu": n,
                        "l2": "flushed (512 MB write) before every timed step; outputs 1.1-4.5 GB per launch",
                        "parallelism": "independent batch per GPU"},
-            "per_precision": per_prec, "tuned": tuned, "unfused_ablation": ablation, "paper_shapes": paper_sweep, "tracking": tracking, "roofline": roofline, "peaks": peaks, "cpu_baseline": cpu, "e2e": e2e,
-            "gpu_launches": a.steps * len(PRECISIONS), "clocks": clk.summary(),
-            "wall_s_timed_region": t_wall,
-        }))
+            "per_precision": per_prec, "tuned": tuned, "unfused_ablation": ablation, "paper_shapes": paper_sweep,
+            "tracking": tracking, "roofline": roofline, "peaks": peaks, "cpu_baseline": cpu, "e2e": e2e,
+            "gpu_launches": a.steps * len(PRECISIONS), "clocks": clk.summary(), "wall_s_timed_region": t_wall}
+        # everything measured goes to stderr (and to a file on request); the
+        # line on stdout holds the result in under LINE_MAX characters, so that
+        # a log which keeps only the end of the output keeps all of it
+        print(json.dumps(full), file=sys.stderr, flush=True)
+        if a.details:
+            with open(a.details, "w") as f:
+                json.dump(full, f, indent=1)
+        print(result_line(full), flush=True)
     if world > 1:
         dist.destroy_process_group()
 
