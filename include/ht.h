@@ -365,7 +365,7 @@ int ht_compact(const int8_t* status, int64_t m, int32_t* path_idx, int32_t* coun
  *   t_end      device [n_paths]: t of the last accepted point
  *   steps      device [n_paths] (int32) steps per path, or NULL
  *   stats      host, or NULL
- * Launch shape: p->team_warps warps per group of 32 paths and
+ * Launch shape: p->team_warps warps per group of paths and
  * p->iters_per_launch Newton rounds per launch, or, where they are 0, the
  * system's tuned shape (ht_tune_track) or the built-in one.  Results do not
  * depend on the shape.

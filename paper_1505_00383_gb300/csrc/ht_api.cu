@@ -363,9 +363,11 @@ int ht_eval_diff_host(ht_system* s, int64_t n_pts, const double* x_host, double*
   // transfer.  Events order the two streams: a slab's copy waits for its
   // evaluation, and the evaluation that reuses a slab waits for that slab's
   // previous copy, so the evaluations never wait for a copy still in flight
-  // unless three are.  Blocks hold at least 8 polynomials (the
-  // block-organised integer kernel deals polynomials to 8 warps); the
-  // three-kernel variant takes one block.
+  // unless three are.  Blocks hold at least 8 polynomials: fewer leave the
+  // block-organised kernel small CTAs, more leave the copies of the last block
+  // uncovered (n = 32, 65,536 points, blocks of 4, 8, 16 and 32: DD 39.1, 34.1,
+  // 37.2 and 41.4 ms, QD 86.6, 68.1, 72.6 and 82.0; at 1,000 points 16 is 10 %
+  // faster than 8).  The three-kernel variant takes one block.
   const size_t L = s->limbs;
   const int64_t rx = (int64_t)s->nv * 2 * L, rv = 2 * L, rj = (int64_t)s->nv * 2 * L;  // doubles per point per row
   int nb = s->np;

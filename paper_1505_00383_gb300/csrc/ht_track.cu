@@ -616,9 +616,9 @@ __global__ void __launch_bounds__(32 * MAXT, MAXT > 8 ? 1 : (L == 1 ? 4 : (L == 
     g.im = r_from<L>(a.gamma_im);
     return g;
   }();
-  // Groups of 32 active paths are taken from a queue (one counter per
-  // launch, zeroed by the compaction before it): a CTA whose groups finish
-  // early takes more, instead of a fixed share of them.
+  // Groups of G active paths are taken from a queue (one counter per launch,
+  // zeroed by the compaction before it): a CTA whose groups finish early takes
+  // more, instead of a fixed share of them.
   // DD and QD on the integer pipe spread few paths thinly: a group is as many
   // paths as give every CTA one, since its rounds shorten with the work the
   // SM shares.  In double a group's cost is its instruction count on the FP64

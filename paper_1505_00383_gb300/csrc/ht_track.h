@@ -71,7 +71,7 @@ struct TrackArgs {
   int polish_only;         // start every path at t = 1 in the polish phase
   const int32_t* idx_in;   // active path indices of this launch
   const int32_t* count_in; // their number (device)
-  int32_t* queue;          // next 32-path group to take (device; zero at launch)
+  int32_t* queue;          // next group to take (device; zero at launch)
   int32_t* idx0;           // init: identity index list
   int32_t* count0;
   // last step summary (features of the learned step) and learned-step state
