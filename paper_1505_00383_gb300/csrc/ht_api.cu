@@ -63,7 +63,7 @@ int sm_count() {
 }
 
 void raise_smem(const void* kernel, size_t bytes) {
-  // limits set so far; kernels or devices past the table's end ask the driver
+  // limits set so far; kernels or devices past the table's end ask the runtime
   constexpr int KERNELS = 32, DEVICES = 64;
   static std::mutex lock;
   static const void* known[KERNELS];
